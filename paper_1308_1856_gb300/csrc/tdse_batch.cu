@@ -33,6 +33,7 @@
 #include "tdse_pulse.h"
 #include "tdse_internal.cuh"
 #include "tdse_stencil.cuh"
+#include "tdse_walk_fixed.cuh"
 
 namespace tdse_dev {
 namespace {
@@ -53,6 +54,9 @@ using namespace stencil;
 // are compile-time constants (the launch schedule never changes them).
 constexpr int kChunkSegs = TDSE_CHUNK_SEGS;  // 32-point row segments per chunk (stencil kernels)
 constexpr int kChunkPts = TDSE_CHUNK_PTS;    // consecutive points per chunk (elementwise kernels)
+constexpr int kFxThreads = 128;              // threads of a block of the fixed-point stencil kernel
+constexpr int kFxBlocksPerSM = 4;            // 128 registers a thread
+constexpr int kFxMaxRows = 32;               // segments of a chunk at most (16: 5% slower on large batches)
 constexpr int kCombinePts = 2;               // points per lane whose Krylov loads the combines overlap
 constexpr int kMixedCombinePts = 2;          // the same for the mixed combine, two vectors per round
 
@@ -77,12 +81,12 @@ __device__ __forceinline__ int find_owner(const ChunkList &cl, int gc) {
 // Add v (every lane) to the chunk's slot and, if this was the instance's last
 // chunk, reduce the instance's chunk partials in order; returns true in every
 // lane of the warp that must finish the instance (with the sum in `total`).
-__device__ __forceinline__ bool chunk_done(const BatchDev &B, const BatchInst &I, int inst, int ci,
-                                           int nchunk, double v, double &total) {
+__device__ __forceinline__ bool chunk_done(const BatchDev &B, double *part, int inst, int ci, int nchunk, double v,
+                                           double &total) {
   v = warp_sum(v);
   unsigned last = 0;
   if ((threadIdx.x & 31) == 0) {
-    I.partial[ci] = v;
+    part[ci] = v;
     __threadfence();
     last = (atomicAdd(&B.ticket[inst], 1u) == (unsigned)(nchunk - 1)) ? 1u : 0u;
   }
@@ -90,7 +94,7 @@ __device__ __forceinline__ bool chunk_done(const BatchDev &B, const BatchInst &I
   if (!last) return false;
   __threadfence();
   double s = 0.0;
-  for (int c = threadIdx.x & 31; c < nchunk; c += 32) s += __ldcg(&I.partial[c]);
+  for (int c = threadIdx.x & 31; c < nchunk; c += 32) s += __ldcg(&part[c]);
   total = warp_sum(s);
   if ((threadIdx.x & 31) == 0) B.ticket[inst] = 0u;
   return true;
@@ -126,6 +130,23 @@ __device__ __forceinline__ void chunk_groups(const BatchInst &I, int ci, F &&f) 
     const int l0 = s - jg * Lp1;
     const int l1 = min(Lp1, l0 + (s_end - s));
     f(jg, l0, l1);
+    s += l1 - l0;
+  }
+}
+
+// Visit chunk ci of an instance in the fixed-point stencil layout: strips of
+// kFxCols columns, I.fx_rows row segments of a strip-major order per chunk.
+// f(j0, l0, l1) is called by every lane of the warp.
+template <typename F>
+__device__ __forceinline__ void chunk_strips(const BatchInst &I, int ci, F &&f) {
+  const int Lp1 = I.L + 1;
+  int s = ci * I.fx_rows;
+  const int s_end = min(s + I.fx_rows, I.fx_seg);
+  while (s < s_end) {
+    const int sg = s / Lp1;
+    const int l0 = s - sg * Lp1;
+    const int l1 = min(Lp1, l0 + (s_end - s));
+    f(sg * kFxCols, l0, l1);
     s += l1 - l0;
   }
 }
@@ -237,10 +258,126 @@ __device__ __forceinline__ StencilIn fp64_in(const BatchDev &B, const BatchInst 
   return in;
 }
 
-// VG: the chunk list holds velocity-gauge instances only (a separate launch).
-template <int ST, int PF, bool VG = false>
+// The recurrence's scale.  z = s_j H U_j - (s_j / sigma_j) ratio_j U_{j-1} with
+// s_j the power of two at or below sigma_j (the scale is then an exponent, not
+// a product per point); with g_j = sigma_j / s_j in [1, 2):
+//   alpha_j = sigma_j g_j Re<U_j, z>,  U_{j+1} = z - alpha_j s_j U_j,
+//   beta_j = g_j ||U_{j+1}||.
+// sigma_j = 0 (a vanished vector) keeps s_j = 1, g_j = 0.
+struct StepScale {
+  double s, g;
+  int k;       // s = 2^k
+};
+__device__ __forceinline__ StepScale step_scale(double sigma) {
+  StepScale r;
+  const int f = (__double2hiint(sigma) >> 20) & 0x7ff;
+  const bool usable = f > 0 && f < 0x7ff;
+  r.k = usable ? f - 1023 : 0;
+  r.s = usable ? __hiloint2double(f << 20, 0) : 1.0;
+  r.g = usable ? __hiloint2double((__double2hiint(sigma) & 0xfffff) | 0x3ff00000, __double2loint(sigma)) : sigma;
+  return r;
+}
+
+// alpha_j and U_{j+1}'s coefficient from the sum of U_j^* z.
+__device__ __forceinline__ void store_alpha(LanczosScalars *ls, int j, double sum) {
+  const double sig = ls->sigma[j];
+  const StepScale sc = step_scale(sig);
+  const double al = (sum * sig) * sc.g;
+  ls->alpha[j] = al;
+  ls->acoef[j] = -al * sc.s;
+}
+// beta_j and the next vector's scalars from ||U_{j+1}||^2.
+__device__ __forceinline__ void store_beta(LanczosScalars *ls, int j, double sumsq) {
+  const double nrm = sqrt(sumsq);
+  const double beta = step_scale(ls->sigma[j]).g * nrm;
+  ls->beta[j] = beta;
+  const double sn = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+  ls->sigma[j + 1] = sn;
+  ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
+}
+
+__device__ __forceinline__ FxIn fixed_in(const BatchDev &B, const BatchInst &I, int inst, const double2 *x, int k) {
+  FxIn in;
+  in.x = x;
+  in.diagq = reinterpret_cast<const long long *>(I.diag);
+  in.rj = I.rj;
+  in.kappa = I.kappa;
+  in.N = I.N;
+  in.L = I.L;
+  in.c1 = I.c1;
+  in.c2 = I.c2;
+  in.E = field_of(B, inst);
+  in.c1q = I.c1q;
+  in.c2q = I.c2q;
+  in.ec = I.fx_ec;
+  in.ok = I.fx_ok;
+  in.k = k;
+  return in;
+}
+
+// Visit the list's chunks one by one, warp w taking chunks w, w + W, ... of the
+// W warps: chunks of different instances cost differently (fx_rows), and a
+// contiguous range each left some SMs three times the work of others.
+template <typename F>
+__device__ __forceinline__ void for_strided_chunks(const ChunkList &cl, F &&f) {
+  const int W = warp_count();
+  int gc = warp_id();
+  if (gc >= cl.total) return;
+  int p = find_owner(cl, gc);
+  for (; gc < cl.total; gc += W) {
+    while (cl.cpre[p + 1] <= gc) ++p;
+    f(cl.act[p], gc - cl.cpre[p]);
+  }
+}
+
+// Phase A of the length-gauge instances: the fixed-point walker
+// (tdse_walk_fixed.cuh) with the recurrence and the dot product in FP64: six
+// FP64 instructions a point (two of them integer conversions) in place of 20.
+// What bounds it: the integer and FP64 pipes' issue together (integer 76%, FP64
+// 58% busy, 16 warps an SM at 128 registers; more warps spill and are slower).
+// All phase A launches of one step of 128 instances (8.1e7 points): 36.9 ms in
+// FP64, 19.5 ms here; of 8 instances (1.3e6 points), 24 ms to 6 ms over 8 steps,
+// where the smaller chunks count as well.
+template <int ST, int EX>
+__global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM) bt_lanczos_a_fixed(BatchDev B, ChunkList cl, int j) {
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX>();
+  for_strided_chunks(cl, [&](int inst, int ci) {
+    const BatchInst &I = B.inst[inst];
+    LanczosScalars *ls = B.ls + inst;
+    const long long G = (long long)I.N * (I.L + 1);
+    const double2 *u = (j == 0) ? I.psi : I.work + (long long)j * G;
+    FxExtra<EX> up;
+    up.p[0] = (j <= 1) ? I.psi : I.work + (long long)(j - 1) * G;
+    double2 *z = I.work;
+    const StepScale s0 = step_scale(ls->sigma[j]);
+    // ratio_j s_j / sigma_j; g_j = 0 only for a vanished vector, whose ratio is 0
+    const double cprev = (EX > 0 && s0.g > 0.0) ? ls->ratio[j] / s0.g : 0.0;
+    const FxIn in = fixed_in(B, I, inst, u, s0.k);
+    double acc = 0.0;
+    chunk_strips(I, ci, [&](int j0, int l0, int l1) {
+      walk_rows_fixed<ST, EX>(in, up, ring, j0, l0, l1,
+                              [&](int idx, double2 t, double2 uc, const double2 (&e)[1]) {
+        double2 o = t;
+        if (EX > 0) {
+          o.x = __fma_rn(-cprev, e[0].x, t.x);
+          o.y = __fma_rn(-cprev, e[0].y, t.y);
+        }
+        z[idx] = o;
+        acc = __fma_rn(uc.x, o.x, acc);
+        acc = __fma_rn(uc.y, o.y, acc);
+      });
+    });
+    double s;
+    if (chunk_done(B, I.dpart, inst, ci, I.nchunk, acc, s) && (threadIdx.x & 31) == 0) store_alpha(ls, j, s);
+  });
+}
+
+// Phase A of the velocity-gauge instances (a launch of its own over their
+// row-segment chunks), all in FP64.
+template <int ST, int PF>
 __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
-    bt_lanczos_a_fp64(BatchDev B, ChunkList cl, int j) {
+    bt_lanczos_a_fp64_vg(BatchDev B, ChunkList cl, int j) {
   for_my_chunks(cl, [&](int inst, int ci) {
     const BatchInst I = B.inst[inst];
     LanczosScalars *ls = B.ls + inst;
@@ -249,12 +386,13 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
     const double2 *up = (j <= 1) ? I.psi : I.work + (long long)(j - 1) * G;
     double2 *z = I.work;
     const double sig = ls->sigma[j];
-    const double cprev = (j > 0) ? ls->ratio[j] : 0.0;
-    // t = sigma_j H U_j directly (the operator scaled by sigma_j)
-    const StencilIn in = scaled(fp64_in(B, I, inst, u), sig);
+    const StepScale sc = step_scale(sig);
+    const double cprev = (j > 0 && sc.g > 0.0) ? ls->ratio[j] / sc.g : 0.0;
+    // t = s_j H U_j directly (the operator scaled by s_j)
+    const StencilIn in = scaled(fp64_in(B, I, inst, u), sc.s);
     double acc = 0.0;
     chunk_columns(I, ci, [&](int i, int l0, int l1) {
-      walk_rows<ST, PF, true, VG>(in, i, l0, l1, [&](int, size_t idx, double2 t, double2 uc) {
+      walk_rows<ST, PF, true, true>(in, i, l0, l1, [&](int, size_t idx, double2 t, double2 uc) {
         double2 o;
         if (j > 0) {
           const double2 pv = up[idx];
@@ -269,14 +407,11 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
       });
     });
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk, acc, s) && (threadIdx.x & 31) == 0) {
-      ls->alpha[j] = s * sig;
-      ls->acoef[j] = -(s * sig) * sig;
-    }
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk, acc, s) && (threadIdx.x & 31) == 0) store_alpha(ls, j, s);
   });
 }
 
-// U_{j+1} = z - alpha_j sigma_j U_j and beta_j = ||U_{j+1}||, chunk by chunk.
+// U_{j+1} = z - alpha_j s_j U_j and beta_j = g_j ||U_{j+1}||, chunk by chunk.
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     bt_lanczos_b_fp64(BatchDev B, ChunkList cl, int j) {
   for_my_chunks(cl, [&](int inst, int ci) {
@@ -297,12 +432,8 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
       acc = __fma_rn(o.y, o.y, acc);
     });
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
-      const double beta = sqrt(s);
-      ls->beta[j] = beta;
-      const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
-      ls->sigma[j + 1] = sn;
-      ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
+      store_beta(ls, j, s);
     }
   });
 }
@@ -319,7 +450,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
       acc = __fma_rn(v.y, v.y, acc);
     });
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
       LanczosScalars *ls = B.ls + inst;
       const double nrm = sqrt(s);
       ls->psinorm = nrm;
@@ -391,7 +522,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
       }
     });
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
       const double nrm = sqrt(s);
       ls->psinorm0 = ls->psinorm;
       ls->psinorm = nrm;
@@ -469,7 +600,7 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
     }
     const double accd = acc.value();
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk, accd, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk, accd, s) && (threadIdx.x & 31) == 0) {
       ls->alpha[j] = s * sigd;
       ls->acoef[j] = -(s * sigd) * sigd;
     }
@@ -509,7 +640,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     });
     const double accd = acc.value();
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
       const double beta = sqrt(s);
       ls->beta[j] = beta;
       const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
@@ -536,7 +667,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     });
     const double accd = acc.value();
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
       LanczosScalars *ls = B.ls + inst;
       const double nrm = sqrt(s);
       ls->psinorm = nrm;
@@ -686,7 +817,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     });
     const double accd = acc.value();
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
       const double nrm = sqrt(s);
       ls->psinorm0 = ls->psinorm;
       ls->psinorm = nrm;
@@ -715,6 +846,30 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
   }
 }
 
+// The diagonal of a new instance, c0 + l(l+1)/(2 r^2) - Z/r in the roundings of
+// plain FP64 (no fused step): as doubles (velocity gauge, or coefficients
+// outside the fixed-point range), encoded for the fixed-point walker, or in
+// FP32 without c0 (mixed).  On the device because a served instance is built
+// while others run: two divisions a point on one host core took longer than
+// an instance's Lanczos step.
+__global__ void __launch_bounds__(256) bt_diag_table(BatchInst I, double c0) {
+  const size_t G = (size_t)I.N * (I.L + 1);
+  for (size_t q = (size_t)blockIdx.x * 256 + threadIdx.x; q < G; q += (size_t)gridDim.x * 256) {
+    const int l = (int)((unsigned)q / (unsigned)I.N);
+    const double r = I.rj[q - (size_t)l * I.N];
+    const double cent = 0.5 * (double)l * (double)(l + 1);
+    const double d = __dsub_rn(__dadd_rn(c0, __ddiv_rn(cent, __dmul_rn(r, r))), __ddiv_rn(I.Z, r));
+    if (I.diagf) {
+      const_cast<float *>(I.diagf)[q] = __double2float_rn(__dsub_rn(d, c0));
+    } else if (I.fx_ok) {
+      reinterpret_cast<long long *>(const_cast<double *>(I.diag))[q] =
+          fx_encode_diag((uint64_t)__double_as_longlong(d), I.fx_ec);
+    } else {
+      const_cast<double *>(I.diag)[q] = d;
+    }
+  }
+}
+
 // ---- Sec. 3: imaginary time ------------------------------------------------
 // After the combine of an imaginary-time step (exp(-T dtau) in the small
 // exponential, no field): psi <- psi / sqrt(dr ||psi||^2), so that the norm
@@ -737,7 +892,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
       acc = __fma_rn(o.y, o.y, acc);
     });
     double s;
-    if (chunk_done(B, I, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
+    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
       const double nrm = sqrt(s);
       energy[inst] = -log(n1 / ls->psinorm0) / dtau[inst];
       ls->psinorm = nrm;
@@ -937,11 +1092,22 @@ constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
 struct Layout {
-  size_t psi, diag, diagf, hi, lo, work, mwork, rj, mask, kappa, rjf, kappaf, partial, dpart, ref0, rinv, rinvf,
-      total;
+  size_t psi, diag, diagf, hi, lo, work, mwork, rj, mask, kappa, rjf, kappaf, partial, dpart, ref0, rinv,
+      rinvf, total;
 };
 
 // Tiles of the mixed tile kernel on an N x (L+1) grid.
+// Row segments and segments per chunk of the fixed-point stencil kernel: at
+// least ~512 chunks an instance, so that a handful of instances fills the SMs'
+// warps, between 32 segments (a chunk loads two halo rows beside its own) and
+// what the chunk partials' room allows: they use the dipole kernel's 4 slots
+// per 64 segments of 32 columns, idle during phase A, so about 9 segments.
+size_t fx_segments(size_t N, size_t Lp1) { return (N + kFxCols - 1) / kFxCols * Lp1; }
+int fx_chunk_rows(size_t N, size_t Lp1) {
+  const size_t nseg = fx_segments(N, Lp1), room = 4 * (((N + 31) / 32 * Lp1 + kChunkSegs - 1) / kChunkSegs);
+  return (int)std::max((nseg + room - 1) / room, std::min<size_t>(kFxMaxRows, nseg / 512));
+}
+
 int tile_count(int N, int L) { return ((N + kTileCols - 1) / kTileCols) * ((L + kTileRows) / kTileRows); }
 
 Layout layout_of(const tdse_instance_spec &s, int precision) {
@@ -1129,11 +1295,14 @@ int Engine::place(int slot, const tdse_instance_spec &s, void *mem) {
   I.L = L;
   I.m = s.krylov;
   I.nseg = (int)((size_t)((N + 31) / 32) * (L + 1));
-  // reduction chunks of the stencil kernel: 64 row segments (FP64 and the
-  // mixed velocity gauge), or tiles of 256 columns x kTileRows rows (the
-  // mixed tile kernel)
+  // reduction chunks of the stencil kernel: row segments (64 of 32 columns in
+  // the velocity gauge, fx_rows of kFxCols in FP64 length gauge), or tiles of
+  // 256 columns x kTileRows rows (the mixed tile kernel)
   const bool vg = s.gauge == TDSE_GAUGE_VELOCITY;
-  I.nchunk = (mixed && !vg) ? tile_count(N, L) : (I.nseg + kChunkSegs - 1) / kChunkSegs;
+  I.fx_seg = (int)fx_segments(N, L + 1);
+  I.fx_rows = fx_chunk_rows(N, L + 1);
+  I.nchunk = vg ? (I.nseg + kChunkSegs - 1) / kChunkSegs
+                : (mixed ? tile_count(N, L) : (I.fx_seg + I.fx_rows - 1) / I.fx_rows);
   I.nchunk_e = (int)((G + kChunkPts - 1) / kChunkPts);
   I.nchunk_d = (I.nseg + kChunkSegs - 1) / kChunkSegs;
   I.dr = s.dr;
@@ -1214,40 +1383,37 @@ int Engine::place(int slot, const tdse_instance_spec &s, void *mem) {
     for (int j = 0; j < N; ++j) ri[j] = 1.0 / rj[j];
     EN_CUDA(cudaMemcpyAsync((void *)I.rinv, ri.data(), sizeof(double) * N, cudaMemcpyHostToDevice, st), "1/r table");
   }
+  std::vector<float> rf, kf, rif;
   if (mixed) {
-    std::vector<float> df(G), rf(N), kf(L + 2);
-    for (int l = 0; l <= L; ++l) {
-      const double cent = 0.5 * (double)l * (double)(l + 1);
-      for (int j = 0; j < N; ++j) {
-        const double r = rj[j];
-        df[(size_t)l * N + j] = (float)((c0 + cent / (r * r) - s.Z / r) - c0);
-      }
-    }
+    rf.resize(N);
+    kf.resize(L + 2);
     for (int j = 0; j < N; ++j) rf[j] = (float)rj[j];
     if (I.rinvf) {
-      std::vector<float> rif(N);
+      rif.resize(N);
       for (int j = 0; j < N; ++j) rif[j] = (float)(1.0 / rj[j]);
       EN_CUDA(cudaMemcpyAsync((void *)I.rinvf, rif.data(), sizeof(float) * N, cudaMemcpyHostToDevice, st),
               "1/r table");
-      EN_CUDA(cudaStreamSynchronize(st), "sync 1/r table");
     }
     for (int l = 0; l < L + 2; ++l) kf[l] = (float)kap[l];
-    EN_CUDA(cudaMemcpyAsync((void *)I.diagf, df.data(), sizeof(float) * G, cudaMemcpyHostToDevice, st), "diag");
     EN_CUDA(cudaMemcpyAsync((void *)I.rjf, rf.data(), sizeof(float) * N, cudaMemcpyHostToDevice, st), "r table");
     EN_CUDA(cudaMemcpyAsync((void *)I.kappaf, kf.data(), sizeof(float) * (L + 2), cudaMemcpyHostToDevice, st), "kappa");
-    EN_CUDA(cudaStreamSynchronize(st), "sync tables");
-  } else {
-    std::vector<double> diag(G);
-    for (int l = 0; l <= L; ++l) {
-      const double cent = 0.5 * (double)l * (double)(l + 1);
-      for (int j = 0; j < N; ++j) {
-        const double r = rj[j];
-        diag[(size_t)l * N + j] = c0 + cent / (r * r) - s.Z / r;
-      }
-    }
-    EN_CUDA(cudaMemcpyAsync((void *)I.diag, diag.data(), sizeof(double) * G, cudaMemcpyHostToDevice, st), "diag");
-    EN_CUDA(cudaStreamSynchronize(st), "sync tables");
   }
+  if (!mixed && !vg) {
+    // largest |diagonal|: the centrifugal and Coulomb terms at the first point
+    const double dmax = c0 + 0.5 * (double)L * (double)(L + 1) / (rj[0] * rj[0]) + std::fabs(s.Z) / rj[0];
+    I.fx_ok = tdse_fx::fx_scale(c0, I.fx_ec) && tdse_fx::fx_diag_fits(dmax, I.fx_ec) ? 1 : 0;
+    auto coef = [&](double v) {
+      uint64_t u;
+      std::memcpy(&u, &v, 8);
+      return tdse_fx::fx_coef(u, I.fx_ec);
+    };
+    if (I.fx_ok) {
+      I.c1q = coef(I.c1);
+      I.c2q = coef(I.c2);
+    }
+  }
+  bt_diag_table<<<(unsigned)(sms * 4), 256, 0, st>>>(I, c0);
+  EN_CUDA(cudaGetLastError(), "diagonal table");
   const int m = s.krylov;
   const double dt = s.dt;
   EN_CUDA(cudaMemcpyAsync(inst + slot, &I, sizeof(BatchInst), cudaMemcpyHostToDevice, st), "descriptor");
@@ -1467,9 +1633,14 @@ namespace {
 constexpr long kGraphMinSteps = 3;   // segments this long replay one captured step graph
 constexpr size_t kGraphCache = 8;    // captured step graphs kept across runs
 
-template <int ST, int PF>
-void launch_a_pf(unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
-  bt_lanczos_a_fp64<ST, PF><<<grid, kBlockJ, 0, st>>>(B, cl, j);
+template <int ST, int EX>
+cudaError_t launch_fixed(unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
+  constexpr int bytes = (kFxThreads / 32) * fx_warp_bytes<EX>();
+  static const cudaError_t ready = cudaFuncSetAttribute(bt_lanczos_a_fixed<ST, EX>,
+                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (ready != cudaSuccess) return ready;
+  bt_lanczos_a_fixed<ST, EX><<<grid, kFxThreads, bytes, st>>>(B, cl, j);
+  return cudaGetLastError();
 }
 
 // The mixed tile kernel: dynamic shared memory of its ring of D row slots,
@@ -1506,22 +1677,12 @@ cudaError_t launch_tile_ring(int ring, unsigned grid, cudaStream_t st, const Bat
 }
 
 template <int ST>
-void launch_a_st(int pf, unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
-  switch (pf) {
-    case 0: launch_a_pf<ST, 0>(grid, st, B, cl, j); break;
-    case 3: launch_a_pf<ST, 3>(grid, st, B, cl, j); break;
-    case 10: launch_a_pf<ST, 10>(grid, st, B, cl, j); break;
-    default: launch_a_pf<ST, 6>(grid, st, B, cl, j); break;
-  }
-}
-
-template <int ST>
 void launch_a_vg_st(int pf, unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
   switch (pf) {
-    case 0: bt_lanczos_a_fp64<ST, 0, true><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-    case 3: bt_lanczos_a_fp64<ST, 3, true><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-    case 10: bt_lanczos_a_fp64<ST, 10, true><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-    default: bt_lanczos_a_fp64<ST, 6, true><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
+    case 0: bt_lanczos_a_fp64_vg<ST, 0><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
+    case 3: bt_lanczos_a_fp64_vg<ST, 3><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
+    case 10: bt_lanczos_a_fp64_vg<ST, 10><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
+    default: bt_lanczos_a_fp64_vg<ST, 6><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
   }
 }
 
@@ -1677,17 +1838,23 @@ int Engine::norm_pass(const BatchDev &B, const std::vector<int> &ids, int off, i
 }
 
 int Engine::launch_a(const BatchDev &B, const ChunkList &cl, int j, const Schedule &s) {
-  const unsigned grid = (unsigned)(sms * s.sblocks);
   if (precision == TDSE_MIXED) {
+    const unsigned grid = (unsigned)(sms * s.sblocks);
     const cudaError_t e = (stencil == 5) ? launch_tile_ring<5>(s.ring, grid, stream, B, cl, j)
                                          : launch_tile_ring<3>(s.ring, grid, stream, B, cl, j);
     EN_CUDA(e, "batch lanczos a (mixed tiles)");
     return TDSE_OK;
   }
-  if (stencil == 5) launch_a_st<5>(s.pf, grid, stream, B, cl, j);
-  else launch_a_st<3>(s.pf, grid, stream, B, cl, j);
-  EN_CUDA(cudaGetLastError(), "batch lanczos a");
+  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM : kFxBlocksPerSM / 2));
+  const cudaError_t e = stencil == 5 ? (j ? launch_fixed<5, 1>(grid, stream, B, cl, j) : launch_fixed<5, 0>(grid, stream, B, cl, j))
+                                     : (j ? launch_fixed<3, 1>(grid, stream, B, cl, j) : launch_fixed<3, 0>(grid, stream, B, cl, j));
+  EN_CUDA(e, "batch lanczos a");
   return TDSE_OK;
+}
+
+// Chunks the phase-A launch takes at once: one per warp (FP64) or block (mixed tiles).
+int Engine::stencil_wave() const {
+  return precision == TDSE_MIXED ? sms * sched.sblocks * (kBlockJ / 32) : sms * kFxBlocksPerSM * (kFxThreads / 32);
 }
 
 // Velocity-gauge instances: the same FP64 kernel with the (A/c) p_z coupling,
@@ -2188,20 +2355,26 @@ int Engine::autotune(const std::vector<int> &slots) {
   float bestA = 1e30f, bestB = 1e30f;
   // the staged rows are the mixed tile kernel's
   const int nring = precision == TDSE_MIXED ? (int)(sizeof(kRingChoices) / sizeof(int)) : 1;
-  // three blocks per SM only for the mixed tile kernel (the FP64 stencil kernel's blocks fill an SM at two)
+  // three blocks per SM only for the mixed tile kernel (the FP64 kernels' blocks fill an SM at two)
   const int sbmax = precision == TDSE_MIXED ? kTileBlocksPerSM : kStencilBlocksPerSM;
-  for (int sb = 1; sb <= sbmax && !rc && sg.total[0] > 0; ++sb)
+  // the prefetch distance is the FP64 velocity-gauge kernel's: the others stage their rows in shared memory
+  const bool tune_pf = precision == TDSE_FP64 && sg.vtotal[0] > 0;
+  const ChunkList v0 = list_at(lists, sg.voff[0], sg.vnact[0], sg.vtotal[0]);
+  for (int sb = 1; sb <= sbmax && !rc && (sg.total[0] > 0 || tune_pf); ++sb)
     for (int ri = 0; ri < nring && !rc; ++ri)
       for (int pf : kPfChoices) {
         const int ring = kRingChoices[ri];
-        // the mixed tile kernel stages its rows itself: the prefetch distance is the FP64 kernel's
-        if (precision == TDSE_MIXED && pf != kPfChoices[0]) continue;
+        if (!tune_pf && pf != kPfChoices[0]) continue;
         Schedule c = sched;
         c.pf = pf;
         c.ring = ring;
         c.sblocks = sb;
         float t = 0.f;
-        rc = time_it([&]() { return launch_a(B, a0, 0, c); }, t);
+        rc = time_it([&]() {
+          int r = sg.total[0] > 0 ? launch_a(B, a0, 0, c) : (int)TDSE_OK;
+          if (!r && tune_pf) r = launch_a_velocity(B, v0, 0, c);
+          return r;
+        }, t);
         if (rc) break;
         if (t < bestA) {
           bestA = t;
@@ -2212,7 +2385,6 @@ int Engine::autotune(const std::vector<int> &slots) {
       }
   if (!rc && sg.vtotal[0] > 0) {
     // the velocity-gauge instances' phase-0 z, which lanczos_b below reads
-    const ChunkList v0 = list_at(lists, sg.voff[0], sg.vnact[0], sg.vtotal[0]);
     rc = launch_a_velocity(B, v0, 0, sched);
   }
   if (!rc && have_b) {
@@ -2460,7 +2632,7 @@ int tdse_batch_propagate_io(tdse_batch_t *b, const double *F_in, double *F_out, 
     coff[i + 1] = coff[i] + (size_t)e.hinst[i].nchunk;
   }
   const double ratio = (b->io_ratio > 0.0) ? b->io_ratio * (double)std::max(nsteps, 1L) : kIoRatioFirst;
-  const size_t wave = (size_t)e.sms * (size_t)e.sched.sblocks * (kBlockJ / 32);
+  const size_t wave = (size_t)e.stencil_wave();
   const std::vector<int> first = tdse_sched::io_groups(coff, groups, ratio, wave);
   auto bytes = [&](int i) { return sizeof(double) * (off[i + 1] - off[i]); };
   // every input copy first, in group order on the input stream, after the

@@ -29,6 +29,9 @@ struct BatchInst {
                          // length-gauge instances)
   int nchunk_e;          // reduction chunks of the elementwise kernels (consecutive points)
   int nchunk_d;          // reduction chunks of the dipole kernel (kChunkSegs row segments, both precisions)
+  int fx_seg, fx_rows;   // fixed-point stencil: row segments of kFxCols columns, segments per chunk
+  int fx_ok, fx_ec;      // whether the coefficients fit the fixed-point form; their exponent
+  long long c1q, c2q;    // c1, c2 against 2^fx_ec
   int gauge;             // TDSE_GAUGE_LENGTH or TDSE_GAUGE_VELOCITY (FP64 only)
   double c1, c2;         // stencil coefficients (c0 is folded into diag)
   double d1c;            // first-derivative scale of the velocity gauge (1/(12 dr) or 1/(2 dr))
@@ -36,7 +39,7 @@ struct BatchInst {
   const double *rinv;    // 1/r_j (FP64 velocity gauge; null otherwise)
   const float *rinvf;    // 1/r_j (mixed velocity gauge; null otherwise)
   double2 *psi;          // (L+1) x N state, l-major
-  const double *diag;    // FP64: c0 + l(l+1)/(2 r^2) - Z/r
+  const double *diag;    // FP64: c0 + l(l+1)/(2 r^2) - Z/r; encoded (fx_encode_diag) in the length gauge if fx_ok
   const float *diagf;    // mixed: l(l+1)/(2 r^2) - Z/r (difference-form stencil)
   const double *rj, *kappa, *mask;
   const float *rjf, *kappaf;
@@ -44,7 +47,7 @@ struct BatchInst {
   double2 *work;         // FP64 Krylov area: slot 0 = z, slots 1..m-1 = U_j
   float2 *mwork;         // mixed Krylov area, same slots
   double *partial;       // max(nchunk, nchunk_e) chunk partial sums
-  double *dpart;         // 4 * nchunk_d chunk partials of the dipole kernel
+  double *dpart;         // 4 * nchunk_d chunk partials of the dipole and the fixed-point stencil kernel
   double2 *ref0;         // N values: the p_ground reference (1s state of the grid)
 };
 
@@ -188,6 +191,9 @@ class Engine {
   std::string err;
   bool poisoned = false;
   cudaStream_t own_stream = nullptr, stream = nullptr;
+
+  // Stencil chunks one phase-A launch works on at a time.
+  int stencil_wave() const;
 
  private:
   int ensure(void **p, size_t &cap, size_t bytes, const char *what);

@@ -1,0 +1,327 @@
+// The FP64 operator's row walker in fixed point (tdse_fixed.cuh): H x of the
+// length gauge with the operand and the result in FP64.
+//
+// A warp owns a strip of kFxCols radial columns and walks it up the partial
+// waves.  Lane k holds columns j0 - 2 + 2k and the one after it, so lanes 0
+// and 31 carry the stencil's halo and lanes 1..30 produce results: 60 of 64
+// columns useful, every operand value loaded and converted once per strip, the
+// radial neighbours exchanged by shuffles.  Two columns a lane halve the
+// shuffles and the row's uniform work against one, and take 94% of the lanes'
+// work against 88% for the same halo.
+//
+// Exponents are local: a lane converts its two columns against their largest
+// exponent field, and forms the stencil's sums against the largest of its own and
+// its two neighbour lanes' (six columns).  One exponent for the whole strip costs
+// ~10% less, but loses what FP64 keeps next to the origin: there a high partial
+// wave is many orders below its value at the strip's other end, and rounding
+// errors relative to that value, put into the stiff centrifugal points, are
+// multiplied by the largest energies of the grid in every Krylov iteration
+// (measured: 3e-12 after one step where FP64 gives 6e-16).
+//
+// Blocks near the limits of FP64 (subnormal values, results that under- or
+// overflow) take separate conversions.  A row with an Inf or NaN in reach is
+// computed by h_point_fp64, one point at a time in FP64, so such values spread
+// exactly as they do there.  These choices are uniform over the warp.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <type_traits>
+
+#include "tdse_fixed.cuh"
+#include "tdse_stencil.cuh"
+
+namespace tdse_dev {
+namespace stencil {
+
+using namespace tdse_fx;
+
+constexpr int kFxCols = 60;    // output columns of a strip
+
+struct FxIn {
+  const double2 *__restrict__ x;
+  const long long *__restrict__ diagq;   // encoded diagonal (ok), or the FP64 diagonal's bits (!ok)
+  const double *__restrict__ rj;
+  const double *__restrict__ kappa;
+  int N, L;
+  double c1, c2, E;
+  long long c1q, c2q;                    // c1, c2 against 2^ec
+  int ec;
+  int ok;                                // 0: the grid's coefficients do not fit, every row runs in FP64
+  int k;                                 // the result is 2^k H x
+};
+
+__device__ __forceinline__ double fx_double(uint64_t b) { return __longlong_as_double((long long)b); }
+
+__device__ __forceinline__ double fx_diag_double(const FxIn &in, long long q) {
+  if (!in.ok) return __longlong_as_double(q);
+  return ldexp((double)fx_diag_value(q), in.ec + fx_diag_shift(q) - 61);
+}
+
+// 2^k (H x)(l, i) in FP64, from global memory (the rare rows; one point per call).
+template <int ST>
+__device__ __noinline__ double2 h_point_fp64(const FxIn &in, int l, int i) {
+  const double2 z = make_double2(0.0, 0.0);
+  const size_t idx = (size_t)l * in.N + i;
+  StencilIn s{};
+  s.x = in.x;
+  s.N = in.N;
+  s.L = in.L;
+  s.c1 = in.c1;
+  s.c2 = in.c2;
+  const double Er = __dmul_rn(in.E, in.rj[i]);
+  constexpr bool CG = true;
+  const double2 prev = l > 0 ? ldx<CG>(in.x + idx - in.N) : z;
+  const double2 next = l < in.L ? ldx<CG>(in.x + idx + in.N) : z;
+  const double2 t = h_point<ST, true, CG>(s, in.x + (size_t)l * in.N, i, fx_diag_double(in, in.diagq[idx]), prev,
+                                          ldx<CG>(in.x + idx), next, __dmul_rn(in.kappa[l], Er),
+                                          __dmul_rn(in.kappa[l + 1], Er));
+  return make_double2(ldexp(t.x, in.k), ldexp(t.y, in.k));
+}
+
+// ---- staging ------------------------------------------------------------------
+// A warp's rows arrive in a ring of kFxSlots slots of shared memory, each lane's
+// own columns by its own cp.async copies, so a lane waits only for itself and
+// no barrier is needed: of row r the operand, of the rows the warp computes
+// also the diagonal and EX further vectors (the epilogue's).  While row l is
+// computed row l + 2 is in flight.  Register double buffering of the operand
+// alone left the epilogue's loads exposed (the top stall) and spilled.
+constexpr int kFxSlots = 3;
+template <int EX>
+constexpr int fx_slot_bytes() { return (2 + 2 * EX + 1) * 32 * 16; }
+template <int EX>
+constexpr int fx_warp_bytes() { return kFxSlots * fx_slot_bytes<EX>(); }
+
+template <int EX>
+struct FxExtra {
+  const double2 *p[EX > 0 ? EX : 1];
+};
+
+// `have` false fills with zeros and reads nothing (the source is then outside the array).
+__device__ __forceinline__ void cp_async16(unsigned dst, const void *src, bool have) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(have ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async8(unsigned dst, const void *src, bool have) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(have ? 8 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
+
+// A row of the strip in fixed point: the lane's two columns.
+struct FxRow {
+  int64_t X[2][2];   // [column][re, im]
+  int e;             // their exponent field (0: zero)
+  bool ok;           // every value of the strip finite (uniform)
+};
+
+__device__ __forceinline__ uint32_t fx_field(double v) { return (uint32_t)__double2hiint(v) & kExpMask; }
+__device__ __forceinline__ int64_t fx_word(double v, uint32_t m) {
+  return fx_from_words(__double2hiint(v), __double2loint(v), m);
+}
+__device__ __forceinline__ int64_t fx_small(double v, int e) {
+  return fx_from_small(__double2hiint(v), __double2loint(v), e);
+}
+
+__device__ __forceinline__ void fx_convert(const double2 &v0, const double2 &v1, FxRow &r) {
+  const uint32_t m = max(max(fx_field(v0.x), fx_field(v0.y)), max(fx_field(v1.x), fx_field(v1.y)));
+  r.e = (int)(m >> 20);
+  r.ok = true;
+  constexpr uint32_t kLo = (uint32_t)kExpSmall << 20;
+  if (__all_sync(0xffffffffu, m - kLo < kExpMask - kLo)) {   // kLo <= m < kExpMask
+    r.X[0][0] = fx_word(v0.x, m);
+    r.X[0][1] = fx_word(v0.y, m);
+    r.X[1][0] = fx_word(v1.x, m);
+    r.X[1][1] = fx_word(v1.y, m);
+  } else {
+    r.ok = __all_sync(0xffffffffu, m != kExpMask) != 0;
+    const int e = max(r.e, 1);
+    r.X[0][0] = fx_small(v0.x, e);
+    r.X[0][1] = fx_small(v0.y, e);
+    r.X[1][0] = fx_small(v1.x, e);
+    r.X[1][1] = fx_small(v1.y, e);
+    r.e = (r.X[0][0] | r.X[0][1] | r.X[1][0] | r.X[1][1]) ? e : 0;
+  }
+}
+
+// V 2^(E - 1079) by the FP64 pipe's integer conversion and an addition to the exponent field.
+__device__ __forceinline__ double fx_result(int64_t V, int E) {
+  const double t = __ll2double_rn(V);
+  const int h = __double2hiint(t);
+  return __hiloint2double(h ? h + ((E - 1079) << 20) : 0, __double2loint(t));
+}
+
+__device__ __forceinline__ int64_t fx_shfl_up(int64_t v) { return __shfl_up_sync(0xffffffffu, v, 1); }
+__device__ __forceinline__ int64_t fx_shfl_down(int64_t v) { return __shfl_down_sync(0xffffffffu, v, 1); }
+
+// Walk rows [l0, l1) of the strip whose first output column is j0: calls
+// f(idx, 2^k (H x), x, extra values) for every output point.  Every lane of the
+// warp calls it with the same j0, l0, l1; ring: the warp's fx_warp_bytes<EX>()
+// of shared memory.  The operand and the extra vectors are read through L2.
+template <int ST, int EX, typename F>
+__device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX> &ex, unsigned char *ring, int j0,
+                                                int l0, int l1, F &&f) {
+  const int N = in.N, L = in.L;
+  const int lane = threadIdx.x & 31;
+  const int j = j0 - 2 + 2 * lane;                         // this lane's first column
+  const bool have0 = j >= 0 && j < N, have1 = j + 1 >= 0 && j + 1 < N;
+  const bool inner = lane >= 1 && lane <= 30;
+  const bool out0 = inner && have0, out1 = inner && have1;
+  // the lane's parts of a slot: 16-byte columns x0, x1, extras, diagonal pair
+  unsigned char *mine = ring + lane * 16;
+  const unsigned smine = (unsigned)__cvta_generic_to_shared(mine);
+  constexpr int kSlot = fx_slot_bytes<EX>();
+  int so = (l0 - 1) * N + j;                               // the lane's element of the next row to stage
+  auto stage = [&](int r, int slot) {
+    const unsigned d = smine + slot * kSlot;
+    if (r <= l1) {   // rows -1 and L + 1 come out as zeros
+      const bool inside = r >= 0 && r <= L;
+      cp_async16(d, in.x + so, have0 && inside);
+      cp_async16(d + 512, in.x + so + 1, have1 && inside);
+    }
+    if (r >= l0 && r < l1) {
+#pragma unroll
+      for (int q = 0; q < EX; ++q) {
+        cp_async16(d + 1024 + 1024 * q, ex.p[q] + so, out0);
+        cp_async16(d + 1536 + 1024 * q, ex.p[q] + so + 1, out1);
+      }
+      cp_async8(d + 1024 + 1024 * EX, in.diagq + so, out0);
+      cp_async8(d + 1024 + 1024 * EX + 8, in.diagq + so + 1, out1);
+    }
+    cp_async_commit();
+    so = (int)((unsigned)so + (unsigned)N);   // past the last row it is not used
+  };
+  auto slot_x = [&](int slot, int c) { return *reinterpret_cast<const double2 *>(mine + slot * kSlot + 512 * c); };
+  auto slow = [&](int l, int slot) {
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c)
+      if (c == 0 ? out0 : out1) {
+        double2 e[EX > 0 ? EX : 1];
+#pragma unroll
+        for (int q = 0; q < EX; ++q)
+          e[q] = *reinterpret_cast<const double2 *>(mine + slot * kSlot + 1024 + 1024 * q + 512 * c);
+        f(l * N + j + c, h_point_fp64<ST>(in, l, j + c), slot_x(slot, c), e);
+      }
+  };
+  // the coupling w_j = E r_j of the lane's columns
+  const double w0 = have0 ? __dmul_rn(in.E, in.rj[j]) : 0.0, w1 = have1 ? __dmul_rn(in.E, in.rj[j + 1]) : 0.0;
+  stage(l0 - 1, 0);
+  stage(l0, 1);
+  stage(l0 + 1, 2);
+  const uint32_t wm = max(fx_field(w0), fx_field(w1));
+  const bool all_ok = in.ok && __all_sync(0xffffffffu, wm != kExpMask) != 0;
+  const int we = max((int)(wm >> 20), 1), ew = we - 1022;  // w = W 2^(ew - 60)
+  const Limb W[2] = {fx_limbs(fx_small(w0, we)), fx_limbs(fx_small(w1, we))};
+  const bool has_w = (W[0].h | W[0].l | W[1].h | W[1].l) != 0;
+  auto coupling = [&](int l, Limb (&a)[2]) {               // a = kappa_l w = A 2^(ew - 61)
+    const Limb kp = fx_limbs(fx_coef((uint64_t)__double_as_longlong(__ldg(in.kappa + l)), 0));
+    a[0] = fx_limbs(fx_coef_product(kp, W[0]));
+    a[1] = fx_limbs(fx_coef_product(kp, W[1]));
+  };
+  const Limb k1 = fx_limbs(in.c1q), k2 = fx_limbs(in.c2q);
+  Limb acur[2], anext[2];
+  coupling(l0, acur);
+  FxRow prev, cur, next;
+  cp_async_wait<1>();
+  fx_convert(slot_x(0, 0), slot_x(0, 1), prev);
+  fx_convert(slot_x(1, 0), slot_x(1, 1), cur);
+  stage(l0 + 2, 0);
+  int s0 = 1, s1 = 2;                                      // slots of rows l and l + 1
+#pragma unroll 1
+  for (int l = l0; l < l1; ++l) {
+    cp_async_wait<1>();
+    fx_convert(slot_x(s1, 0), slot_x(s1, 1), next);
+    coupling(l + 1, anext);
+    const int eU = __shfl_up_sync(0xffffffffu, cur.e, 1), eD = __shfl_down_sync(0xffffffffu, cur.e, 1);
+    // exponent of the point's sum: the largest of its terms', coefficients included
+    const int eb = max(cur.e, max(eU, eD));
+    const int EP = (prev.e && has_w) ? prev.e + ew : kNone;
+    const int EN = (next.e && has_w) ? next.e + ew : kNone;
+    const int Em = max(eb ? eb + in.ec : kNone, max(EP, EN));
+    if (all_ok && prev.ok && cur.ok && next.ok) {
+      const unsigned char *body = mine + s0 * kSlot;
+      const longlong2 dq = *reinterpret_cast<const longlong2 *>(body + 1024 + 1024 * EX);
+      // every operand is moved to that exponent before its product
+      const int eL = Em == kNone ? 0 : Em - in.ec;
+      const int sC = min(eL - cur.e, 63), sU = min(eL - eU, 63), sD = min(eL - eD, 63);
+      const int sP = min(Em - EP, 63), sN = min(Em - EN, 63);
+      const int E = Em + in.k;
+      int64_t V[2][2];
+      // the sums without (D = false) or with the diagonal's term
+      auto sums = [&](auto with_d) {
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+          const int64_t lB = fx_shfl_up(cur.X[1][p]) >> sU, rA = fx_shfl_down(cur.X[0][p]) >> sD;
+          int64_t lA = 0, rB = 0;
+          if (ST == 5) {
+            lA = fx_shfl_up(cur.X[0][p]) >> sU;
+            rB = fx_shfl_down(cur.X[1][p]) >> sD;
+          }
+          const int64_t A = cur.X[0][p] >> sC, B = cur.X[1][p] >> sC;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            int64_t hh = 0, mm = kHalf;
+            fx_mac(fx_limbs(c == 0 ? lB + B : A + rA), k1, hh, mm);
+            if (ST == 5) fx_mac(fx_limbs(c == 0 ? lA + rA : lB + rB), k2, hh, mm);
+            fx_mac(fx_limbs(prev.X[c][p] >> sP), acur[c], hh, mm);
+            fx_mac(fx_limbs(next.X[c][p] >> sN), anext[c], hh, mm);
+            if (decltype(with_d)::value) fx_mac(fx_limbs(c == 0 ? A : B), fx_limbs(c == 0 ? dq.x : dq.y), hh, mm);
+            V[c][p] = fx_value(hh, mm);
+          }
+        }
+      };
+      int Ev[2] = {E, E};
+      if (!__any_sync(0xffffffffu, ((dq.x | dq.y) & kDiagMask) != 0)) {
+        sums(std::true_type{});
+      } else {   // entries above 2^ec: the other terms move down to their scale
+        sums(std::false_type{});
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const int64_t d = c == 0 ? dq.x : dq.y;
+          const int s = fx_diag_shift(d);
+#pragma unroll
+          for (int p = 0; p < 2; ++p) {
+            int64_t hd = 0, md = kHalf;
+            fx_mac(fx_limbs(cur.X[c][p] >> sC), fx_limbs(fx_diag_value(d)), hd, md);
+            V[c][p] = (V[c][p] >> s) + fx_value(hd, md);
+          }
+          Ev[c] += s;
+        }
+      }
+      double t[2][2];
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int p = 0; p < 2; ++p) t[c][p] = fx_result(V[c][p], Ev[c]);
+      if (!__all_sync(0xffffffffu, Em == kNone || (E >= kOutLo && E <= kOutHi))) {   // near FP64's limits
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int p = 0; p < 2; ++p)
+            t[c][p] = ldexp(fx_double(fx_to_bits(V[c][p], 1000)), V[c][p] ? Ev[c] - 1000 : 0);
+      }
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        if (c == 0 ? out0 : out1) {
+          double2 e[EX > 0 ? EX : 1];
+#pragma unroll
+          for (int q = 0; q < EX; ++q) e[q] = *reinterpret_cast<const double2 *>(body + 1024 + 1024 * q + 512 * c);
+          f(l * N + j + c, make_double2(t[c][0], t[c][1]), *reinterpret_cast<const double2 *>(body + 512 * c), e);
+        }
+    } else {
+      slow(l, s0);
+    }
+    stage(l + 3, s0);
+    const int s2 = kFxSlots - s0 - s1;
+    s0 = s1;
+    s1 = s2;
+    prev = cur;
+    cur = next;
+    acur[0] = anext[0];
+    acur[1] = anext[1];
+  }
+  cp_async_wait<0>();   // the ring is free for the next call
+}
+
+}  // namespace stencil
+}  // namespace tdse_dev
