@@ -44,16 +44,17 @@ using namespace stencil;
 #ifndef TDSE_CHUNK_SEGS
 #define TDSE_CHUNK_SEGS 64
 #endif
-#ifndef TDSE_CHUNK_PTS
-#define TDSE_CHUNK_PTS 2048
-#endif
 #ifndef TDSE_TILE_ROWS
 #define TDSE_TILE_ROWS 32
 #endif
 // Reduction chunks.  Their sizes fix each instance's summation order, so they
 // are compile-time constants (the launch schedule never changes them).
 constexpr int kChunkSegs = TDSE_CHUNK_SEGS;  // 32-point row segments per chunk (stencil kernels)
-constexpr int kChunkPts = TDSE_CHUNK_PTS;    // consecutive points per chunk (elementwise kernels)
+// Consecutive points per chunk of the elementwise kernels: small enough that a
+// batch of a few instances fills the SMs' warps, and one size for all, since a
+// warp takes an equal count of chunks.  The partials use the dipole kernel's
+// slots (one per 512 points).
+constexpr int kChunkPts = 512;
 constexpr int kFxThreads = 128;              // threads of a block of the fixed-point stencil kernel
 constexpr int kFxBlocksPerSM = 4;            // 128 registers a thread
 constexpr int kFxMaxRows = 32;               // segments of a chunk at most (16: 5% slower on large batches)
@@ -239,6 +240,79 @@ __device__ __forceinline__ void for_my_chunks(const ChunkList &cl, F &&f) {
   }
 }
 
+// The lane's shares of up to kChunkGroup chunk sums.
+constexpr int kChunkGroup = 4;
+struct ChunkSums {
+  double a[kChunkGroup] = {0.0, 0.0, 0.0, 0.0};
+  __device__ __forceinline__ void set(int q, double v) {
+#pragma unroll
+    for (int k = 0; k < kChunkGroup; ++k)
+      if (k == q) a[k] = v;
+  }
+};
+
+// The four sums over the warp, sum (lane >> 3) in every lane: each summed over
+// lane bits 16, 8, 4, 2, 1 as warp_sum does, so a chunk's sum does not depend on
+// which others it is reduced with.  Six additions instead of 20.
+__device__ __forceinline__ double warp_sum4(const ChunkSums &s) {
+  const int lane = threadIdx.x & 31;
+  const bool h = lane & 16, q = lane & 8;
+  const double k0 = h ? s.a[2] : s.a[0], k1 = h ? s.a[3] : s.a[1];
+  const double g0 = h ? s.a[0] : s.a[2], g1 = h ? s.a[1] : s.a[3];
+  const double b0 = k0 + __shfl_xor_sync(0xffffffffu, g0, 16), b1 = k1 + __shfl_xor_sync(0xffffffffu, g1, 16);
+  double v = (q ? b1 : b0) + __shfl_xor_sync(0xffffffffu, q ? b0 : b1, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// The elementwise kernels' loop: f(inst, I, ci, n, sums) works on the n <=
+// kChunkGroup chunks from ci and leaves the lane's share of each one's sum;
+// fin(inst, total) runs in one lane once an instance's chunks are all in, with
+// their sum in chunk order.  A warp's chunks are consecutive: it reduces four at
+// a time and reports once per instance it touched, so that small chunks, which
+// a batch of a few instances needs to fill the warps, cost a large batch little
+// (one reduction and one atomic a chunk of 512 points made its elementwise
+// kernels 1.5 times slower than chunks of 2048).
+template <typename F, typename Fin>
+__device__ __forceinline__ void for_elem_chunks(const BatchDev &B, const ChunkList &cl, F &&f, Fin &&fin) {
+  long long c0, c1;
+  warp_range(cl.total, c0, c1);
+  if (c0 >= c1) return;
+  const int lane = threadIdx.x & 31;
+  int p = find_owner(cl, (int)c0);
+  for (int gc = (int)c0; gc < (int)c1;) {
+    while (cl.cpre[p + 1] <= gc) ++p;
+    const int inst = cl.act[p];
+    const BatchInst I = B.inst[inst];
+    const int end = min((int)c1, cl.cpre[p + 1]), count = end - gc;
+    for (; gc < end; gc += kChunkGroup) {
+      const int ci = gc - cl.cpre[p], n = min(kChunkGroup, end - gc);
+      ChunkSums sums;
+      f(inst, I, ci, n, sums);
+      const double v = warp_sum4(sums);
+      if ((lane & 7) == 0 && (lane >> 3) < n) I.dpart[ci + (lane >> 3)] = v;
+    }
+    gc = end;
+    __threadfence();
+    __syncwarp();
+    unsigned last = 0;
+    if (lane == 0)
+      last = (atomicAdd(&B.ticket[inst], (unsigned)count) + (unsigned)count == (unsigned)I.nchunk_e) ? 1u : 0u;
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (!last) continue;
+    __threadfence();
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = lane; c < I.nchunk_e; c += 32) s += __ldcg(&I.dpart[c]);
+    s = warp_sum(s);
+    if (lane == 0) {
+      B.ticket[inst] = 0u;
+      fin(inst, s);
+    }
+  }
+}
+
 // ---- FP64 ------------------------------------------------------------------
 __device__ __forceinline__ StencilIn fp64_in(const BatchDev &B, const BatchInst &I, int inst,
                                              const double2 *x) {
@@ -414,49 +488,49 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
 // U_{j+1} = z - alpha_j s_j U_j and beta_j = g_j ||U_{j+1}||, chunk by chunk.
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     bt_lanczos_b_fp64(BatchDev B, ChunkList cl, int j) {
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     LanczosScalars *ls = B.ls + inst;
     const long long G = (long long)I.N * (I.L + 1);
     const double2 *u = (j == 0) ? I.psi : I.work + (long long)j * G;
     const double2 *z = I.work;
     double2 *un = I.work + (long long)(j + 1) * G;
     const double c = ls->acoef[j];
-    double acc = 0.0;
-    struct ZU { double2 z, u; };
-    chunk_points_x4(I, ci, [&](size_t idx) { return ZU{z[idx], u[idx]}; },
-                    [&](size_t idx, int, const ZU &v) {
-      const double2 o = make_double2(__fma_rn(c, v.u.x, v.z.x), __fma_rn(c, v.u.y, v.z.y));
-      un[idx] = o;
-      acc = __fma_rn(o.x, o.x, acc);
-      acc = __fma_rn(o.y, o.y, acc);
-    });
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
-      store_beta(ls, j, s);
+    for (int q = 0; q < n; ++q) {
+      double acc = 0.0;
+      struct ZU { double2 z, u; };
+      chunk_points_x4(I, ci + q, [&](size_t idx) { return ZU{z[idx], u[idx]}; },
+                      [&](size_t idx, int, const ZU &v) {
+        const double2 o = make_double2(__fma_rn(c, v.u.x, v.z.x), __fma_rn(c, v.u.y, v.z.y));
+        un[idx] = o;
+        acc = __fma_rn(o.x, o.x, acc);
+        acc = __fma_rn(o.y, o.y, acc);
+      });
+      sums.set(q, acc);
     }
+  }, [&](int inst, double s) {
+    store_beta(B.ls + inst, j, s);
   });
 }
 
 // ||psi|| -> sigma_0, psinorm (FP64).
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     bt_norm_fp64(BatchDev B, ChunkList cl) {
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     const double2 *x = I.psi;
-    double acc = 0.0;
-    chunk_points_x4(I, ci, [&](size_t idx) { return x[idx]; }, [&](size_t, int, const double2 &v) {
-      acc = __fma_rn(v.x, v.x, acc);
-      acc = __fma_rn(v.y, v.y, acc);
-    });
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
-      LanczosScalars *ls = B.ls + inst;
-      const double nrm = sqrt(s);
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
+    for (int q = 0; q < n; ++q) {
+      double acc = 0.0;
+      chunk_points_x4(I, ci + q, [&](size_t idx) { return x[idx]; }, [&](size_t, int, const double2 &v) {
+        acc = __fma_rn(v.x, v.x, acc);
+        acc = __fma_rn(v.y, v.y, acc);
+      });
+      sums.set(q, acc);
     }
+  }, [&](int inst, double s) {
+    LanczosScalars *ls = B.ls + inst;
+    const double nrm = sqrt(s);
+    ls->psinorm = nrm;
+    ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+    if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
   });
 }
 
@@ -467,8 +541,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
   // the chunk's coefficients, one copy per warp
   __shared__ double2 wcoef[kElemThreads / 32][kMaxKrylov];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     LanczosScalars *ls = B.ls + inst;
     const long long G = (long long)I.N * (I.L + 1);
     double2 *psi = I.psi;
@@ -479,56 +552,58 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     if (lane < k) wcoef[wib][lane] = ls->coef[lane];
     __syncwarp();
     const double2 c0 = wcoef[wib][0];
-    double acc = 0.0;
-    // kCombinePts points at a time, Krylov vector by Krylov vector
-    chunk_groups_of<kCombinePts>(I, ci, [&](const size_t (&ix)[kCombinePts], const int (&iq)[kCombinePts], int nq) {
-      double ox[kCombinePts], oy[kCombinePts];
-#pragma unroll
-      for (int q = 0; q < kCombinePts; ++q) {
-        if (q < nq) {
-          const double2 u0 = psi[ix[q]];
-          ox[q] = __fma_rn(c0.x, u0.x, __dmul_rn(-c0.y, u0.y));
-          oy[q] = __fma_rn(c0.x, u0.y, __dmul_rn(c0.y, u0.x));
-        }
-      }
-      for (int jj = 1; jj < k; ++jj) {
-        double2 u[kCombinePts];
-#pragma unroll
-        for (int q = 0; q < kCombinePts; ++q)
-          if (q < nq) u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
-        const double2 c = wcoef[wib][jj];
+    for (int q = 0; q < n; ++q) {
+      double acc = 0.0;
+      // kCombinePts points at a time, Krylov vector by Krylov vector
+      chunk_groups_of<kCombinePts>(I, ci + q, [&](const size_t (&ix)[kCombinePts], const int (&iq)[kCombinePts], int nq) {
+        double ox[kCombinePts], oy[kCombinePts];
 #pragma unroll
         for (int q = 0; q < kCombinePts; ++q) {
           if (q < nq) {
-            ox[q] = __fma_rn(c.x, u[q].x, ox[q]);
-            ox[q] = __fma_rn(-c.y, u[q].y, ox[q]);
-            oy[q] = __fma_rn(c.x, u[q].y, oy[q]);
-            oy[q] = __fma_rn(c.y, u[q].x, oy[q]);
+            const double2 u0 = psi[ix[q]];
+            ox[q] = __fma_rn(c0.x, u0.x, __dmul_rn(-c0.y, u0.y));
+            oy[q] = __fma_rn(c0.x, u0.y, __dmul_rn(c0.y, u0.x));
           }
         }
-      }
+        for (int jj = 1; jj < k; ++jj) {
+          double2 u[kCombinePts];
 #pragma unroll
-      for (int q = 0; q < kCombinePts; ++q) {
-        if (q < nq) {
-          if (mask_on && iq[q] >= I.mask_start) {
-            const double mv = mask[iq[q]];
-            ox[q] = __dmul_rn(mv, ox[q]);
-            oy[q] = __dmul_rn(mv, oy[q]);
+          for (int q = 0; q < kCombinePts; ++q)
+            if (q < nq) u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
+          const double2 c = wcoef[wib][jj];
+#pragma unroll
+          for (int q = 0; q < kCombinePts; ++q) {
+            if (q < nq) {
+              ox[q] = __fma_rn(c.x, u[q].x, ox[q]);
+              ox[q] = __fma_rn(-c.y, u[q].y, ox[q]);
+              oy[q] = __fma_rn(c.x, u[q].y, oy[q]);
+              oy[q] = __fma_rn(c.y, u[q].x, oy[q]);
+            }
           }
-          psi[ix[q]] = make_double2(ox[q], oy[q]);
-          acc = __fma_rn(ox[q], ox[q], acc);
-          acc = __fma_rn(oy[q], oy[q], acc);
         }
-      }
-    });
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
-      const double nrm = sqrt(s);
-      ls->psinorm0 = ls->psinorm;
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
+#pragma unroll
+        for (int q = 0; q < kCombinePts; ++q) {
+          if (q < nq) {
+            if (mask_on && iq[q] >= I.mask_start) {
+              const double mv = mask[iq[q]];
+              ox[q] = __dmul_rn(mv, ox[q]);
+              oy[q] = __dmul_rn(mv, oy[q]);
+            }
+            psi[ix[q]] = make_double2(ox[q], oy[q]);
+            acc = __fma_rn(ox[q], ox[q], acc);
+            acc = __fma_rn(oy[q], oy[q], acc);
+          }
+        }
+      });
+      sums.set(q, acc);
     }
+  }, [&](int inst, double s) {
+    LanczosScalars *ls = B.ls + inst;
+    const double nrm = sqrt(s);
+    ls->psinorm0 = ls->psinorm;
+    ls->psinorm = nrm;
+    ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+    if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
   });
 }
 
@@ -613,8 +688,7 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
 template <bool SPLIT>
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     bt_lanczos_b_mixed(BatchDev B, ChunkList cl, int j) {
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     LanczosScalars *ls = B.ls + inst;
     const long long G = (long long)I.N * (I.L + 1);
     const float2 *u = I.mwork + (long long)j * G;
@@ -622,58 +696,58 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     const float2 *z = I.mwork;
     float2 *un = I.mwork + (long long)(j + 1) * G;
     const float c = (float)ls->acoef[j];
-    PairSum acc;
-    struct ZU { float2 z, u; };
-    chunk_points_x4(I, ci, [&](size_t idx) {
-      float2 uu;
-      if (!SPLIT) {
-        uu = u[idx];
-      } else {
-        const float2 h = hi[idx], lw = lo[idx];
-        uu = make_float2(h.x + lw.x, h.y + lw.y);
-      }
-      return ZU{z[idx], uu};
-    }, [&](size_t idx, int, const ZU &v) {
-      const float2 o = make_float2(fmaf(c, v.u.x, v.z.x), fmaf(c, v.u.y, v.z.y));
-      un[idx] = o;
-      acc.add(fmaf(o.x, o.x, o.y * o.y));
-    });
-    const double accd = acc.value();
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
-      const double beta = sqrt(s);
-      ls->beta[j] = beta;
-      const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
-      ls->sigma[j + 1] = sn;
-      ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
+    for (int q = 0; q < n; ++q) {
+      PairSum acc;
+      struct ZU { float2 z, u; };
+      chunk_points_x4(I, ci + q, [&](size_t idx) {
+        float2 uu;
+        if (!SPLIT) {
+          uu = u[idx];
+        } else {
+          const float2 h = hi[idx], lw = lo[idx];
+          uu = make_float2(h.x + lw.x, h.y + lw.y);
+        }
+        return ZU{z[idx], uu};
+      }, [&](size_t idx, int, const ZU &v) {
+        const float2 o = make_float2(fmaf(c, v.u.x, v.z.x), fmaf(c, v.u.y, v.z.y));
+        un[idx] = o;
+        acc.add(fmaf(o.x, o.x, o.y * o.y));
+      });
+      sums.set(q, acc.value());
     }
+  }, [&](int inst, double s) {
+    LanczosScalars *ls = B.ls + inst;
+    const double beta = sqrt(s);
+    ls->beta[j] = beta;
+    const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
+    ls->sigma[j + 1] = sn;
+    ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
   });
 }
 
 // psi -> (hi, lo) and ||psi|| (FP32 products summed in FP32 pairs, then FP64).
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     bt_split_mixed(BatchDev B, ChunkList cl) {
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     const double2 *x = I.psi;
     float2 *hi = I.hi, *lo = I.lo;
-    PairSum acc;
-    chunk_points_x4(I, ci, [&](size_t idx) { return x[idx]; }, [&](size_t idx, int, const double2 &v) {
-      float2 h, lw;
-      split2(v, h, lw);
-      hi[idx] = h;
-      lo[idx] = lw;
-      acc.add(fmaf(h.x, h.x, h.y * h.y));
-    });
-    const double accd = acc.value();
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
-      LanczosScalars *ls = B.ls + inst;
-      const double nrm = sqrt(s);
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
+    for (int q = 0; q < n; ++q) {
+      PairSum acc;
+      chunk_points_x4(I, ci + q, [&](size_t idx) { return x[idx]; }, [&](size_t idx, int, const double2 &v) {
+        float2 h, lw;
+        split2(v, h, lw);
+        hi[idx] = h;
+        lo[idx] = lw;
+        acc.add(fmaf(h.x, h.x, h.y * h.y));
+      });
+      sums.set(q, acc.value());
     }
+  }, [&](int inst, double s) {
+    LanczosScalars *ls = B.ls + inst;
+    const double nrm = sqrt(s);
+    ls->psinorm = nrm;
+    ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+    if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
   });
 }
 
@@ -715,8 +789,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
   // the chunk's FP32 coefficients, converted once and kept per warp
   __shared__ float2 wcoef[kElemThreads / 32][kMaxKrylov];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     LanczosScalars *ls = B.ls + inst;
     const long long G = (long long)I.N * (I.L + 1);
     double2 *psi = I.psi;
@@ -734,96 +807,97 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
       wcoef[wib][lane] = make_float2((float)cd.x, (float)cd.y);
     }
     __syncwarp();
-    PairSum acc;
-    // kMixedCombinePts points at a time, two Krylov vectors per round (their
-    // loads issued together); each point takes its terms in vector order
-    constexpr int Q = kMixedCombinePts;
-    chunk_groups_of<Q>(I, ci, [&](const size_t (&ix)[Q], const int (&iq)[Q], int nq) {
-      float cx[Q], cy[Q];
+    for (int q = 0; q < n; ++q) {
+      PairSum acc;
+      // kMixedCombinePts points at a time, two Krylov vectors per round (their
+      // loads issued together); each point takes its terms in vector order
+      constexpr int Q = kMixedCombinePts;
+      chunk_groups_of<Q>(I, ci + q, [&](const size_t (&ix)[Q], const int (&iq)[Q], int nq) {
+        float cx[Q], cy[Q];
 #pragma unroll
-      for (int q = 0; q < Q; ++q) cx[q] = cy[q] = 0.f;
-      int jj = 1;
-      for (; jj + 1 < k; jj += 2) {
-        float2 u[Q], u2[Q];
+        for (int q = 0; q < Q; ++q) cx[q] = cy[q] = 0.f;
+        int jj = 1;
+        for (; jj + 1 < k; jj += 2) {
+          float2 u[Q], u2[Q];
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
-          if (q < nq) {
-            u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
-            u2[q] = U1[(size_t)jj * G + ix[q]];
+          for (int q = 0; q < Q; ++q)
+            if (q < nq) {
+              u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
+              u2[q] = U1[(size_t)jj * G + ix[q]];
+            }
+          const float2 c = wcoef[wib][jj], c2 = wcoef[wib][jj + 1];
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            if (q < nq) {
+              cx[q] = fmaf(c.x, u[q].x, cx[q]);
+              cx[q] = fmaf(-c.y, u[q].y, cx[q]);
+              cy[q] = fmaf(c.x, u[q].y, cy[q]);
+              cy[q] = fmaf(c.y, u[q].x, cy[q]);
+              cx[q] = fmaf(c2.x, u2[q].x, cx[q]);
+              cx[q] = fmaf(-c2.y, u2[q].y, cx[q]);
+              cy[q] = fmaf(c2.x, u2[q].y, cy[q]);
+              cy[q] = fmaf(c2.y, u2[q].x, cy[q]);
+            }
           }
-        const float2 c = wcoef[wib][jj], c2 = wcoef[wib][jj + 1];
+        }
+        if (jj < k) {
+          float2 u[Q];
+#pragma unroll
+          for (int q = 0; q < Q; ++q)
+            if (q < nq) u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
+          const float2 c = wcoef[wib][jj];
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            if (q < nq) {
+              cx[q] = fmaf(c.x, u[q].x, cx[q]);
+              cx[q] = fmaf(-c.y, u[q].y, cx[q]);
+              cy[q] = fmaf(c.x, u[q].y, cy[q]);
+              cy[q] = fmaf(c.y, u[q].x, cy[q]);
+            }
+          }
+        }
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
           if (q < nq) {
-            cx[q] = fmaf(c.x, u[q].x, cx[q]);
-            cx[q] = fmaf(-c.y, u[q].y, cx[q]);
-            cy[q] = fmaf(c.x, u[q].y, cy[q]);
-            cy[q] = fmaf(c.y, u[q].x, cy[q]);
-            cx[q] = fmaf(c2.x, u2[q].x, cx[q]);
-            cx[q] = fmaf(-c2.y, u2[q].y, cx[q]);
-            cy[q] = fmaf(c2.x, u2[q].y, cy[q]);
-            cy[q] = fmaf(c2.y, u2[q].x, cy[q]);
+            const float2 ph = hi[ix[q]], pl = lo[ix[q]];
+            // Re: c0x px - c0y py + cx;  Im: c0x py + c0y px + cy
+            float a1, a1l, a2, a2l, b1, b1l, b2, b2l;
+            pair_mul(c0xh, c0xl, ph.x, pl.x, a1, a1l);
+            pair_mul(c0yh, c0yl, ph.y, pl.y, a2, a2l);
+            pair_mul(c0xh, c0xl, ph.y, pl.y, b1, b1l);
+            pair_mul(c0yh, c0yl, ph.x, pl.x, b2, b2l);
+            float sx, ex, sx2, ex2, sy, ey, sy2, ey2;
+            two_sum(a1, -a2, sx, ex);
+            two_sum(sx, cx[q], sx2, ex2);
+            two_sum(b1, b2, sy, ey);
+            two_sum(sy, cy[q], sy2, ey2);
+            float oxh, oxl, oyh, oyl;
+            fast_two_sum(sx2, __fadd_rn(__fadd_rn(__fsub_rn(a1l, a2l), ex), ex2), oxh, oxl);
+            fast_two_sum(sy2, __fadd_rn(__fadd_rn(__fadd_rn(b1l, b2l), ey), ey2), oyh, oyl);
+            if (iq[q] >= I.mask_start) {
+              float mh, ml, t, tl;
+              split1(mask[iq[q]], mh, ml);
+              pair_mul(oxh, oxl, mh, ml, t, tl);
+              fast_two_sum(t, tl, oxh, oxl);
+              pair_mul(oyh, oyl, mh, ml, t, tl);
+              fast_two_sum(t, tl, oyh, oyl);
+            }
+            hi[ix[q]] = make_float2(oxh, oyh);
+            lo[ix[q]] = make_float2(oxl, oyl);
+            if (WRITE_PSI) psi[ix[q]] = make_double2((double)oxh + (double)oxl, (double)oyh + (double)oyl);
+            acc.add(fmaf(oxh, oxh, oyh * oyh));
           }
         }
-      }
-      if (jj < k) {
-        float2 u[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q)
-          if (q < nq) u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
-        const float2 c = wcoef[wib][jj];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          if (q < nq) {
-            cx[q] = fmaf(c.x, u[q].x, cx[q]);
-            cx[q] = fmaf(-c.y, u[q].y, cx[q]);
-            cy[q] = fmaf(c.x, u[q].y, cy[q]);
-            cy[q] = fmaf(c.y, u[q].x, cy[q]);
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        if (q < nq) {
-          const float2 ph = hi[ix[q]], pl = lo[ix[q]];
-          // Re: c0x px - c0y py + cx;  Im: c0x py + c0y px + cy
-          float a1, a1l, a2, a2l, b1, b1l, b2, b2l;
-          pair_mul(c0xh, c0xl, ph.x, pl.x, a1, a1l);
-          pair_mul(c0yh, c0yl, ph.y, pl.y, a2, a2l);
-          pair_mul(c0xh, c0xl, ph.y, pl.y, b1, b1l);
-          pair_mul(c0yh, c0yl, ph.x, pl.x, b2, b2l);
-          float sx, ex, sx2, ex2, sy, ey, sy2, ey2;
-          two_sum(a1, -a2, sx, ex);
-          two_sum(sx, cx[q], sx2, ex2);
-          two_sum(b1, b2, sy, ey);
-          two_sum(sy, cy[q], sy2, ey2);
-          float oxh, oxl, oyh, oyl;
-          fast_two_sum(sx2, __fadd_rn(__fadd_rn(__fsub_rn(a1l, a2l), ex), ex2), oxh, oxl);
-          fast_two_sum(sy2, __fadd_rn(__fadd_rn(__fadd_rn(b1l, b2l), ey), ey2), oyh, oyl);
-          if (iq[q] >= I.mask_start) {
-            float mh, ml, t, tl;
-            split1(mask[iq[q]], mh, ml);
-            pair_mul(oxh, oxl, mh, ml, t, tl);
-            fast_two_sum(t, tl, oxh, oxl);
-            pair_mul(oyh, oyl, mh, ml, t, tl);
-            fast_two_sum(t, tl, oyh, oyl);
-          }
-          hi[ix[q]] = make_float2(oxh, oyh);
-          lo[ix[q]] = make_float2(oxl, oyl);
-          if (WRITE_PSI) psi[ix[q]] = make_double2((double)oxh + (double)oxl, (double)oyh + (double)oyl);
-          acc.add(fmaf(oxh, oxh, oyh * oyh));
-        }
-      }
-    });
-    const double accd = acc.value();
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, accd, s) && (threadIdx.x & 31) == 0) {
-      const double nrm = sqrt(s);
-      ls->psinorm0 = ls->psinorm;
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
+      });
+      sums.set(q, acc.value());
     }
+  }, [&](int inst, double s) {
+    LanczosScalars *ls = B.ls + inst;
+    const double nrm = sqrt(s);
+    ls->psinorm0 = ls->psinorm;
+    ls->psinorm = nrm;
+    ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+    if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
   });
 }
 
@@ -878,27 +952,28 @@ __global__ void __launch_bounds__(256) bt_diag_table(BatchInst I, double c0) {
 // of the step (the decay rate of the norm).
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     bt_imag_normalize(BatchDev B, ChunkList cl, const double *__restrict__ dtau, double *energy) {
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
+  for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
     LanczosScalars *ls = B.ls + inst;
     const double n1 = ls->psinorm;   // every chunk reads it before the last one rewrites it
     const double sc = 1.0 / (sqrt(I.dr) * n1);
     double2 *x = I.psi;
-    double acc = 0.0;
-    chunk_points_x4(I, ci, [&](size_t idx) { return x[idx]; }, [&](size_t idx, int, const double2 &v) {
-      const double2 o = make_double2(__dmul_rn(sc, v.x), __dmul_rn(sc, v.y));
-      x[idx] = o;
-      acc = __fma_rn(o.x, o.x, acc);
-      acc = __fma_rn(o.y, o.y, acc);
-    });
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk_e, acc, s) && (threadIdx.x & 31) == 0) {
-      const double nrm = sqrt(s);
-      energy[inst] = -log(n1 / ls->psinorm0) / dtau[inst];
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-      if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
+    for (int q = 0; q < n; ++q) {
+      double acc = 0.0;
+      chunk_points_x4(I, ci + q, [&](size_t idx) { return x[idx]; }, [&](size_t idx, int, const double2 &v) {
+        const double2 o = make_double2(__dmul_rn(sc, v.x), __dmul_rn(sc, v.y));
+        x[idx] = o;
+        acc = __fma_rn(o.x, o.x, acc);
+        acc = __fma_rn(o.y, o.y, acc);
+      });
+      sums.set(q, acc);
     }
+  }, [&](int inst, double s) {
+    LanczosScalars *ls = B.ls + inst;
+    const double nrm = sqrt(s);
+    energy[inst] = -log(ls->psinorm / ls->psinorm0) / dtau[inst];
+    ls->psinorm = nrm;
+    ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+    if (!isfinite(s)) atomicOr(B.status, kStatusNonFinite);
   });
 }
 
@@ -1096,7 +1171,6 @@ struct Layout {
       rinvf, total;
 };
 
-// Tiles of the mixed tile kernel on an N x (L+1) grid.
 // Row segments and segments per chunk of the fixed-point stencil kernel: at
 // least ~512 chunks an instance, so that a handful of instances fills the SMs'
 // warps, between 32 segments (a chunk loads two halo rows beside its own) and
@@ -1108,12 +1182,13 @@ int fx_chunk_rows(size_t N, size_t Lp1) {
   return (int)std::max((nseg + room - 1) / room, std::min<size_t>(kFxMaxRows, nseg / 512));
 }
 
+// Tiles of the mixed tile kernel on an N x (L+1) grid.
 int tile_count(int N, int L) { return ((N + kTileCols - 1) / kTileCols) * ((L + kTileRows) / kTileRows); }
 
 Layout layout_of(const tdse_instance_spec &s, int precision) {
   const size_t N = (size_t)s.N, Lp1 = (size_t)s.lmax + 1, G = N * Lp1, m = (size_t)s.krylov;
   const size_t nseg = ((N + 31) / 32) * Lp1;
-  const size_t nchunk = std::max({(nseg + kChunkSegs - 1) / kChunkSegs, (G + kChunkPts - 1) / kChunkPts,
+  const size_t nchunk = std::max({(nseg + kChunkSegs - 1) / kChunkSegs, (G + 2047) / 2048,
                                   (size_t)tile_count(s.N, s.lmax)});
   const bool mixed = precision == TDSE_MIXED;
   Layout L;

@@ -46,8 +46,8 @@ struct BatchInst {
   float2 *hi, *lo;       // mixed: split of psi
   double2 *work;         // FP64 Krylov area: slot 0 = z, slots 1..m-1 = U_j
   float2 *mwork;         // mixed Krylov area, same slots
-  double *partial;       // max(nchunk, nchunk_e) chunk partial sums
-  double *dpart;         // 4 * nchunk_d chunk partials of the dipole and the fixed-point stencil kernel
+  double *partial;       // chunk partials of the mixed and the velocity-gauge stencil kernels
+  double *dpart;         // 4 * nchunk_d chunk partials of the dipole, fixed-point stencil and elementwise kernels
   double2 *ref0;         // N values: the p_ground reference (1s state of the grid)
 };
 
