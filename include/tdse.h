@@ -373,8 +373,8 @@ int tdse_apply_h(tdse_t *h, double E, const void *x_dev, void *y_dev);
  * separates stages by cluster barriers and adds the Lanczos dot products and
  * norms in a fixed order (every CTA holds the same sums, and forms the small
  * exponential of each Lanczos step itself).  Taylor and RK4 give bitwise the
- * states of the multi-launch path; Lanczos differs only in the association
- * of its grid sums.  It applies to FP64 length-gauge propagation with no
+ * states of the multi-launch path; Lanczos differs in rounding (its
+ * multi-launch operator runs in fixed point, its grid sums associate otherwise).  It applies to FP64 length-gauge propagation with no
  * per-step observables set up (dipole series, flux, record), when the state
  * and the method's work vectors (Taylor 3, RK4 4, Lanczos order + 1 vectors
  * of the state's size, plus the diagonal table) fit in the cluster's shared
@@ -394,7 +394,7 @@ int tdse_small_grid_path_used(const tdse_t *h);
  * Larger grids: every FP64 length-gauge Lanczos step of a tdse_propagate call
  * in one cooperative launch (Appendix "Lanczos methods"), when no per-step
  * observables are set up.  The multi-launch path issues 2 order + 1 launches
- * per step; here one grid of 2 blocks of 512 threads per SM stays resident,
+ * per step; here one grid of one block of 512 threads per SM stays resident,
  * separates the phases by grid-wide barriers (bounded waits) and has every
  * block add each reduction's block partials in the multi-launch path's fixed
  * order, so the results equal that path's bitwise.  The modes are those of

@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "tdse_fixed.cuh"
 #include "tdse_internal.cuh"
 #include "tdse_pulse.h"
 
@@ -30,6 +31,9 @@ struct tdse {
   size_t work_vecs = 0;
   double *diag = nullptr, *rj = nullptr, *kappa = nullptr, *mask = nullptr;
   double *rinv = nullptr;          // 1 / r_j (velocity gauge)
+  long long *diagq = nullptr;      // diag for the fixed-point walker; null where it does not fit or memory is short
+  long long c1q = 0, c2q = 0;      // c1, c2 likewise
+  int fx_ec = 0;
   int mask_start = 0;
   Reduction *red = nullptr;
   LanczosScalars *ls = nullptr;
@@ -160,6 +164,11 @@ OperatorView view(const tdse *h) {
   op.mask = h->mask;
   op.rinv = h->rinv;
   op.mask_start = (h->opts.absorber) ? h->mask_start : h->g.N;
+  op.diagq = h->diagq;
+  op.c1q = h->c1q;
+  op.c2q = h->c2q;
+  op.fx_ec = h->fx_ec;
+  op.fx_ok = h->diagq ? 1 : 0;
   return op;
 }
 
@@ -170,6 +179,76 @@ MixedView mview(const tdse *h) {
   mv.kappa = h->kappaf;
   mv.rinv = h->rinvf;
   return mv;
+}
+
+void dfree(tdse *h, void *p) {
+  if (!p) return;
+  for (size_t i = 0; i < h->allocs.size(); ++i)
+    if (h->allocs[i].user == p) {
+      cudaFree(h->allocs[i].base);
+      h->allocs.erase(h->allocs.begin() + (long)i);
+      return;
+    }
+  cudaFree(p);
+}
+
+// Device allocation of the handle: bytes between two guard bands of h->guard
+// bytes (0: none), registered so that dfree and the guard check find it.
+template <typename T>
+cudaError_t dmalloc(tdse *h, T **p, size_t bytes, const char *name) {
+  char *base = nullptr;
+  const size_t g = h->guard;
+  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&base), bytes + 2 * g);
+  if (e != cudaSuccess && h->diagq) {   // memory is short: the encoded diagonal is a copy the handle can do without
+    cudaGetLastError();
+    dfree(h, h->diagq);
+    h->diagq = nullptr;
+    e = cudaMalloc(reinterpret_cast<void **>(&base), bytes + 2 * g);
+  }
+  if (e != cudaSuccess) {
+    *p = nullptr;
+    return e;
+  }
+  if (g) {
+    e = cudaMemset(base, 0xff, g);
+    if (e == cudaSuccess) e = cudaMemset(base + g + bytes, 0xff, g);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) {
+      cudaFree(base);
+      *p = nullptr;
+      return e;
+    }
+  }
+  *p = reinterpret_cast<T *>(base + g);
+  h->allocs.push_back({base, base + g, bytes, name});
+  return cudaSuccess;
+}
+#define DMALLOC(h, field, bytes) dmalloc(h, &(h)->field, bytes, #field)
+
+// The fixed-point walker's form of the operator, from the FP64 diagonal on the
+// device; dmax bounds its magnitude.  Left out (the walker then runs in FP64
+// point by point) where the coefficients do not fit the encoding, and where
+// there is no memory for the table.
+int build_fixed(tdse *h, double dmax) {
+  if (!(tdse_fx::fx_scale(h->g.c0, h->fx_ec) && tdse_fx::fx_diag_fits(dmax, h->fx_ec))) {
+    dfree(h, h->diagq);
+    h->diagq = nullptr;
+    return TDSE_OK;
+  }
+  auto coef = [&](double v) {
+    uint64_t u;
+    std::memcpy(&u, &v, 8);
+    return (long long)tdse_fx::fx_coef(u, h->fx_ec);
+  };
+  h->c1q = coef(h->g.c1);
+  h->c2q = coef(h->g.c2);
+  if (!h->diagq && DMALLOC(h, diagq, sizeof(long long) * npts(h)) != cudaSuccess) {
+    cudaGetLastError();
+    h->diagq = nullptr;
+    return TDSE_OK;
+  }
+  TDSE_CUDA(h, launch_fx_diag(h->diag, npts(h), h->fx_ec, h->diagq, h->g, h->stream), "fixed-point diagonal");
+  return TDSE_OK;
 }
 
 // Grid r_j = j*dr + offset (j = 1..N) and the tables of the operator.
@@ -223,48 +302,17 @@ int build_tables(tdse *h) {
   for (int j = 0; j < N; ++j) ri[j] = 1.0 / r[j];
   TDSE_CUDA(h, cudaMemcpyAsync(h->rinv, ri.data(), sizeof(double) * N, cudaMemcpyHostToDevice, s), "copy 1/r");
   TDSE_CUDA(h, cudaMemcpyAsync(h->diag, d.data(), sizeof(double) * d.size(), cudaMemcpyHostToDevice, s), "copy diag");
+  double dmax = 0.0;   // a bound of |diag|: c0 (twice: the ghost's fold), the largest centrifugal term, the potential
+  for (int j = 0; j < N; ++j) {
+    const double V = std::fabs(h->vtab.empty() ? h->Z / r[j] : h->vtab[j]);
+    dmax = V <= 1e300 ? std::fmax(dmax, V) : INFINITY;   // Inf and NaN: Inf, which stays
+  }
+  const int rcf = build_fixed(h, dmax + 2.0 * g.c0 + 0.5 * (double)L * (double)(L + 1) / (r[0] * r[0]));
+  if (rcf) return rcf;
   TDSE_CUDA(h, cudaMemcpyAsync(h->kappa, kap.data(), sizeof(double) * (L + 2), cudaMemcpyHostToDevice, s), "copy kappa");
   TDSE_CUDA(h, cudaMemcpyAsync(h->mask, msk.data(), sizeof(double) * N, cudaMemcpyHostToDevice, s), "copy mask");
   TDSE_CUDA(h, cudaStreamSynchronize(s), "sync tables");
   return TDSE_OK;
-}
-
-// Device allocation of the handle: bytes between two guard bands of h->guard
-// bytes (0: none), registered so that dfree and the guard check find it.
-template <typename T>
-cudaError_t dmalloc(tdse *h, T **p, size_t bytes, const char *name) {
-  char *base = nullptr;
-  const size_t g = h->guard;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&base), bytes + 2 * g);
-  if (e != cudaSuccess) {
-    *p = nullptr;
-    return e;
-  }
-  if (g) {
-    e = cudaMemset(base, 0xff, g);
-    if (e == cudaSuccess) e = cudaMemset(base + g + bytes, 0xff, g);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) {
-      cudaFree(base);
-      *p = nullptr;
-      return e;
-    }
-  }
-  *p = reinterpret_cast<T *>(base + g);
-  h->allocs.push_back({base, base + g, bytes, name});
-  return cudaSuccess;
-}
-#define DMALLOC(h, field, bytes) dmalloc(h, &(h)->field, bytes, #field)
-
-void dfree(tdse *h, void *p) {
-  if (!p) return;
-  for (size_t i = 0; i < h->allocs.size(); ++i)
-    if (h->allocs[i].user == p) {
-      cudaFree(h->allocs[i].base);
-      h->allocs.erase(h->allocs.begin() + (long)i);
-      return;
-    }
-  cudaFree(p);
 }
 
 void free_all(tdse *h) {
@@ -272,6 +320,7 @@ void free_all(tdse *h) {
   dfree(h, h->ref0);
   dfree(h, h->work);
   dfree(h, h->diag);
+  dfree(h, h->diagq);
   dfree(h, h->rj);
   dfree(h, h->rinv);
   dfree(h, h->etab);
@@ -559,6 +608,22 @@ int mx_lanczos_steps(tdse *h, int m, double dt, long nsteps) {
 // bound on the multi-launch path.
 constexpr size_t kSmallGridAutoPoints = 16384;
 
+// The cluster path's plan, cached for one method and order.
+const SmallPlan &small_plan(tdse *h, int method, int order) {
+  if (h->small_method != method || h->small_order != order) {
+    h->small_plan = plan_small_grid(h->g, method, order);
+    h->small_method = method;
+    h->small_order = order;
+  }
+  return h->small_plan;
+}
+
+// Whether the cluster path could run these explicit steps (its shared memory
+// holds at most ~58,000 points): their multi-launch stages then give its bits.
+bool fits_cluster(tdse *h, int method, int order) {
+  return h->g.gauge == 0 && npts(h) <= 65536 && small_plan(h, method, order).ok;
+}
+
 // Run the steps on the cluster path if it applies; *done tells whether it did.
 // The coupling at every step of a one-launch run (three per RK4 step: the
 // stage times; one per Taylor or Lanczos step: the mid-point), on the device.
@@ -601,12 +666,7 @@ int small_grid_steps(tdse *h, int method, int order, double dt, long nsteps, boo
       h->opts.precision != TDSE_FP64 || h->g.gauge != 0)
     return TDSE_OK;
   if (h->small_mode == TDSE_SMALL_GRID_AUTO && npts(h) > kSmallGridAutoPoints) return TDSE_OK;
-  if (h->small_method != method || h->small_order != order) {
-    h->small_plan = plan_small_grid(h->g, method, order);
-    h->small_method = method;
-    h->small_order = order;
-  }
-  if (!h->small_plan.ok) return TDSE_OK;
+  if (!small_plan(h, method, order).ok) return TDSE_OK;
   const int rce = upload_etab(h, method, dt, nsteps);
   if (rce) return rce;
   TDSE_LAUNCH(h, TDSE_K_SMALL_GRID,
@@ -625,7 +685,8 @@ int taylor_steps(tdse *h, int P, double dt, long nsteps) {
   if (rc || done) return rc;
   rc = ensure_work(h, 2);
   if (rc) return rc;
-  const OperatorView op = view(h);
+  OperatorView op = view(h);
+  op.plain = fits_cluster(h, TDSE_TAYLOR, P);
   const size_t G = npts(h);
   double2 *buf[2] = {h->work, h->work + G};
   const double t0 = h->t;
@@ -653,17 +714,18 @@ int rk4_steps(tdse *h, double dt, long nsteps) {
   if (rc || done) return rc;
   rc = ensure_work(h, 3);
   if (rc) return rc;
-  const OperatorView op = view(h);
+  OperatorView op = view(h);
+  op.plain = fits_cluster(h, TDSE_RK4, 4);
   const size_t G = npts(h);
   double2 *ga = h->work, *gb = h->work + G, *acc = h->work + 2 * G;
   const double t0 = h->t;
   for (long n = 0; n < nsteps; ++n) {
     const double tn = t0 + (double)n * dt;
     const double E1 = coupling_at(h, tn), E2 = coupling_at(h, tn + 0.5 * dt), E4 = coupling_at(h, tn + dt);
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E1, 1, dt, h->psi, h->psi, h->psi, acc, ga, nullptr, h->stream), "rk stage 1");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E2, 2, dt, ga, h->psi, acc, acc, gb, nullptr, h->stream), "rk stage 2");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E2, 3, dt, gb, h->psi, acc, acc, ga, nullptr, h->stream), "rk stage 3");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E4, 4, dt, ga, h->psi, acc, nullptr, nullptr, h->psi, h->stream), "rk stage 4");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E1, 1, dt, h->psi, h->psi, acc, ga, nullptr, h->stream), "rk stage 1");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E2, 2, dt, ga, h->psi, acc, gb, nullptr, h->stream), "rk stage 2");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E2, 3, dt, gb, h->psi, acc, ga, nullptr, h->stream), "rk stage 3");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E4, 4, dt, ga, h->psi, acc, nullptr, h->psi, h->stream), "rk stage 4");
     TDSE_HOOK(h, t0 + (double)(n + 1) * dt, dt);
   }
   return TDSE_OK;
@@ -894,10 +956,10 @@ int imag_steps(tdse *h, int method, int order, double dt, long nsteps, double *e
                   "taylor copy");
     } else if (method == TDSE_RK4) {
       double2 *ga = h->work, *gb = h->work + G, *acc = h->work + 2 * G;
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 1, dt, h->psi, h->psi, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 1");
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 2, dt, ga, h->psi, acc, acc, gb, nullptr, h->stream, true), "rk stage 2");
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 3, dt, gb, h->psi, acc, acc, ga, nullptr, h->stream, true), "rk stage 3");
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 4, dt, ga, h->psi, acc, nullptr, nullptr, h->psi, h->stream, true), "rk stage 4");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 1, dt, h->psi, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 1");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 2, dt, ga, h->psi, acc, gb, nullptr, h->stream, true), "rk stage 2");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 3, dt, gb, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 3");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 4, dt, ga, h->psi, acc, nullptr, h->psi, h->stream, true), "rk stage 4");
     } else {
       const int m = order;
       double2 *z = h->work;

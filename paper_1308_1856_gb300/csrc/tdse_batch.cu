@@ -332,44 +332,6 @@ __device__ __forceinline__ StencilIn fp64_in(const BatchDev &B, const BatchInst 
   return in;
 }
 
-// The recurrence's scale.  z = s_j H U_j - (s_j / sigma_j) ratio_j U_{j-1} with
-// s_j the power of two at or below sigma_j (the scale is then an exponent, not
-// a product per point); with g_j = sigma_j / s_j in [1, 2):
-//   alpha_j = sigma_j g_j Re<U_j, z>,  U_{j+1} = z - alpha_j s_j U_j,
-//   beta_j = g_j ||U_{j+1}||.
-// sigma_j = 0 (a vanished vector) keeps s_j = 1, g_j = 0.
-struct StepScale {
-  double s, g;
-  int k;       // s = 2^k
-};
-__device__ __forceinline__ StepScale step_scale(double sigma) {
-  StepScale r;
-  const int f = (__double2hiint(sigma) >> 20) & 0x7ff;
-  const bool usable = f > 0 && f < 0x7ff;
-  r.k = usable ? f - 1023 : 0;
-  r.s = usable ? __hiloint2double(f << 20, 0) : 1.0;
-  r.g = usable ? __hiloint2double((__double2hiint(sigma) & 0xfffff) | 0x3ff00000, __double2loint(sigma)) : sigma;
-  return r;
-}
-
-// alpha_j and U_{j+1}'s coefficient from the sum of U_j^* z.
-__device__ __forceinline__ void store_alpha(LanczosScalars *ls, int j, double sum) {
-  const double sig = ls->sigma[j];
-  const StepScale sc = step_scale(sig);
-  const double al = (sum * sig) * sc.g;
-  ls->alpha[j] = al;
-  ls->acoef[j] = -al * sc.s;
-}
-// beta_j and the next vector's scalars from ||U_{j+1}||^2.
-__device__ __forceinline__ void store_beta(LanczosScalars *ls, int j, double sumsq) {
-  const double nrm = sqrt(sumsq);
-  const double beta = step_scale(ls->sigma[j]).g * nrm;
-  ls->beta[j] = beta;
-  const double sn = (nrm > 0.0) ? 1.0 / nrm : 0.0;
-  ls->sigma[j + 1] = sn;
-  ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
-}
-
 __device__ __forceinline__ FxIn fixed_in(const BatchDev &B, const BatchInst &I, int inst, const double2 *x, int k) {
   FxIn in;
   in.x = x;
@@ -425,13 +387,12 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM) bt_lanczos_a_fixed
     up.p[0] = (j <= 1) ? I.psi : I.work + (long long)(j - 1) * G;
     double2 *z = I.work;
     const StepScale s0 = step_scale(ls->sigma[j]);
-    // ratio_j s_j / sigma_j; g_j = 0 only for a vanished vector, whose ratio is 0
-    const double cprev = (EX > 0 && s0.g > 0.0) ? ls->ratio[j] / s0.g : 0.0;
+    const double cprev = EX > 0 ? ls->ratio[j] : 0.0;
     const FxIn in = fixed_in(B, I, inst, u, s0.k);
     double acc = 0.0;
     chunk_strips(I, ci, [&](int j0, int l0, int l1) {
       walk_rows_fixed<ST, EX>(in, up, ring, j0, l0, l1,
-                              [&](int idx, double2 t, double2 uc, const double2 (&e)[1]) {
+                              [&](int idx, int, double2 t, double2 uc, const double2 (&e)[1]) {
         double2 o = t;
         if (EX > 0) {
           o.x = __fma_rn(-cprev, e[0].x, t.x);
@@ -461,7 +422,7 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
     double2 *z = I.work;
     const double sig = ls->sigma[j];
     const StepScale sc = step_scale(sig);
-    const double cprev = (j > 0 && sc.g > 0.0) ? ls->ratio[j] / sc.g : 0.0;
+    const double cprev = (j > 0) ? ls->ratio[j] : 0.0;
     // t = s_j H U_j directly (the operator scaled by s_j)
     const StencilIn in = scaled(fp64_in(B, I, inst, u), sc.s);
     double acc = 0.0;

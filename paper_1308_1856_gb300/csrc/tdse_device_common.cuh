@@ -110,5 +110,46 @@ __device__ __forceinline__ bool publish_block_partial(double v, Reduction *red, 
   return s_last != 0;
 }
 
+// The scale of the FP64 Lanczos recurrence.  z = s_j H U_j - ratio_j U_{j-1} with
+// s_j the power of two at or below sigma_j (the scale is then an exponent, not
+// a product per point) and ratio_j = beta_{j-1} sigma_{j-1} / g_j; with
+// g_j = sigma_j / s_j in [1, 2):
+//   alpha_j = sigma_j g_j Re<U_j, z>,  U_{j+1} = z - alpha_j s_j U_j,
+//   beta_j = g_j ||U_{j+1}||.
+// sigma_j = 0 (a vanished vector) keeps s_j = 1, g_j = 0.
+struct StepScale {
+  double s, g;
+  int k;       // s = 2^k
+};
+__device__ __forceinline__ StepScale step_scale(double sigma) {
+  StepScale r;
+  const int f = (__double2hiint(sigma) >> 20) & 0x7ff;
+  const bool usable = f > 0 && f < 0x7ff;
+  r.k = usable ? f - 1023 : 0;
+  r.s = usable ? __hiloint2double(f << 20, 0) : 1.0;
+  r.g = usable ? __hiloint2double((__double2hiint(sigma) & 0xfffff) | 0x3ff00000, __double2loint(sigma)) : sigma;
+  return r;
+}
+
+// alpha_j and U_{j+1}'s coefficient from the sum of U_j^* z.
+__device__ __forceinline__ void store_alpha(LanczosScalars *ls, int j, double sum) {
+  const double sig = ls->sigma[j];
+  const StepScale sc = step_scale(sig);
+  const double al = (sum * sig) * sc.g;
+  ls->alpha[j] = al;
+  ls->acoef[j] = -al * sc.s;
+}
+// beta_j and the next vector's scalars from ||U_{j+1}||^2.
+__device__ __forceinline__ void store_beta(LanczosScalars *ls, int j, double sumsq) {
+  const double nrm = sqrt(sumsq);
+  const double beta = step_scale(ls->sigma[j]).g * nrm;
+  ls->beta[j] = beta;
+  const double sn = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+  ls->sigma[j + 1] = sn;
+  // 1 / g_{j+1} = s_{j+1} ||U_{j+1}||.  Formed here, in one thread: as a division in every
+  // warp of the next kernel it took 2 us of that kernel
+  ls->ratio[j + 1] = (sn > 0.0) ? (ls->sigma[j] * beta) * (nrm * step_scale(sn).s) : 0.0;
+}
+
 }  // namespace common
 }  // namespace tdse_dev

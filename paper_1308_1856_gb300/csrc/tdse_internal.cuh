@@ -41,10 +41,10 @@ constexpr int kMaxPartials = 16384;     // block partial slots of one grid reduc
 // Scalars of one Lanczos step, resident in device memory.
 struct LanczosScalars {
   double alpha[kMaxKrylov];      // alpha_j = <q_j, H q_j>
-  double beta[kMaxKrylov];       // beta_j = ||w_j|| (beta[j] links q_j and q_{j+1})
+  double beta[kMaxKrylov];       // beta_j = g_j ||U_{j+1}|| (beta[j] links q_j and q_{j+1}; FP64: step_scale's g_j)
   double sigma[kMaxKrylov + 1];  // sigma_j = 1 / ||U_j||  (U_0 = psi, U_j unnormalised)
-  double ratio[kMaxKrylov + 1];  // ratio_j = sigma_{j-1} / sigma_j  (= beta_{j-1} sigma_{j-1})
-  double acoef[kMaxKrylov];      // -alpha_j sigma_j (coefficient of U_j in U_{j+1})
+  double ratio[kMaxKrylov + 1];  // coefficient of -U_{j-1} in z: beta_{j-1} sigma_{j-1}, in FP64 over step_scale's g_j
+  double acoef[kMaxKrylov];      // coefficient of U_j in U_{j+1}: -alpha_j s_j in FP64 (step_scale), -alpha_j sigma_j mixed
   double psinorm;                // ||psi|| at the start of the step
   double psinorm0;               // batch: ||psi|| before the last combine (imaginary-time energy)
   double2 coef[kMaxKrylov];      // psi_new = sum_j coef_j U_j
@@ -76,18 +76,26 @@ struct OperatorView {
   const double *diag, *rj, *kappa, *mask;
   const double *rinv = nullptr;   // 1 / r_j (velocity gauge)
   int mask_start;                 // first j index (0-based) with mask != 1; N if none
+  // the fixed-point walker's tables (tdse_walk_fixed.cuh); fx_ok 0: not held
+  const long long *diagq = nullptr;
+  long long c1q = 0, c2q = 0;
+  int fx_ec = 0, fx_ok = 0;
+  bool plain = false;             // length gauge: Taylor and RK4 stages in FP64 (see launch_taylor_stage)
 };
+
+// diagq = diag in the fixed-point walker's encoding (fx_encode_diag).
+cudaError_t launch_fx_diag(const double *diag, size_t G, int ec, long long *diagq, const Geometry &g, cudaStream_t s);
 
 cudaError_t launch_apply_h(const Geometry &g, const OperatorView &op, double E,
                            const double2 *x, double2 *y, cudaStream_t s);
+// op.plain: all in FP64, bitwise the cluster path's arithmetic.
 // imag: the stage of exp(-H dt) (imaginary time: -H instead of -i H, no mask).
 cudaError_t launch_taylor_stage(const Geometry &g, const OperatorView &op, double E, double s,
                                 const double2 *v_in, const double2 *psi, double2 *v_out,
                                 bool final_stage, cudaStream_t st, bool imag = false);
 cudaError_t launch_rk_stage(const Geometry &g, const OperatorView &op, double E, int stage,
-                            double dt, const double2 *gin, const double2 *psi,
-                            const double2 *acc_in, double2 *acc_out, double2 *g_next,
-                            double2 *psi_out, cudaStream_t st, bool imag = false);
+                            double dt, const double2 *gin, const double2 *psi, double2 *acc,
+                            double2 *g_next, double2 *psi_out, cudaStream_t st, bool imag = false);
 // One stage of an explicit Runge-Kutta method with up to kRkMaxStages stages
 // (appendix "Runge-Kutta"): stage i computes k_i = -i H(E) g_i at every point
 // (g_i = gin; g_0 is psi itself) and then, pointwise,

@@ -7,27 +7,32 @@
 // with D_{l,j} = c0 + l(l+1)/(2 r_j^2) + V(r_j) read from a table, H real and
 // symmetric, so the real and imaginary parts go through the same real operator.
 //
-// Work decomposition: the grid is persistent (a few blocks per SM) and the
-// (L+1) x N points are cut into segments of 32 consecutive radial points of
-// one partial wave, ordered radial-group-major.  Warp w takes a contiguous,
-// balanced range of the T segments (warp_range), so every warp gets the same
-// amount of work to within one segment and the assignment (hence every
-// reduction order) is fixed.  Inside a range a lane owns one radial index j
-// and walks l upwards keeping x_{l-1,j}, x_{l,j}, x_{l+1,j} in registers, so
-// each l-neighbour is loaded once and the coupling coefficient
-// kappa_{l+1} E r_j is shared by rows l and l+1.  The radial neighbours come
-// from L1/L2 (neighbouring lanes load the same lines).
+// Length gauge: the fixed-point walker (tdse_walk_fixed.cuh).  An FP64
+// instruction of a warp takes its SM sub-partition 64 cycles, so the 15 of a
+// point's H x bounded these kernels; in fixed point the operator runs on the
+// integer pipe and only the epilogue is FP64.  The (L+1) rows of the strips of
+// kFxCols columns form one strip-major sequence of row segments; warp w of the
+// persistent grid takes a contiguous, balanced range of it (for_my_strips).  The
+// warps' numbers run across the blocks, so that the warps with one segment more
+// are spread evenly over the SMs.  What bounds it now is the integer pipe's issue
+// with the FP64 epilogue beside it.  512,000 points (8000 x 64): H x 23.5 to
+// 14.4 us a call, a Taylor stage 19.5 to 13.6, an RK4 stage 22.2 to 16.8, a
+// Lanczos-12 step 607 to 497.
 //
-// On GB300 an FP64 instruction issues at 2 lanes/clock/SM, so these kernels
-// are FP64-issue bound: the arithmetic is written with explicit __dmul_rn /
-// __dadd_rn / __fma_rn so that each grid point costs a known number of FP64
-// instructions (5-point Taylor stage: 17).
+// Velocity gauge, and Taylor and RK4 stages of grids that fit the one-launch
+// cluster path, whose states are bitwise these: all in FP64, in
+// segments of 32 radial points of one partial wave, ordered
+// radial-group-major, a contiguous balanced range for each warp (warp_range).
+// A lane owns one radial index j and walks l upwards keeping x_{l-1,j},
+// x_{l,j}, x_{l+1,j} in registers; the arithmetic is written with explicit
+// __dmul_rn / __dadd_rn / __fma_rn.
 #include <cuda_runtime.h>
 
 #include <type_traits>
 
 #include "tdse_device_common.cuh"
 #include "tdse_stencil.cuh"
+#include "tdse_walk_fixed.cuh"
 #include "tdse_internal.cuh"
 
 namespace tdse_dev {
@@ -56,11 +61,39 @@ __device__ __forceinline__ void for_my_segments(const StencilIn &in, F &&f) {
   }
 }
 
+// How a stencil kernel walks the grid: in fixed point (length gauge), or in FP64.
+enum Walk { kFixed, kPlain, kPlainVG };
+template <int WALK>
+using OpIn = std::conditional_t<WALK == kFixed, FxIn, StencilIn>;
+// Blocks an SM: one of 16 warps with 128 registers a thread and its rings in
+// fixed point, two of 64 registers in FP64.
+template <int WALK>
+constexpr int kOpBlocksPerSM = WALK == kFixed ? 1 : kStencilBlocksPerSM;
+
+// Call f(idx, i, H x, x, extra values) at every point this thread owns.
+template <int ST, int WALK, int EX, bool SCALED = false, typename F>
+__device__ __forceinline__ void for_my_points(const OpIn<WALK> &in, const FxExtra<EX> &ex, F &&f) {
+  if constexpr (WALK != kFixed) {
+    for_my_segments<ST, SCALED, WALK == kPlainVG>(in, [&](int i, size_t idx, double2 t, double2 u) {
+      double2 e[EX > 0 ? EX : 1];
+#pragma unroll
+      for (int q = 0; q < EX; ++q) e[q] = ex.p[q][idx];
+      f((int)idx, i, t, u, e);
+    });
+  } else {
+    extern __shared__ __align__(16) unsigned char fx_smem[];
+    unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX>();
+    for_my_strips(in, [&](int j0, int l0, int l1) { walk_rows_fixed<ST, EX>(in, ex, ring, j0, l0, l1, f); });
+  }
+}
+
 // ---------------------------------------------------------------------------
 // y = H(E) x
-template <int ST, bool VG>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) apply_h_kernel(StencilIn in, double2 *__restrict__ y) {
-  for_my_segments<ST, false, VG>(in, [&](int, size_t idx, double2 t, double2) { y[idx] = t; });
+template <int ST, int WALK>
+__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>) apply_h_kernel(OpIn<WALK> in, double2 *__restrict__ y) {
+  for_my_points<ST, WALK, 0>(in, FxExtra<0>{}, [&](int idx, int, double2 t, double2, const double2 (&)[1]) {
+    y[idx] = t;
+  });
 }
 
 // Horner stage of the Taylor polynomial (Eq. (Taylor)):
@@ -69,22 +102,22 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) apply_h_kernel(S
 // The last stage (k = 1, FIN) writes psi itself and applies the absorber
 // mask; the other stages carry no mask code at all (a predicated-off FP64
 // instruction still takes its issue slot on the FP64 pipe).
-template <int ST, bool IMAG, bool VG, bool FIN>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
-    taylor_stage_kernel(StencilIn in, double s, const double2 *__restrict__ psi,
-                        double2 *__restrict__ out, const double *__restrict__ mask,
+template <int ST, bool IMAG, int WALK, bool FIN>
+__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
+    taylor_stage_kernel(OpIn<WALK> in, double s, const double2 *psi, double2 *out, const double *__restrict__ mask,
                         int mask_start) {
   pdl_wait();
-  for_my_segments<ST, false, VG>(in, [&](int i, size_t idx, double2 t, double2) {
+  FxExtra<1> ex;
+  ex.p[0] = psi;
+  for_my_points<ST, WALK, 1>(in, ex, [&](int idx, int i, double2 t, double2, const double2 (&e)[1]) {
     const bool masked = FIN && i >= mask_start;
-    const double2 p = psi[idx];
     double2 o;
     if (IMAG) {
-      o.x = __fma_rn(-s, t.x, p.x);
-      o.y = __fma_rn(-s, t.y, p.y);
+      o.x = __fma_rn(-s, t.x, e[0].x);
+      o.y = __fma_rn(-s, t.y, e[0].y);
     } else {
-      o.x = __fma_rn(s, t.y, p.x);     // (-i s)(tx + i ty) = s ty - i s tx
-      o.y = __fma_rn(-s, t.x, p.y);
+      o.x = __fma_rn(s, t.y, e[0].x);     // (-i s)(tx + i ty) = s ty - i s tx
+      o.y = __fma_rn(-s, t.x, e[0].y);
     }
     if (masked) { const double mv = mask[i]; o.x = __dmul_rn(mv, o.x); o.y = __dmul_rn(mv, o.y); }
     out[idx] = o;
@@ -92,33 +125,35 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
   pdl_trigger();
 }
 
-// Stage `stage` (1..4) of classic RK4 (Eq. (RKDeriv)) with k = -i H(t_n + c dt) g:
-//   stages 1-3: g_next = psi + (dt a) k,  acc_out = acc_in + (dt b) k  (acc_in = psi at stage 1)
-//   stage 4:    psi    = acc_in + (dt b) k, then the absorber mask.
+// A stage of classic RK4 (Eq. (RKDeriv)) with k = -i H(t_n + c dt) g:
+//   PART 0, stage 1 (g = psi):  g_next = psi + ca k,  acc = psi + cb k
+//   PART 1, stages 2 and 3:     g_next = psi + ca k,  acc = acc + cb k
+//   PART 2, stage 4:            psi    = acc + cb k, then the absorber mask.
 // IMAG: k = -H g (imaginary time) instead of -i H g.
-template <int ST, bool IMAG, bool VG>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
-    rk_stage_kernel(StencilIn in, int stage, double ca, double cb,
-                    const double2 *__restrict__ psi, const double2 *__restrict__ acc_in,
-                    double2 *__restrict__ acc_out, double2 *__restrict__ g_next,
-                    double2 *__restrict__ psi_out, const double *__restrict__ mask,
-                    int mask_start) {
-  const int mstart = (stage == 4) ? mask_start : in.N;
+template <int ST, bool IMAG, int WALK, int PART>
+__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
+    rk_stage_kernel(OpIn<WALK> in, double ca, double cb, const double2 *psi, double2 *acc, double2 *g_next,
+                    double2 *psi_out, const double *__restrict__ mask, int mask_start) {
   pdl_wait();
-  for_my_segments<ST, false, VG>(in, [&](int i, size_t idx, double2 t, double2) {
-    const double2 a = acc_in[idx];
+  constexpr int EX = PART == 0 ? 0 : (PART == 1 ? 2 : 1);
+  FxExtra<EX> ex;
+  if (PART > 0) ex.p[0] = acc;
+  if constexpr (PART == 1) ex.p[1] = psi;
+  for_my_points<ST, WALK, EX>(in, ex, [&](int idx, int i, double2 t, double2 u, const double2 (&e)[EX > 0 ? EX : 1]) {
     // c k with k = -i t:  (c t.y, -c t.x);  with k = -t:  (-c t.x, -c t.y)
     auto add = [&](double c, double2 base) {
       return IMAG ? make_double2(__fma_rn(-c, t.x, base.x), __fma_rn(-c, t.y, base.y))
                   : make_double2(__fma_rn(c, t.y, base.x), __fma_rn(-c, t.x, base.y));
     };
-    if (stage < 4) {
-      const double2 p = psi[idx];
-      g_next[idx] = add(ca, p);
-      acc_out[idx] = add(cb, a);
+    if constexpr (PART == 0) {
+      g_next[idx] = add(ca, u);
+      acc[idx] = add(cb, u);
+    } else if constexpr (PART == 1) {
+      g_next[idx] = add(ca, e[1]);
+      acc[idx] = add(cb, e[0]);
     } else {
-      double2 o = add(cb, a);
-      if (i >= mstart) { const double mv = mask[i]; o.x = __dmul_rn(mv, o.x); o.y = __dmul_rn(mv, o.y); }
+      double2 o = add(cb, e[0]);
+      if (i >= mask_start) { const double mv = mask[i]; o.x = __dmul_rn(mv, o.x); o.y = __dmul_rn(mv, o.y); }
       psi_out[idx] = o;
     }
   });
@@ -137,23 +172,30 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
 //           coefficients, so only Delta is formed.
 // The slopes of the earlier stages are read pointwise and combined in stage
 // order, the new slope k_i = -i H g_i last, so the sums round in the same
-// order as the oracle's.
-template <int ST, bool VG, int NK, int MODE>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
-    rk_general_stage_kernel(StencilIn in, RkStageArgs a, const double2 *__restrict__ psi,
-                            const double *__restrict__ mask, int mask_start, Reduction *red,
-                            double S) {
+// order as the oracle's.  psi (or, in MODE 2, k_0) and the first slope come
+// through the walker's ring, which has room for two vectors; further slopes are
+// loaded where they are used.
+template <int ST, int WALK, int NK, int MODE>
+__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
+    rk_general_stage_kernel(OpIn<WALK> in, RkStageArgs a, const double2 *psi, const double *__restrict__ mask,
+                            int mask_start, Reduction *red, double S) {
   constexpr bool LAST = MODE != 0;
   constexpr bool FSAL = MODE == 2;
+  constexpr int VECS = FSAL ? NK - 1 : NK;          // psi unless FSAL, then the earlier slopes
+  constexpr int EX = VECS < 2 ? VECS : 2;
+  constexpr int KOFF = FSAL ? 0 : 1;                // slope j is vector j + KOFF
   __shared__ double sh[kBlockJ / 32 + 1];
   double acc = 0.0;
   pdl_wait();
-  for_my_segments<ST, false, VG>(in, [&](int r, size_t idx, double2 t, double2 u) {
+  FxExtra<EX> ex;
+#pragma unroll
+  for (int q = 0; q < EX; ++q) ex.p[q] = (q < KOFF) ? psi : a.k[q - KOFF];
+  for_my_points<ST, WALK, EX>(in, ex, [&](int idx, int r, double2 t, double2 u, const double2 (&e)[EX > 0 ? EX : 1]) {
     const double2 ki = make_double2(t.y, -t.x);   // -i (tx + i ty)
     double2 kj[NK > 1 ? NK - 1 : 1];
 #pragma unroll
-    for (int j = 0; j < NK - 1; ++j) kj[j] = a.k[j][idx];
-    double2 o = FSAL ? u : psi[idx];
+    for (int j = 0; j < NK - 1; ++j) kj[j] = (j + KOFF < EX) ? e[j + KOFF] : a.k[j][idx];
+    double2 o = FSAL ? u : e[0];
     double2 d = make_double2(0.0, 0.0);
 #pragma unroll
     for (int j = 0; j < NK - 1; ++j) {
@@ -193,27 +235,27 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
 }
 
 // Lanczos iteration j, first half (Appendix "Lanczos methods"):
-//   z = H q_j - beta_{j-1} q_{j-1},   q_j = sigma_j U_j,
-//   beta_{j-1} q_{j-1} = (sigma_{j-1} / sigma_j) U_{j-1},
-//   alpha_j = Re <q_j, z> = sigma_j Re <U_j, z>  (grid reduction; last block stores it).
-template <int ST, bool VG>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
-    lanczos_a_kernel(StencilIn in, int j, const double2 *__restrict__ uprev,
-                     double2 *__restrict__ z, Reduction *red, LanczosScalars *ls) {
+//   z = s_j H U_j - ratio_j U_{j-1},  alpha_j from sum Re(U_j^* z)
+// with s_j the power of two at or below sigma_j (step_scale; the grid
+// reduction's last block stores the scalars).  EX = 1 where U_{j-1} exists.
+template <int ST, int WALK, int EX>
+__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
+    lanczos_a_kernel(OpIn<WALK> in, int j, const double2 *__restrict__ uprev, double2 *__restrict__ z, Reduction *red,
+                     LanczosScalars *ls) {
   __shared__ double sh[kBlockJ / 32 + 1];
   pdl_wait();
-  const double sig = ls->sigma[j];
-  const double cprev = (j > 0) ? ls->ratio[j] : 0.0;
+  const StepScale sc = step_scale(ls->sigma[j]);
+  const double cprev = EX > 0 ? ls->ratio[j] : 0.0;
   double acc = 0.0;
-  // t = sigma_j H U_j directly (the operator scaled by sigma_j)
-  for_my_segments<ST, true, VG>(scaled(in, sig), [&](int, size_t idx, double2 t, double2 u) {
-    double2 o;
-    if (j > 0) {
-      const double2 up = uprev[idx];
-      o.x = __fma_rn(-cprev, up.x, t.x);
-      o.y = __fma_rn(-cprev, up.y, t.y);
-    } else {
-      o = t;
+  FxExtra<EX> ex;
+  if (EX > 0) ex.p[0] = uprev;
+  if constexpr (WALK == kFixed) in.k = sc.k;
+  else in = scaled(in, sc.s);
+  for_my_points<ST, WALK, EX, true>(in, ex, [&](int idx, int, double2 t, double2 u, const double2 (&e)[1]) {
+    double2 o = t;
+    if (EX > 0) {
+      o.x = __fma_rn(-cprev, e[0].x, t.x);
+      o.y = __fma_rn(-cprev, e[0].y, t.y);
     }
     z[idx] = o;
     acc = __fma_rn(u.x, o.x, acc);
@@ -222,10 +264,7 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
   pdl_trigger();
   if (publish_block_partial(acc, red, sh)) {
     const double s = reduce_partials(red, gridDim.x, sh);
-    if (threadIdx.x == 0) {
-      ls->alpha[j] = s * sig;
-      ls->acoef[j] = -(s * sig) * sig;
-    }
+    if (threadIdx.x == 0) store_alpha(ls, j, s);
   }
 }
 
@@ -247,7 +286,7 @@ __device__ __forceinline__ void for_my_groups(size_t G, F &&f) {
 // used, so their memory latencies overlap.
 constexpr int kUnroll = 4;
 
-// Lanczos iteration j, second half: U_{j+1} = z - alpha_j sigma_j U_j; beta_j = ||U_{j+1}||.
+// Lanczos iteration j, second half: U_{j+1} = z - alpha_j s_j U_j and its norm (beta_j).
 __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     lanczos_b_kernel(size_t G, int j, const double2 *__restrict__ z, const double2 *__restrict__ u,
                      double2 *__restrict__ unext, Reduction *red, LanczosScalars *ls) {
@@ -281,13 +320,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
   pdl_trigger();
   if (publish_block_partial(acc0 + acc1, red, sh)) {
     const double s = reduce_partials(red, gridDim.x, sh);
-    if (threadIdx.x == 0) {
-      const double beta = sqrt(s);
-      ls->beta[j] = beta;
-      const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
-      ls->sigma[j + 1] = sn;
-      ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
-    }
+    if (threadIdx.x == 0) store_beta(ls, j, s);
   }
 }
 
@@ -396,6 +429,13 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
   }
 }
 
+// The diagonal in the fixed-point walker's encoding.
+__global__ void __launch_bounds__(256) fx_diag_kernel(const double *__restrict__ diag, size_t G, int ec,
+                                                      long long *__restrict__ diagq) {
+  for (size_t q = (size_t)blockIdx.x * 256 + threadIdx.x; q < G; q += (size_t)gridDim.x * 256)
+    diagq[q] = fx_encode_diag((uint64_t)__double_as_longlong(diag[q]), ec);
+}
+
 // Observables (Sec. 4): per block of row l, partial sums of
 //   q0: sum |f|^2, q1: sum_{r_j <= r_b} |f|^2, q2: sum r_j Re(conj(f_l) f_{l+1}),
 //   q3, q4: sum conj(ref_j) f_{0,j} (row 0 only).
@@ -478,10 +518,23 @@ __global__ void __launch_bounds__(kObsThreads)
   }
 }
 
-StencilIn make_in(const Geometry &g, const OperatorView &op, double E, const double2 *x) {
-  StencilIn in;
+template <int WALK>
+OpIn<WALK> make_in(const Geometry &g, const OperatorView &op, double E, const double2 *x) {
+  OpIn<WALK> in;
+  if constexpr (WALK != kFixed) {
+    in.diag = op.diag;
+    in.dscale = 1.0;
+    in.rinv = op.rinv;
+    in.d1c = (g.stencil == 5) ? 1.0 / (12.0 * g.dr) : 1.0 / (2.0 * g.dr);
+  } else {
+    in.diagq = op.fx_ok ? op.diagq : reinterpret_cast<const long long *>(op.diag);
+    in.c1q = op.c1q;
+    in.c2q = op.c2q;
+    in.ec = op.fx_ec;
+    in.ok = op.fx_ok;
+    in.k = 0;
+  }
   in.x = x;
-  in.diag = op.diag;
   in.rj = op.rj;
   in.kappa = op.kappa;
   in.N = g.N;
@@ -489,9 +542,6 @@ StencilIn make_in(const Geometry &g, const OperatorView &op, double E, const dou
   in.c1 = g.c1;
   in.c2 = g.c2;
   in.E = E;
-  in.dscale = 1.0;
-  in.rinv = op.rinv;
-  in.d1c = (g.stencil == 5) ? 1.0 / (12.0 * g.dr) : 1.0 / (2.0 * g.dr);
   return in;
 }
 
@@ -500,107 +550,158 @@ using IC = std::integral_constant<int, V>;
 template <bool V>
 using BC = std::integral_constant<bool, V>;
 
-// f(stencil, velocity gauge) with both as compile-time constants.
-template <typename F>
-void dispatch(const Geometry &g, bool vg, F &&f) {
-  if (g.stencil == 5) {
-    if (vg) f(IC<5>{}, BC<true>{});
-    else f(IC<5>{}, BC<false>{});
-  } else {
-    if (vg) f(IC<3>{}, BC<true>{});
-    else f(IC<3>{}, BC<false>{});
-  }
+// f(stencil, walk) with both as compile-time constants.  PLAIN: whether the
+// caller has a use for the length gauge's FP64 walk, taken where `plain` says so.
+template <bool PLAIN, typename F>
+void dispatch(const Geometry &g, bool vg, bool plain, F &&f) {
+  auto go = [&](auto st) {
+    if (vg) return f(st, IC<kPlainVG>{});
+    if constexpr (PLAIN)
+      if (plain) return f(st, IC<kPlain>{});
+    f(st, IC<kFixed>{});
+  };
+  if (g.stencil == 5) go(IC<5>{});
+  else go(IC<3>{});
 }
 
 // Persistent grids: a few blocks per SM (all resident at once).
-inline unsigned stencil_blocks(const Geometry &g) { return (unsigned)(g.sms * kStencilBlocksPerSM); }
+template <int WALK>
+inline unsigned stencil_blocks(const Geometry &g) { return (unsigned)(g.sms * kOpBlocksPerSM<WALK>); }
 inline unsigned elem_blocks(const Geometry &g) { return (unsigned)(g.sms * kElemBlocksPerSM); }
+
+
+// The parts a fixed-point launch's blocks are cut to: half the warps where the
+// strips' row segments need no more.  Two blocks then fit on an SM, so that the
+// next kernel of the chain is resident and waiting when this one ends.  The
+// warps' numbers, and so every sum, stay the same.  (Lanczos-12, 17,600
+// points: 312 to 267 us a step.)
+inline unsigned block_parts(const Geometry &g) {
+  const size_t per_sm = ((size_t)((g.N + kFxCols - 1) / kFxCols) * (g.L + 1) + g.sms - 1) / g.sms;
+  return per_sm <= kBlockJ / 64 && (unsigned)g.sms <= kBlockJ / 2 ? 2u : 1u;
+}
+
+// A stencil kernel's launch: its rings are dynamic shared memory, raised above
+// the 48 KB default once per instantiation (kern is a compile-time constant).
+template <auto KERN, int WALK, int EX, bool PDL = true, typename... Args>
+cudaError_t launch_op(const Geometry &g, cudaStream_t st, Args... args) {
+  constexpr size_t bytes = WALK == kFixed ? (kBlockJ / 32) * (size_t)fx_warp_bytes<EX>() : 0;
+  const unsigned parts = WALK == kFixed ? block_parts(g) : 1u;
+  if (WALK == kFixed) {
+    static const cudaError_t ready = [] {
+      // one split of L1 and shared memory for all of them: a kernel that wants
+      // another than its predecessor's waits for the SM to drain (Dormand-Prince
+      // on 50,000 points: 279 us for four steps, 233 with one split)
+      const cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                                 cudaSharedmemCarveoutMaxShared);
+      return e != cudaSuccess ? e : cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    }();
+    if (ready != cudaSuccess) return ready;
+  }
+  cudaError_t e = cudaSuccess;
+  if (PDL) e = launch_pdl(KERN, stencil_blocks<WALK>(g), kBlockJ / parts, bytes / parts, st, args...);
+  else KERN<<<stencil_blocks<WALK>(g), kBlockJ / parts, bytes / parts, st>>>(args...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
 
 }  // namespace
 
 // ---------------------------------------------------------------------------
+cudaError_t launch_fx_diag(const double *diag, size_t G, int ec, long long *diagq, const Geometry &g, cudaStream_t s) {
+  fx_diag_kernel<<<(unsigned)(g.sms * 4), 256, 0, s>>>(diag, G, ec, diagq);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_apply_h(const Geometry &g, const OperatorView &op, double E,
                            const double2 *x, double2 *y, cudaStream_t s) {
-  const StencilIn in = make_in(g, op, E, x);
-  const unsigned grid = stencil_blocks(g);
-  dispatch(g, g.gauge == 1, [&](auto st, auto vg) {
-    apply_h_kernel<decltype(st)::value, decltype(vg)::value><<<grid, kBlockJ, 0, s>>>(in, y);
+  cudaError_t e = cudaSuccess;
+  dispatch<false>(g, g.gauge == 1, false, [&](auto st, auto walk) {
+    constexpr int ST = decltype(st)::value;
+    constexpr int WALK = decltype(walk)::value;
+    e = launch_op<apply_h_kernel<ST, WALK>, WALK, 0, false>(g, s, make_in<WALK>(g, op, E, x), y);
   });
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_taylor_stage(const Geometry &g, const OperatorView &op, double E, double s,
                                 const double2 *v_in, const double2 *psi, double2 *v_out,
                                 bool final_stage, cudaStream_t st, bool imag) {
-  const StencilIn in = make_in(g, op, E, v_in);
-  const unsigned grid = stencil_blocks(g);
   const int mstart = op.mask_start;
   cudaError_t e = cudaSuccess;
-  dispatch(g, !imag && g.gauge == 1, [&](auto stc, auto vg) {
+  dispatch<true>(g, !imag && g.gauge == 1, !imag && op.plain, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
-    constexpr bool VG = decltype(vg)::value;
-    if (imag)   // imaginary time: no absorber, no field
-      e = launch_pdl(taylor_stage_kernel<ST, true, false, false>, grid, kBlockJ, 0, st, in, s, psi, v_out, op.mask, mstart);
-    else if (final_stage)
-      e = launch_pdl(taylor_stage_kernel<ST, false, VG, true>, grid, kBlockJ, 0, st, in, s, psi, v_out, op.mask, mstart);
+    constexpr int WALK = decltype(walk)::value;
+    const auto in = make_in<WALK>(g, op, E, v_in);
+    if constexpr (WALK == kFixed)   // imaginary time: no absorber, no field
+      if (imag) {
+        e = launch_op<taylor_stage_kernel<ST, true, kFixed, false>, kFixed, 1>(g, st, in, s, psi, v_out, op.mask, mstart);
+        return;
+      }
+    if (final_stage)
+      e = launch_op<taylor_stage_kernel<ST, false, WALK, true>, WALK, 1>(g, st, in, s, psi, v_out, op.mask, mstart);
     else
-      e = launch_pdl(taylor_stage_kernel<ST, false, VG, false>, grid, kBlockJ, 0, st, in, s, psi, v_out, op.mask, mstart);
+      e = launch_op<taylor_stage_kernel<ST, false, WALK, false>, WALK, 1>(g, st, in, s, psi, v_out, op.mask, mstart);
   });
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_rk_stage(const Geometry &g, const OperatorView &op, double E, int stage,
-                            double dt, const double2 *gin, const double2 *psi,
-                            const double2 *acc_in, double2 *acc_out, double2 *g_next,
-                            double2 *psi_out, cudaStream_t st, bool imag) {
+                            double dt, const double2 *gin, const double2 *psi, double2 *acc,
+                            double2 *g_next, double2 *psi_out, cudaStream_t st, bool imag) {
   // classic tableau: a_{s+1,s} = (1/2, 1/2, 1), b = (1, 2, 2, 1) / 6
   static const double a_next[4] = {0.5, 0.5, 1.0, 0.0};
   static const double b[4] = {1.0 / 6.0, 1.0 / 3.0, 1.0 / 3.0, 1.0 / 6.0};
-  const StencilIn in = make_in(g, op, E, gin);
-  const unsigned grid = stencil_blocks(g);
   const double ca = dt * a_next[stage - 1], cb = dt * b[stage - 1];
   const int mstart = imag ? g.N : op.mask_start;
   cudaError_t e = cudaSuccess;
-  dispatch(g, !imag && g.gauge == 1, [&](auto stc, auto vg) {
+  dispatch<true>(g, !imag && g.gauge == 1, !imag && op.plain, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
-    constexpr bool VG = decltype(vg)::value;
-    if (imag)
-      e = launch_pdl(rk_stage_kernel<ST, true, false>, grid, kBlockJ, 0, st, in, stage, ca, cb, psi, acc_in, acc_out,
-                     g_next, psi_out, op.mask, mstart);
-    else
-      e = launch_pdl(rk_stage_kernel<ST, false, VG>, grid, kBlockJ, 0, st, in, stage, ca, cb, psi, acc_in, acc_out,
-                     g_next, psi_out, op.mask, mstart);
+    constexpr int WALK = decltype(walk)::value;
+    const auto in = make_in<WALK>(g, op, E, gin);
+    auto go = [&](auto part, auto im) {
+      constexpr int PART = decltype(part)::value;
+      constexpr bool IMAG = decltype(im)::value;
+      constexpr int EX = PART == 0 ? 0 : (PART == 1 ? 2 : 1);
+      e = launch_op<rk_stage_kernel<ST, IMAG, WALK, PART>, WALK, EX>(g, st, in, ca, cb, psi, acc, g_next, psi_out, op.mask,
+                                                                 mstart);
+    };
+    auto parts = [&](auto im) {
+      if (stage == 1) go(IC<0>{}, im);
+      else if (stage < 4) go(IC<1>{}, im);
+      else go(IC<2>{}, im);
+    };
+    if constexpr (WALK == kFixed)
+      if (imag) return parts(BC<true>{});
+    parts(BC<false>{});
   });
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_rk_general_stage(const Geometry &g, const OperatorView &op, double E,
                                     const double2 *gin, const double2 *psi, const RkStageArgs &a,
                                     Reduction *red, cudaStream_t st) {
   if (a.stage < 0 || a.stage >= kRkMaxStages) return cudaErrorInvalidValue;
-  const StencilIn in = make_in(g, op, E, gin);
-  const unsigned grid = stencil_blocks(g);
   const double S = (double)g.N * (double)(g.L + 1);
   const int mode = a.last ? (a.fsal ? 2 : 1) : 0;
   cudaError_t e = cudaSuccess;
   if (!a.last && a.stage == kRkMaxStages - 1) return cudaErrorInvalidValue;   // no stage after the last
   if (a.fsal && (!a.last || a.stage == 0)) return cudaErrorInvalidValue;
-  dispatch(g, g.gauge == 1, [&](auto stc, auto vg) {
+  dispatch<false>(g, g.gauge == 1, false, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
-    constexpr bool VG = decltype(vg)::value;
+    constexpr int WALK = decltype(walk)::value;
+    const auto in = make_in<WALK>(g, op, E, gin);
+    auto launch = [&](auto nk, auto md) {
+      constexpr int NK = decltype(nk)::value, MODE = decltype(md)::value;
+      constexpr int VECS = MODE == 2 ? NK - 1 : NK;
+      e = launch_op<rk_general_stage_kernel<ST, WALK, NK, MODE>, WALK, (VECS < 2 ? VECS : 2)>(
+          g, st, in, a, psi, op.mask, op.mask_start, red, S);
+    };
     auto go = [&](auto nk) {
       constexpr int NK = decltype(nk)::value;
-      if (mode == 1)
-        e = launch_pdl(rk_general_stage_kernel<ST, VG, NK, 1>, grid, kBlockJ, 0, st, in, a, psi, op.mask,
-                       op.mask_start, red, S);
-      else if constexpr (NK > 1)
-        if (mode == 2)
-          e = launch_pdl(rk_general_stage_kernel<ST, VG, NK, 2>, grid, kBlockJ, 0, st, in, a, psi, op.mask,
-                         op.mask_start, red, S);
+      if (mode == 1) launch(nk, IC<1>{});
+      if constexpr (NK > 1)
+        if (mode == 2) launch(nk, IC<2>{});
       if constexpr (NK < kRkMaxStages)
-        if (mode == 0)
-          e = launch_pdl(rk_general_stage_kernel<ST, VG, NK, 0>, grid, kBlockJ, 0, st, in, a, psi, op.mask,
-                         op.mask_start, red, S);
+        if (mode == 0) launch(nk, IC<0>{});
     };
     switch (a.stage + 1) {
       case 1: go(IC<1>{}); break;
@@ -612,7 +713,7 @@ cudaError_t launch_rk_general_stage(const Geometry &g, const OperatorView &op, d
       default: go(IC<7>{}); break;
     }
   });
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_imag_begin(const Reduction *red, double dr, double *imag_dev, cudaStream_t st) {
@@ -637,14 +738,15 @@ cudaError_t launch_norm(const Geometry &g, const double2 *x, Reduction *red,
 cudaError_t launch_lanczos_a(const Geometry &g, const OperatorView &op, double E, int j,
                              const double2 *u, const double2 *uprev, double2 *z,
                              Reduction *red, LanczosScalars *ls, cudaStream_t st) {
-  const StencilIn in = make_in(g, op, E, u);
-  const unsigned grid = stencil_blocks(g);
   cudaError_t e = cudaSuccess;
-  dispatch(g, g.gauge == 1, [&](auto stc, auto vg) {
-    e = launch_pdl(lanczos_a_kernel<decltype(stc)::value, decltype(vg)::value>, grid, kBlockJ, 0, st, in, j, uprev,
-                   z, red, ls);
+  dispatch<false>(g, g.gauge == 1, false, [&](auto stc, auto walk) {
+    constexpr int ST = decltype(stc)::value;
+    constexpr int WALK = decltype(walk)::value;
+    const auto in = make_in<WALK>(g, op, E, u);
+    if (j > 0) e = launch_op<lanczos_a_kernel<ST, WALK, 1>, WALK, 1>(g, st, in, j, uprev, z, red, ls);
+    else e = launch_op<lanczos_a_kernel<ST, WALK, 0>, WALK, 0>(g, st, in, j, uprev, z, red, ls);
   });
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_lanczos_b(const Geometry &g, int j, const double2 *z, const double2 *u,

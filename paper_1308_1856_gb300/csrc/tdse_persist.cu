@@ -9,9 +9,10 @@
 // behind a launch, a ramp and a grid reduction's tail.  Here the grid stays
 // resident for the whole call and the phases are separated by a grid-wide
 // barrier:
-//   - the grid is the multi-launch path's (2 blocks of 512 threads per SM),
-//     and every phase walks exactly the multi-launch kernel's work split with
-//     the same arithmetic;
+//   - the grid is the multi-launch stencil kernel's (one block of 512 threads
+//     per SM), and every phase walks exactly the multi-launch kernel's work
+//     split with the same arithmetic; in the elementwise phases, whose kernels
+//     have kElemBlocksPerSM blocks an SM, a block stands for as many of them in turn;
 //   - a reduction stores the block's partial, crosses the barrier, and then
 //     EVERY block adds all partials in the multi-launch last block's fixed
 //     order, so every block holds the same scalars and the results equal the
@@ -31,6 +32,7 @@
 #include "tdse_internal.cuh"
 #include "tdse_small_expm.cuh"
 #include "tdse_stencil.cuh"
+#include "tdse_walk_fixed.cuh"
 
 namespace tdse_dev {
 namespace {
@@ -42,7 +44,7 @@ constexpr long long kGridSpins = 1LL << 21;   // polls of the barrier's generati
 constexpr int kUnrollB = 4;                   // phase B: groups loaded before use (as the B kernel)
 
 struct PersistArgs {
-  StencilIn in;              // operator; x and E are set per phase
+  FxIn in;                   // operator; x, k and E are set per phase
   double2 *psi;              // U_0, rewritten by the combine
   double2 *work;             // slot 0: z; slots 1..m-1: U_j
   size_t G;
@@ -88,41 +90,40 @@ __device__ __forceinline__ void grid_sync(unsigned *bar, unsigned nblocks, int *
   __syncthreads();
 }
 
-// The block's partial, the barrier, then every block's fixed-order sum of all
-// partials (the multi-launch last block's reduce_partials).
-__device__ __forceinline__ double grid_reduce(double v, Reduction *r, double *sh, const PersistArgs &a) {
-  const double b = block_sum(v, sh);
-  if (threadIdx.x == 0) r->partial[blockIdx.x] = b;
+// The partials of the multi-launch blocks this block stands for (v[q]: block
+// q gridDim + blockIdx of V gridDim blocks), the barrier, then every block's
+// fixed-order sum of all partials (the multi-launch last block's reduce_partials).
+template <int V>
+__device__ __forceinline__ double grid_reduce(const double (&v)[V], Reduction *r, double *sh, const PersistArgs &a) {
+#pragma unroll
+  for (int q = 0; q < V; ++q) {
+    const double b = block_sum(v[q], sh);
+    if (threadIdx.x == 0) r->partial[q * gridDim.x + blockIdx.x] = b;
+  }
   grid_sync(a.bar, gridDim.x, a.status);
-  return reduce_partials(r, gridDim.x, sh);
+  return reduce_partials(r, V * gridDim.x, sh);
 }
 
-// The stencil phase's work split (the multi-launch stencil kernels' walker),
-// with the operand read from L2.
-template <int ST, typename F>
-__device__ __forceinline__ void segments_cg(const StencilIn &in, F &&f) {
-  const int lane = threadIdx.x & 31;
-  const int Lp1 = in.L + 1;
-  const long long NJ = (in.N + 31) >> 5;
-  long long s, s_end;
-  warp_range(NJ * Lp1, s, s_end);
-  while (s < s_end) {
-    const int jg = (int)((unsigned)s / (unsigned)Lp1);
-    const int l0 = (int)(s - (long long)jg * Lp1);
-    const long long left = s_end - s;
-    const int l1 = (left < (long long)(Lp1 - l0)) ? l0 + (int)left : Lp1;
-    const int i = jg * 32 + lane;
-    if (i < in.N) walk_rows<ST, 0, true, false, true>(in, i, l0, l1, f);
-    s += l1 - l0;
-  }
+// warp_range for multi-launch block q gridDim + blockIdx of V gridDim blocks.
+template <int V>
+__device__ __forceinline__ void elem_range(int q, long long total, long long &s0, long long &s1) {
+  const unsigned nw = blockDim.x >> 5, W = V * gridDim.x * nw;
+  const unsigned w = (q * gridDim.x + blockIdx.x) * nw + (threadIdx.x >> 5);
+  const unsigned T = (unsigned)total, n = T / W, r = T - n * W;
+  s0 = (long long)w * n + (w < r ? w : r);
+  s1 = s0 + n + (w < r ? 1u : 0u);
 }
 
 template <int ST>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) lanczos_persistent_kernel(PersistArgs a) {
+__global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistArgs a) {
   __shared__ double sh[kBlockJ / 32 + 1];
   __shared__ double s_sigma[kMaxKrylov + 1], s_ratio[kMaxKrylov + 1], s_acoef[kMaxKrylov];
+  __shared__ double s_g[kMaxKrylov];   // step_scale's g_j
   __shared__ double2 s_coef[kMaxKrylov];
   __shared__ int s_k;
+  extern __shared__ __align__(16) unsigned char fx_smem[];
+  constexpr int V = kElemBlocksPerSM;
+  static_assert(kElemThreads == kBlockJ, "a block stands for whole elementwise blocks");
   const int tid = threadIdx.x, lane = tid & 31;
   const bool lead = blockIdx.x == 0;
   const size_t G = a.G;
@@ -130,37 +131,48 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) lanczos_persiste
   if (tid == 0) s_sigma[0] = __ldcg(&a.ls->sigma[0]);
   __syncthreads();
   for (long n = 0; n < a.nsteps; ++n) {
-    StencilIn in = a.in;
+    FxIn in = a.in;
     in.E = a.etab[n];
     for (int j = 0; j < a.m; ++j) {
       // ---- phase A (the lanczos_a kernel's arithmetic)
       const double sig = s_sigma[j];
+      const StepScale sc = step_scale(sig);
       const double cprev = (j > 0) ? s_ratio[j] : 0.0;
       const double2 *u = (j == 0) ? a.psi : a.work + (size_t)j * G;
-      const double2 *up = (j == 0) ? nullptr : ((j == 1) ? a.psi : a.work + (size_t)(j - 1) * G);
       double2 *z = a.work;
       in.x = u;
-      double acc = 0.0;
-      segments_cg<ST>(scaled(in, sig), [&](int, size_t idx, double2 t, double2 uu) {
-        double2 o;
-        if (j > 0) {
-          const double2 p = __ldcg(up + idx);
-          o.x = __fma_rn(-cprev, p.x, t.x);
-          o.y = __fma_rn(-cprev, p.y, t.y);
-        } else {
-          o = t;
-        }
-        z[idx] = o;
-        acc = __fma_rn(uu.x, o.x, acc);
-        acc = __fma_rn(uu.y, o.y, acc);
-      });
+      in.k = sc.k;
+      double acc[1] = {0.0};
+      auto phase_a = [&](auto has_prev) {
+        constexpr int EX = decltype(has_prev)::value;
+        unsigned char *ring = fx_smem + (tid >> 5) * fx_warp_bytes<EX>();
+        FxExtra<EX> ex;
+        if (EX > 0) ex.p[0] = (j == 1) ? a.psi : a.work + (size_t)(j - 1) * G;
+        for_my_strips(in, [&](int j0, int l0, int l1) {
+          walk_rows_fixed<ST, EX>(in, ex, ring, j0, l0, l1,
+                                  [&](int idx, int, double2 t, double2 uu, const double2 (&e)[1]) {
+            double2 o = t;
+            if (EX > 0) {
+              o.x = __fma_rn(-cprev, e[0].x, t.x);
+              o.y = __fma_rn(-cprev, e[0].y, t.y);
+            }
+            z[idx] = o;
+            acc[0] = __fma_rn(uu.x, o.x, acc[0]);
+            acc[0] = __fma_rn(uu.y, o.y, acc[0]);
+          });
+        });
+      };
+      if (j > 0) phase_a(std::integral_constant<int, 1>{});
+      else phase_a(std::integral_constant<int, 0>{});
       const double sa = grid_reduce(acc, a.rp + par, sh, a);
       par ^= 1;
       if (tid == 0) {
-        s_acoef[j] = -(sa * sig) * sig;
+        const double al = (sa * sig) * sc.g;   // store_alpha
+        s_acoef[j] = -al * sc.s;
+        s_g[j] = sc.g;
         if (lead) {
-          a.ls->alpha[j] = sa * sig;
-          a.ls->acoef[j] = -(sa * sig) * sig;
+          a.ls->alpha[j] = al;
+          a.ls->acoef[j] = -al * sc.s;
         }
       }
       __syncthreads();
@@ -168,35 +180,41 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) lanczos_persiste
       // ---- phase B (the lanczos_b kernel's arithmetic and work split)
       const double c = s_acoef[j];
       double2 *un = a.work + (size_t)(j + 1) * G;
-      double acc0 = 0.0, acc1 = 0.0;
-      long long g0, g1;
-      warp_range((long long)((G + 31) >> 5), g0, g1);
-      for (long long gb = g0; gb < g1; gb += kUnrollB) {
-        double2 zz[kUnrollB], vv[kUnrollB];
+      double accb[V];
+#pragma unroll 1
+      for (int q = 0; q < V; ++q) {
+        double acc0 = 0.0, acc1 = 0.0;
+        long long g0, g1;
+        elem_range<V>(q, (long long)((G + 31) >> 5), g0, g1);
+        for (long long gb = g0; gb < g1; gb += kUnrollB) {
+          double2 zz[kUnrollB], vv[kUnrollB];
 #pragma unroll
-        for (int r = 0; r < kUnrollB; ++r) {
-          const size_t idx = (size_t)(gb + r) * 32 + lane;
-          const bool ok = (gb + r < g1) && idx < G;
-          zz[r] = ok ? __ldcg(z + idx) : make_double2(0.0, 0.0);
-          vv[r] = ok ? __ldcg(u + idx) : make_double2(0.0, 0.0);
-        }
+          for (int r = 0; r < kUnrollB; ++r) {
+            const size_t idx = (size_t)(gb + r) * 32 + lane;
+            const bool ok = (gb + r < g1) && idx < G;
+            zz[r] = ok ? __ldcg(z + idx) : make_double2(0.0, 0.0);
+            vv[r] = ok ? __ldcg(u + idx) : make_double2(0.0, 0.0);
+          }
 #pragma unroll
-        for (int r = 0; r < kUnrollB; ++r) {
-          const size_t idx = (size_t)(gb + r) * 32 + lane;
-          if ((gb + r < g1) && idx < G) {
-            const double2 o = make_double2(__fma_rn(c, vv[r].x, zz[r].x), __fma_rn(c, vv[r].y, zz[r].y));
-            un[idx] = o;
-            acc0 = __fma_rn(o.x, o.x, acc0);
-            acc1 = __fma_rn(o.y, o.y, acc1);
+          for (int r = 0; r < kUnrollB; ++r) {
+            const size_t idx = (size_t)(gb + r) * 32 + lane;
+            if ((gb + r < g1) && idx < G) {
+              const double2 o = make_double2(__fma_rn(c, vv[r].x, zz[r].x), __fma_rn(c, vv[r].y, zz[r].y));
+              un[idx] = o;
+              acc0 = __fma_rn(o.x, o.x, acc0);
+              acc1 = __fma_rn(o.y, o.y, acc1);
+            }
           }
         }
+        accb[q] = acc0 + acc1;
       }
-      const double sb = grid_reduce(acc0 + acc1, a.rp + par, sh, a);
+      const double sb = grid_reduce(accb, a.rp + par, sh, a);
       par ^= 1;
       if (tid == 0) {
-        const double beta = sqrt(sb);
-        const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
-        const double ratio = (sn > 0.0) ? s_sigma[j] * beta : 0.0;
+        const double nrm = sqrt(sb);           // store_beta
+        const double beta = s_g[j] * nrm;
+        const double sn = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+        const double ratio = (sn > 0.0) ? (s_sigma[j] * beta) * (nrm * step_scale(sn).s) : 0.0;
         s_sigma[j + 1] = sn;
         s_ratio[j + 1] = ratio;
         if (lead) {
@@ -217,10 +235,12 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) lanczos_persiste
     const int k = s_k;
     const int N = a.in.N;
     const double2 *U1 = a.work + G;
-    double accn = 0.0;
-    {
+    double accn[V];
+#pragma unroll 1
+    for (int q = 0; q < V; ++q) {
+      double acc = 0.0;
       long long g0, g1;
-      warp_range((long long)((G + 31) >> 5), g0, g1);
+      elem_range<V>(q, (long long)((G + 31) >> 5), g0, g1);
       for (long long gi = g0; gi < g1; ++gi) {
         const size_t idx = (size_t)gi * 32 + lane;
         if (idx >= G) continue;
@@ -242,9 +262,10 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) lanczos_persiste
           oy = __dmul_rn(mv, oy);
         }
         a.psi[idx] = make_double2(ox, oy);
-        accn = __fma_rn(ox, ox, accn);
-        accn = __fma_rn(oy, oy, accn);
+        acc = __fma_rn(ox, ox, acc);
+        acc = __fma_rn(oy, oy, acc);
       }
+      accn[q] = acc;
     }
     const double sn2 = grid_reduce(accn, a.rp + par, sh, a);
     par ^= 1;
@@ -264,6 +285,8 @@ __global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM) lanczos_persiste
 
 }  // namespace
 
+constexpr int kPersistSmem = (kBlockJ / 32) * fx_warp_bytes<1>();
+
 bool lanczos_persistent_fits(int stencil) {
   int dev = 0, coop = 0, nb = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -271,14 +294,14 @@ bool lanczos_persistent_fits(int stencil) {
     cudaGetLastError();
     return false;
   }
-  const cudaError_t e = (stencil == 5)
-      ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, lanczos_persistent_kernel<5>, kBlockJ, 0)
-      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, lanczos_persistent_kernel<3>, kBlockJ, 0);
+  auto *kern = (stencil == 5) ? lanczos_persistent_kernel<5> : lanczos_persistent_kernel<3>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersistSmem);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kBlockJ, kPersistSmem);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return nb >= kStencilBlocksPerSM;
+  return nb >= 1;
 }
 
 size_t lanczos_persistent_scratch_bytes() { return 2 * sizeof(Reduction) + 2 * sizeof(unsigned); }
@@ -287,19 +310,21 @@ cudaError_t launch_lanczos_persistent(const Geometry &g, const OperatorView &op,
                                       const double *etab, double2 *psi, double2 *work, LanczosScalars *ls,
                                       Reduction *red, void *scratch, int *status, cudaStream_t st) {
   PersistArgs a;
-  StencilIn &in = a.in;
+  FxIn &in = a.in;
   in.x = psi;
-  in.diag = op.diag;
+  in.diagq = op.fx_ok ? op.diagq : reinterpret_cast<const long long *>(op.diag);
   in.rj = op.rj;
   in.kappa = op.kappa;
   in.N = g.N;
   in.L = g.L;
   in.c1 = g.c1;
   in.c2 = g.c2;
+  in.c1q = op.c1q;
+  in.c2q = op.c2q;
+  in.ec = op.fx_ec;
+  in.ok = op.fx_ok;
+  in.k = 0;
   in.E = 0.0;
-  in.dscale = 1.0;
-  in.rinv = nullptr;
-  in.d1c = 0.0;
   a.psi = psi;
   a.work = work;
   a.G = (size_t)g.N * (g.L + 1);
@@ -317,9 +342,9 @@ cudaError_t launch_lanczos_persistent(const Geometry &g, const OperatorView &op,
   cudaError_t e = cudaMemsetAsync(a.bar, 0, 2 * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(g.sms * kStencilBlocksPerSM), 1, 1);
+  cfg.gridDim = dim3((unsigned)g.sms, 1, 1);
   cfg.blockDim = dim3(kBlockJ, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = kPersistSmem;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

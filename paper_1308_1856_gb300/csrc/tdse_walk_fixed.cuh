@@ -155,7 +155,7 @@ __device__ __forceinline__ int64_t fx_shfl_up(int64_t v) { return __shfl_up_sync
 __device__ __forceinline__ int64_t fx_shfl_down(int64_t v) { return __shfl_down_sync(0xffffffffu, v, 1); }
 
 // Walk rows [l0, l1) of the strip whose first output column is j0: calls
-// f(idx, 2^k (H x), x, extra values) for every output point.  Every lane of the
+// f(idx, column, 2^k (H x), x, extra values) for every output point.  Every lane of the
 // warp calls it with the same j0, l0, l1; ring: the warp's fx_warp_bytes<EX>()
 // of shared memory.  The operand and the extra vectors are read through L2.
 template <int ST, int EX, typename F>
@@ -200,27 +200,32 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
 #pragma unroll
         for (int q = 0; q < EX; ++q)
           e[q] = *reinterpret_cast<const double2 *>(mine + slot * kSlot + 1024 + 1024 * q + 512 * c);
-        f(l * N + j + c, h_point_fp64<ST>(in, l, j + c), slot_x(slot, c), e);
+        f(l * N + j + c, j + c, h_point_fp64<ST>(in, l, j + c), slot_x(slot, c), e);
       }
   };
-  // the coupling w_j = E r_j of the lane's columns
-  const double w0 = have0 ? __dmul_rn(in.E, in.rj[j]) : 0.0, w1 = have1 ? __dmul_rn(in.E, in.rj[j + 1]) : 0.0;
+  // the tables' first entries are asked for before the rows, so that their
+  // latencies overlap: a warp's share is often a single row
+  const double rj0 = have0 ? in.rj[j] : 0.0, rj1 = have1 ? in.rj[j + 1] : 0.0;
+  const double kap0 = __ldg(in.kappa + l0);
+  double kap = __ldg(in.kappa + l0 + 1);                   // kappa of the next row
   stage(l0 - 1, 0);
   stage(l0, 1);
   stage(l0 + 1, 2);
+  // the coupling w_j = E r_j of the lane's columns
+  const double w0 = __dmul_rn(in.E, rj0), w1 = __dmul_rn(in.E, rj1);
   const uint32_t wm = max(fx_field(w0), fx_field(w1));
   const bool all_ok = in.ok && __all_sync(0xffffffffu, wm != kExpMask) != 0;
   const int we = max((int)(wm >> 20), 1), ew = we - 1022;  // w = W 2^(ew - 60)
   const Limb W[2] = {fx_limbs(fx_small(w0, we)), fx_limbs(fx_small(w1, we))};
   const bool has_w = (W[0].h | W[0].l | W[1].h | W[1].l) != 0;
-  auto coupling = [&](int l, Limb (&a)[2]) {               // a = kappa_l w = A 2^(ew - 61)
-    const Limb kp = fx_limbs(fx_coef((uint64_t)__double_as_longlong(__ldg(in.kappa + l)), 0));
+  auto coupling = [&](double kappa, Limb (&a)[2]) {        // a = kappa_l w = A 2^(ew - 61)
+    const Limb kp = fx_limbs(fx_coef((uint64_t)__double_as_longlong(kappa), 0));
     a[0] = fx_limbs(fx_coef_product(kp, W[0]));
     a[1] = fx_limbs(fx_coef_product(kp, W[1]));
   };
   const Limb k1 = fx_limbs(in.c1q), k2 = fx_limbs(in.c2q);
   Limb acur[2], anext[2];
-  coupling(l0, acur);
+  coupling(kap0, acur);
   FxRow prev, cur, next;
   cp_async_wait<1>();
   fx_convert(slot_x(0, 0), slot_x(0, 1), prev);
@@ -231,7 +236,8 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
   for (int l = l0; l < l1; ++l) {
     cp_async_wait<1>();
     fx_convert(slot_x(s1, 0), slot_x(s1, 1), next);
-    coupling(l + 1, anext);
+    coupling(kap, anext);
+    if (l + 1 < l1) kap = __ldg(in.kappa + l + 2);
     const int eU = __shfl_up_sync(0xffffffffu, cur.e, 1), eD = __shfl_down_sync(0xffffffffu, cur.e, 1);
     // exponent of the point's sum: the largest of its terms', coefficients included
     const int eb = max(cur.e, max(eU, eD));
@@ -306,7 +312,8 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
           double2 e[EX > 0 ? EX : 1];
 #pragma unroll
           for (int q = 0; q < EX; ++q) e[q] = *reinterpret_cast<const double2 *>(body + 1024 + 1024 * q + 512 * c);
-          f(l * N + j + c, make_double2(t[c][0], t[c][1]), *reinterpret_cast<const double2 *>(body + 512 * c), e);
+          f(l * N + j + c, j + c, make_double2(t[c][0], t[c][1]), *reinterpret_cast<const double2 *>(body + 512 * c),
+            e);
         }
     } else {
       slow(l, s0);
@@ -321,6 +328,24 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
     acur[1] = anext[1];
   }
   cp_async_wait<0>();   // the ring is free for the next call
+}
+
+// Visit this warp's share of the strips' row segments (strip-major): f(j0, l0,
+// l1), by every lane.  Warp k of block b of a grid of B blocks has number
+// k B + b: the first of the numbers take one segment more, and so do as many
+// warps of every block.
+template <typename F>
+__device__ __forceinline__ void for_my_strips(const FxIn &in, F &&f) {
+  const unsigned Lp1 = (unsigned)in.L + 1u, T = (((unsigned)in.N + kFxCols - 1u) / kFxCols) * Lp1;
+  const unsigned W = gridDim.x * (blockDim.x >> 5), w = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const unsigned q = T / W, r = T - q * W;
+  unsigned s = w * q + min(w, r);
+  const unsigned s_end = s + q + (w < r ? 1u : 0u);
+  while (s < s_end) {
+    const unsigned sg = s / Lp1, l0 = s - sg * Lp1, l1 = min(Lp1, l0 + (s_end - s));
+    f((int)(sg * kFxCols), (int)l0, (int)l1);
+    s += l1 - l0;
+  }
 }
 
 }  // namespace stencil
