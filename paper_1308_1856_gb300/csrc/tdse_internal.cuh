@@ -255,4 +255,17 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
 }
 
+// A kernel's launch shape, or why it could not be set up.
+struct OpLaunch {
+  unsigned grid, threads;
+  size_t bytes;
+  cudaError_t ready;
+};
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), const OpLaunch &o, cudaStream_t st, Args... args) {
+  if (o.ready != cudaSuccess) return o.ready;
+  const cudaError_t e = launch_pdl(kern, o.grid, o.threads, o.bytes, st, args...);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 }  // namespace tdse_dev

@@ -90,7 +90,8 @@ __device__ __forceinline__ void for_my_points(const OpIn<WALK> &in, const FxExtr
 // ---------------------------------------------------------------------------
 // y = H(E) x
 template <int ST, int WALK>
-__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>) apply_h_kernel(OpIn<WALK> in, double2 *__restrict__ y) {
+__global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
+    apply_h_kernel(OpIn<WALK> in, double2 *__restrict__ y) {
   for_my_points<ST, WALK, 0>(in, FxExtra<0>{}, [&](int idx, int, double2 t, double2, const double2 (&)[1]) {
     y[idx] = t;
   });
@@ -569,7 +570,6 @@ template <int WALK>
 inline unsigned stencil_blocks(const Geometry &g) { return (unsigned)(g.sms * kOpBlocksPerSM<WALK>); }
 inline unsigned elem_blocks(const Geometry &g) { return (unsigned)(g.sms * kElemBlocksPerSM); }
 
-
 // The parts a fixed-point launch's blocks are cut to: half the warps where the
 // strips' row segments need no more.  Two blocks then fit on an SM, so that the
 // next kernel of the chain is resident and waiting when this one ends.  The
@@ -582,8 +582,8 @@ inline unsigned block_parts(const Geometry &g) {
 
 // A stencil kernel's launch: its rings are dynamic shared memory, raised above
 // the 48 KB default once per instantiation (kern is a compile-time constant).
-template <auto KERN, int WALK, int EX, bool PDL = true, typename... Args>
-cudaError_t launch_op(const Geometry &g, cudaStream_t st, Args... args) {
+template <auto KERN, int WALK, int EX>
+OpLaunch op_launch(const Geometry &g) {
   constexpr size_t bytes = WALK == kFixed ? (kBlockJ / 32) * (size_t)fx_warp_bytes<EX>() : 0;
   const unsigned parts = WALK == kFixed ? block_parts(g) : 1u;
   if (WALK == kFixed) {
@@ -595,12 +595,9 @@ cudaError_t launch_op(const Geometry &g, cudaStream_t st, Args... args) {
                                                  cudaSharedmemCarveoutMaxShared);
       return e != cudaSuccess ? e : cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     }();
-    if (ready != cudaSuccess) return ready;
+    if (ready != cudaSuccess) return OpLaunch{0, 0, 0, ready};
   }
-  cudaError_t e = cudaSuccess;
-  if (PDL) e = launch_pdl(KERN, stencil_blocks<WALK>(g), kBlockJ / parts, bytes / parts, st, args...);
-  else KERN<<<stencil_blocks<WALK>(g), kBlockJ / parts, bytes / parts, st>>>(args...);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return OpLaunch{stencil_blocks<WALK>(g), kBlockJ / parts, bytes / parts, cudaSuccess};
 }
 
 }  // namespace
@@ -617,7 +614,10 @@ cudaError_t launch_apply_h(const Geometry &g, const OperatorView &op, double E,
   dispatch<false>(g, g.gauge == 1, false, [&](auto st, auto walk) {
     constexpr int ST = decltype(st)::value;
     constexpr int WALK = decltype(walk)::value;
-    e = launch_op<apply_h_kernel<ST, WALK>, WALK, 0, false>(g, s, make_in<WALK>(g, op, E, x), y);
+    const OpLaunch o = op_launch<apply_h_kernel<ST, WALK>, WALK, 0>(g);
+    if ((e = o.ready) != cudaSuccess) return;
+    apply_h_kernel<ST, WALK><<<o.grid, o.threads, o.bytes, s>>>(make_in<WALK>(g, op, E, x), y);
+    e = cudaGetLastError();
   });
   return e;
 }
@@ -633,13 +633,19 @@ cudaError_t launch_taylor_stage(const Geometry &g, const OperatorView &op, doubl
     const auto in = make_in<WALK>(g, op, E, v_in);
     if constexpr (WALK == kFixed)   // imaginary time: no absorber, no field
       if (imag) {
-        e = launch_op<taylor_stage_kernel<ST, true, kFixed, false>, kFixed, 1>(g, st, in, s, psi, v_out, op.mask, mstart);
+        e = launch_pdl(taylor_stage_kernel<ST, true, kFixed, false>,
+                       op_launch<taylor_stage_kernel<ST, true, kFixed, false>, kFixed, 1>(g), st, in, s, psi,
+                       v_out, op.mask, mstart);
         return;
       }
     if (final_stage)
-      e = launch_op<taylor_stage_kernel<ST, false, WALK, true>, WALK, 1>(g, st, in, s, psi, v_out, op.mask, mstart);
+      e = launch_pdl(taylor_stage_kernel<ST, false, WALK, true>,
+                     op_launch<taylor_stage_kernel<ST, false, WALK, true>, WALK, 1>(g), st, in, s, psi, v_out,
+                     op.mask, mstart);
     else
-      e = launch_op<taylor_stage_kernel<ST, false, WALK, false>, WALK, 1>(g, st, in, s, psi, v_out, op.mask, mstart);
+      e = launch_pdl(taylor_stage_kernel<ST, false, WALK, false>,
+                     op_launch<taylor_stage_kernel<ST, false, WALK, false>, WALK, 1>(g), st, in, s, psi, v_out,
+                     op.mask, mstart);
   });
   return e;
 }
@@ -661,8 +667,9 @@ cudaError_t launch_rk_stage(const Geometry &g, const OperatorView &op, double E,
       constexpr int PART = decltype(part)::value;
       constexpr bool IMAG = decltype(im)::value;
       constexpr int EX = PART == 0 ? 0 : (PART == 1 ? 2 : 1);
-      e = launch_op<rk_stage_kernel<ST, IMAG, WALK, PART>, WALK, EX>(g, st, in, ca, cb, psi, acc, g_next, psi_out, op.mask,
-                                                                 mstart);
+      e = launch_pdl(rk_stage_kernel<ST, IMAG, WALK, PART>,
+                     op_launch<rk_stage_kernel<ST, IMAG, WALK, PART>, WALK, EX>(g), st, in, ca, cb, psi, acc, g_next,
+                     psi_out, op.mask, mstart);
     };
     auto parts = [&](auto im) {
       if (stage == 1) go(IC<0>{}, im);
@@ -691,9 +698,10 @@ cudaError_t launch_rk_general_stage(const Geometry &g, const OperatorView &op, d
     const auto in = make_in<WALK>(g, op, E, gin);
     auto launch = [&](auto nk, auto md) {
       constexpr int NK = decltype(nk)::value, MODE = decltype(md)::value;
-      constexpr int VECS = MODE == 2 ? NK - 1 : NK;
-      e = launch_op<rk_general_stage_kernel<ST, WALK, NK, MODE>, WALK, (VECS < 2 ? VECS : 2)>(
-          g, st, in, a, psi, op.mask, op.mask_start, red, S);
+      constexpr int VECS = MODE == 2 ? NK - 1 : NK, EX = VECS < 2 ? VECS : 2;
+      e = launch_pdl(rk_general_stage_kernel<ST, WALK, NK, MODE>,
+                     op_launch<rk_general_stage_kernel<ST, WALK, NK, MODE>, WALK, EX>(g), st, in, a, psi, op.mask,
+                     op.mask_start, red, S);
     };
     auto go = [&](auto nk) {
       constexpr int NK = decltype(nk)::value;
@@ -743,8 +751,10 @@ cudaError_t launch_lanczos_a(const Geometry &g, const OperatorView &op, double E
     constexpr int ST = decltype(stc)::value;
     constexpr int WALK = decltype(walk)::value;
     const auto in = make_in<WALK>(g, op, E, u);
-    if (j > 0) e = launch_op<lanczos_a_kernel<ST, WALK, 1>, WALK, 1>(g, st, in, j, uprev, z, red, ls);
-    else e = launch_op<lanczos_a_kernel<ST, WALK, 0>, WALK, 0>(g, st, in, j, uprev, z, red, ls);
+    if (j > 0) e = launch_pdl(lanczos_a_kernel<ST, WALK, 1>,
+                   op_launch<lanczos_a_kernel<ST, WALK, 1>, WALK, 1>(g), st, in, j, uprev, z, red, ls);
+    else e = launch_pdl(lanczos_a_kernel<ST, WALK, 0>,
+                   op_launch<lanczos_a_kernel<ST, WALK, 0>, WALK, 0>(g), st, in, j, uprev, z, red, ls);
   });
   return e;
 }
