@@ -44,7 +44,8 @@ namespace tdse_dev {
 
 namespace {
 
-using common::warp_sum;
+using common::norm_and_inverse;
+using common::warp_sum_fx;
 
 constexpr int kCT = 256;   // threads per CTA
 static_assert(kCT == kEx, "the small exponential body runs on the whole CTA");
@@ -164,14 +165,15 @@ __device__ __forceinline__ void for_points(const Slab &s, const Lanes &ln, F &&f
 }
 
 // Sum over the cluster, the same bits in every CTA.  Every warp publishes its
-// shuffle-tree sum in one of two slot sets (alternating, so a set is
+// sum in one of two slot sets (alternating, so a set is
 // rewritten only after a later cluster barrier, when every CTA has read it);
 // after the cluster barrier warp 0 of every CTA adds the C x 8 warp sums in
 // one fixed order (lane t: the sums t, t + 32, t + 64, t + 96 in pairs, then
-// a shuffle tree), and thread 0 hands the total to `fin`, whose results the
+// the warp's sum), and thread 0 hands the total to `fin`, whose results the
 // closing CTA barrier publishes.  Each FP64 instruction of this dependent
 // chain holds the narrow FP64 pipe for a full pass, so the chain is kept
-// short: 12 additions and one CTA barrier besides the cluster barrier.
+// short: two additions, two integer conversions (warp_sum_fx) and one CTA
+// barrier besides the cluster barrier.
 constexpr int kWarps = kCT / 32;
 static_assert(kMaxCluster * kWarps <= 128, "four warp sums per lane of warp 0");
 struct ClusterSum {
@@ -184,7 +186,7 @@ __device__ __forceinline__ void cluster_sum(const cg::cluster_group &cl, Cluster
                                             Fin &&fin) {
   const int lane = (int)threadIdx.x & 31, w = (int)threadIdx.x >> 5;
   double *set = cs.slot + cs.par * kWarps;
-  v = warp_sum(v);
+  v = warp_sum_fx(v);
   if (lane == 0) set[w] = v;
   cl.sync();
   if (w == 0) {
@@ -194,24 +196,11 @@ __device__ __forceinline__ void cluster_sum(const cg::cluster_group &cl, Cluster
       const int i = lane + 32 * q;   // warp i % kWarps of CTA i / kWarps
       p[q] = (i < C * kWarps) ? *cl.map_shared_rank(set + (i % kWarps), i / kWarps) : 0.0;
     }
-    const double t = warp_sum(__dadd_rn(__dadd_rn(p[0], p[1]), __dadd_rn(p[2], p[3])));
+    const double t = warp_sum_fx(__dadd_rn(__dadd_rn(p[0], p[1]), __dadd_rn(p[2], p[3])));
     if (lane == 0) fin(t);
   }
   __syncthreads();
   cs.par ^= 1;
-}
-
-// ||x|| and 1 / ||x|| from ||x||^2 with one reciprocal square root and one
-// product (about half the dependent FP64 instructions of a square root and a
-// division); 0 gives (0, 0), Inf or NaN gives (sqrt, 0).
-__device__ __forceinline__ void norm_and_inverse(double s2, double &nrm, double &inv) {
-  if (s2 > 0.0 && s2 <= 1.7976931348623157e308) {
-    inv = rsqrt(s2);
-    nrm = __dmul_rn(s2, inv);
-  } else {
-    nrm = sqrt(s2);
-    inv = 0.0;
-  }
 }
 
 // Sum of |x|^2 over this thread's points, in the order of the Lanczos combine.

@@ -146,6 +146,23 @@ FX_HD uint64_t fx_to_bits(int64_t V, int E) {
   return A ? b : 0;
 }
 
+// A warp's sum of 32 doubles: each is held as a 58-bit integer against the
+// largest exponent field e of the warp (kSumLo <= e <= kSumHi), rounded to
+// nearest, v = X 2^(e - kSumBias), |X| <= 2^57, so that the sum stays below 2^62;
+// the values within 2^-4 of the largest are exact and the others are off by at
+// most half of 2^-57 of the largest's power of two, where an FP64 addition rounds
+// to 2^-53 of its sum.  The integers are added as three pieces of 20, 20 and 18 bits.
+constexpr int kSumBias = 1079, kSumLo = 128, kSumHi = 2000;
+FX_HD int64_t fx_addend(uint32_t hi, uint32_t lo, int e) {
+  const int f = (int)((hi & kExpMask) >> 20);
+  const uint64_t M = ((uint64_t)((hi & 0xfffffu) | (f ? 0x100000u : 0u)) << 32) | lo;
+  const int d = e - f;                                 // subnormal values (f = 0) fall below the last bit
+  return fx_signed((((M << 5) >> (d < 63 ? d : 63)) + 1) >> 1, hi);
+}
+FX_HD int64_t fx_total(uint32_t p0, uint32_t p1, int32_t p2) {
+  return (int64_t)(((uint64_t)(int64_t)p2 << 40) + ((uint64_t)p1 << 20) + p0);
+}
+
 // The exponent of the Laplacian's and the diagonal's coefficients: room for
 // diagonal entries of more than twice c0, the value the diagonal tends to;
 // larger ones (the centrifugal term next to the origin) carry a shift of their

@@ -354,9 +354,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     const double s = reduce_partials(red, gridDim.x, sh);
     if (threadIdx.x == 0) {
       red->normsq = s;
-      const double nrm = sqrt(s);
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+      norm_and_inverse(s, ls->psinorm, ls->sigma[0]);
       if (!isfinite(s)) atomicOr(status, kStatusNonFinite);
     }
   }
@@ -422,9 +420,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     const double s = reduce_partials(red, gridDim.x, sh);
     if (threadIdx.x == 0) {
       red->normsq = s;
-      const double nrm = sqrt(s);
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+      norm_and_inverse(s, ls->psinorm, ls->sigma[0]);
       if (!isfinite(s)) atomicOr(status, kStatusNonFinite);
     }
   }

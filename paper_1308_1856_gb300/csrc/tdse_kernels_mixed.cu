@@ -89,9 +89,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     const double s = reduce_partials(red, gridDim.x, sh);
     if (threadIdx.x == 0) {
       red->normsq = s;
-      const double nrm = sqrt(s);
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+      norm_and_inverse(s, ls->psinorm, ls->sigma[0]);
       if (!isfinite(s)) atomicOr(status, kStatusNonFinite);
     }
   }
@@ -202,9 +200,9 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
   if (publish_block_partial(accd, red, sh)) {
     const double s = reduce_partials(red, gridDim.x, sh);
     if (threadIdx.x == 0) {
-      const double beta = sqrt(s);
+      double beta, sn;
+      norm_and_inverse(s, beta, sn);
       ls->beta[j] = beta;
-      const double sn = (beta > 0.0) ? 1.0 / beta : 0.0;
       ls->sigma[j + 1] = sn;
       ls->ratio[j + 1] = (sn > 0.0) ? ls->sigma[j] * beta : 0.0;
     }
@@ -276,9 +274,7 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
     const double s = reduce_partials(red, gridDim.x, sh);
     if (threadIdx.x == 0) {
       red->normsq = s;
-      const double nrm = sqrt(s);
-      ls->psinorm = nrm;
-      ls->sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+      norm_and_inverse(s, ls->psinorm, ls->sigma[0]);
       if (!isfinite(s)) atomicOr(status, kStatusNonFinite);
     }
   }

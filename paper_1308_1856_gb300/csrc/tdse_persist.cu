@@ -211,9 +211,9 @@ __global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistA
       const double sb = grid_reduce(accb, a.rp + par, sh, a);
       par ^= 1;
       if (tid == 0) {
-        const double nrm = sqrt(sb);           // store_beta
+        double nrm, sn;                        // store_beta
+        norm_and_inverse(sb, nrm, sn);
         const double beta = s_g[j] * nrm;
-        const double sn = (nrm > 0.0) ? 1.0 / nrm : 0.0;
         const double ratio = (sn > 0.0) ? (s_sigma[j] * beta) * (nrm * step_scale(sn).s) : 0.0;
         s_sigma[j + 1] = sn;
         s_ratio[j + 1] = ratio;
@@ -270,8 +270,8 @@ __global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistA
     const double sn2 = grid_reduce(accn, a.rp + par, sh, a);
     par ^= 1;
     if (tid == 0) {
-      const double nrm = sqrt(sn2);
-      s_sigma[0] = (nrm > 0.0) ? 1.0 / nrm : 0.0;
+      double nrm;
+      norm_and_inverse(sn2, nrm, s_sigma[0]);
       if (lead) {
         a.red->normsq = sn2;
         a.ls->psinorm = nrm;
