@@ -314,24 +314,6 @@ __device__ __forceinline__ void for_elem_chunks(const BatchDev &B, const ChunkLi
 }
 
 // ---- FP64 ------------------------------------------------------------------
-__device__ __forceinline__ StencilIn fp64_in(const BatchDev &B, const BatchInst &I, int inst,
-                                             const double2 *x) {
-  StencilIn in;
-  in.x = x;
-  in.diag = I.diag;
-  in.rj = I.rj;
-  in.kappa = I.kappa;
-  in.N = I.N;
-  in.L = I.L;
-  in.c1 = I.c1;
-  in.c2 = I.c2;
-  in.E = field_of(B, inst);   // A/c for a velocity-gauge instance
-  in.dscale = 1.0;
-  in.rinv = I.rinv;
-  in.d1c = I.d1c;
-  return in;
-}
-
 __device__ __forceinline__ FxIn fixed_in(const BatchDev &B, const BatchInst &I, int inst, const double2 *x, int k) {
   FxIn in;
   in.x = x;
@@ -348,6 +330,8 @@ __device__ __forceinline__ FxIn fixed_in(const BatchDev &B, const BatchInst &I, 
   in.ec = I.fx_ec;
   in.ok = I.fx_ok;
   in.k = k;
+  in.rinv = I.rinv;
+  in.d1c = I.d1c;
   return in;
 }
 
@@ -366,7 +350,7 @@ __device__ __forceinline__ void for_strided_chunks(const ChunkList &cl, F &&f) {
   }
 }
 
-// Phase A of the length-gauge instances: the fixed-point walker
+// Phase A (a launch for each gauge's instances): the fixed-point walker
 // (tdse_walk_fixed.cuh) with the recurrence and the dot product in FP64: six
 // FP64 instructions a point (two of them integer conversions) in place of 20.
 // What bounds it: the integer and FP64 pipes' issue together (integer 76%, FP64
@@ -374,10 +358,10 @@ __device__ __forceinline__ void for_strided_chunks(const ChunkList &cl, F &&f) {
 // All phase A launches of one step of 128 instances (8.1e7 points): 36.9 ms in
 // FP64, 19.5 ms here; of 8 instances (1.3e6 points), 24 ms to 6 ms over 8 steps,
 // where the smaller chunks count as well.
-template <int ST, int EX>
+template <int ST, bool VG, int EX>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM) bt_lanczos_a_fixed(BatchDev B, ChunkList cl, int j) {
   extern __shared__ __align__(16) unsigned char fx_smem[];
-  unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX>();
+  unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX, VG>();
   for_strided_chunks(cl, [&](int inst, int ci) {
     const BatchInst &I = B.inst[inst];
     LanczosScalars *ls = B.ls + inst;
@@ -391,7 +375,7 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM) bt_lanczos_a_fixed
     const FxIn in = fixed_in(B, I, inst, u, s0.k);
     double acc = 0.0;
     chunk_strips(I, ci, [&](int j0, int l0, int l1) {
-      walk_rows_fixed<ST, EX>(in, up, ring, j0, l0, l1,
+      walk_rows_fixed<ST, VG, EX>(in, up, ring, j0, l0, l1,
                               [&](int idx, int, double2 t, double2 uc, const double2 (&e)[1]) {
         double2 o = t;
         if (EX > 0) {
@@ -405,44 +389,6 @@ __global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM) bt_lanczos_a_fixed
     });
     double s;
     if (chunk_done(B, I.dpart, inst, ci, I.nchunk, acc, s) && (threadIdx.x & 31) == 0) store_alpha(ls, j, s);
-  });
-}
-
-// Phase A of the velocity-gauge instances (a launch of its own over their
-// row-segment chunks), all in FP64.
-template <int ST, int PF>
-__global__ void __launch_bounds__(kBlockJ, kStencilBlocksPerSM)
-    bt_lanczos_a_fp64_vg(BatchDev B, ChunkList cl, int j) {
-  for_my_chunks(cl, [&](int inst, int ci) {
-    const BatchInst I = B.inst[inst];
-    LanczosScalars *ls = B.ls + inst;
-    const long long G = (long long)I.N * (I.L + 1);
-    const double2 *u = (j == 0) ? I.psi : I.work + (long long)j * G;
-    const double2 *up = (j <= 1) ? I.psi : I.work + (long long)(j - 1) * G;
-    double2 *z = I.work;
-    const double sig = ls->sigma[j];
-    const StepScale sc = step_scale(sig);
-    const double cprev = (j > 0) ? ls->ratio[j] : 0.0;
-    // t = s_j H U_j directly (the operator scaled by s_j)
-    const StencilIn in = scaled(fp64_in(B, I, inst, u), sc.s);
-    double acc = 0.0;
-    chunk_columns(I, ci, [&](int i, int l0, int l1) {
-      walk_rows<ST, PF, true, true>(in, i, l0, l1, [&](int, size_t idx, double2 t, double2 uc) {
-        double2 o;
-        if (j > 0) {
-          const double2 pv = up[idx];
-          o.x = __fma_rn(-cprev, pv.x, t.x);
-          o.y = __fma_rn(-cprev, pv.y, t.y);
-        } else {
-          o = t;
-        }
-        z[idx] = o;
-        acc = __fma_rn(uc.x, o.x, acc);
-        acc = __fma_rn(uc.y, o.y, acc);
-      });
-    });
-    double s;
-    if (chunk_done(B, I.partial, inst, ci, I.nchunk, acc, s) && (threadIdx.x & 31) == 0) store_alpha(ls, j, s);
   });
 }
 
@@ -1331,14 +1277,14 @@ int Engine::place(int slot, const tdse_instance_spec &s, void *mem) {
   I.L = L;
   I.m = s.krylov;
   I.nseg = (int)((size_t)((N + 31) / 32) * (L + 1));
-  // reduction chunks of the stencil kernel: row segments (64 of 32 columns in
-  // the velocity gauge, fx_rows of kFxCols in FP64 length gauge), or tiles of
+  // reduction chunks of the stencil kernel: row segments (fx_rows of kFxCols in
+  // FP64, 64 of 32 columns in the mixed velocity gauge), or tiles of
   // 256 columns x kTileRows rows (the mixed tile kernel)
   const bool vg = s.gauge == TDSE_GAUGE_VELOCITY;
   I.fx_seg = (int)fx_segments(N, L + 1);
   I.fx_rows = fx_chunk_rows(N, L + 1);
-  I.nchunk = vg ? (I.nseg + kChunkSegs - 1) / kChunkSegs
-                : (mixed ? tile_count(N, L) : (I.fx_seg + I.fx_rows - 1) / I.fx_rows);
+  I.nchunk = !mixed ? (I.fx_seg + I.fx_rows - 1) / I.fx_rows
+                    : (vg ? (I.nseg + kChunkSegs - 1) / kChunkSegs : tile_count(N, L));
   I.nchunk_e = (int)((G + kChunkPts - 1) / kChunkPts);
   I.nchunk_d = (I.nseg + kChunkSegs - 1) / kChunkSegs;
   I.dr = s.dr;
@@ -1434,7 +1380,7 @@ int Engine::place(int slot, const tdse_instance_spec &s, void *mem) {
     EN_CUDA(cudaMemcpyAsync((void *)I.rjf, rf.data(), sizeof(float) * N, cudaMemcpyHostToDevice, st), "r table");
     EN_CUDA(cudaMemcpyAsync((void *)I.kappaf, kf.data(), sizeof(float) * (L + 2), cudaMemcpyHostToDevice, st), "kappa");
   }
-  if (!mixed && !vg) {
+  if (!mixed) {
     // largest |diagonal|: the centrifugal and Coulomb terms at the first point
     const double dmax = c0 + 0.5 * (double)L * (double)(L + 1) / (rj[0] * rj[0]) + std::fabs(s.Z) / rj[0];
     I.fx_ok = tdse_fx::fx_scale(c0, I.fx_ec) && tdse_fx::fx_diag_fits(dmax, I.fx_ec) ? 1 : 0;
@@ -1669,14 +1615,19 @@ namespace {
 constexpr long kGraphMinSteps = 3;   // segments this long replay one captured step graph
 constexpr size_t kGraphCache = 8;    // captured step graphs kept across runs
 
-template <int ST, int EX>
-cudaError_t launch_fixed(unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
-  constexpr int bytes = (kFxThreads / 32) * fx_warp_bytes<EX>();
-  static const cudaError_t ready = cudaFuncSetAttribute(bt_lanczos_a_fixed<ST, EX>,
+template <int ST, bool VG, int EX>
+cudaError_t launch_fixed_ex(unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
+  constexpr int bytes = (kFxThreads / 32) * fx_warp_bytes<EX, VG>();
+  static const cudaError_t ready = cudaFuncSetAttribute(bt_lanczos_a_fixed<ST, VG, EX>,
                                                         cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (ready != cudaSuccess) return ready;
-  bt_lanczos_a_fixed<ST, EX><<<grid, kFxThreads, bytes, st>>>(B, cl, j);
+  bt_lanczos_a_fixed<ST, VG, EX><<<grid, kFxThreads, bytes, st>>>(B, cl, j);
   return cudaGetLastError();
+}
+
+template <int ST, bool VG>
+cudaError_t launch_fixed(unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
+  return j ? launch_fixed_ex<ST, VG, 1>(grid, st, B, cl, j) : launch_fixed_ex<ST, VG, 0>(grid, st, B, cl, j);
 }
 
 // The mixed tile kernel: dynamic shared memory of its ring of D row slots,
@@ -1710,16 +1661,6 @@ cudaError_t launch_tile_ring(int ring, unsigned grid, cudaStream_t st, const Bat
   if (ring == 0) return launch_tile<ST, 4>(grid, st, B, cl, j);
   if (ring == 3) return launch_tile<ST, 8>(grid, st, B, cl, j);
   return launch_tile<ST, 12>(grid, st, B, cl, j);
-}
-
-template <int ST>
-void launch_a_vg_st(int pf, unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
-  switch (pf) {
-    case 0: bt_lanczos_a_fp64_vg<ST, 0><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-    case 3: bt_lanczos_a_fp64_vg<ST, 3><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-    case 10: bt_lanczos_a_fp64_vg<ST, 10><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-    default: bt_lanczos_a_fp64_vg<ST, 6><<<grid, kBlockJ, 0, st>>>(B, cl, j); break;
-  }
 }
 
 }  // namespace
@@ -1882,8 +1823,8 @@ int Engine::launch_a(const BatchDev &B, const ChunkList &cl, int j, const Schedu
     return TDSE_OK;
   }
   const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM : kFxBlocksPerSM / 2));
-  const cudaError_t e = stencil == 5 ? (j ? launch_fixed<5, 1>(grid, stream, B, cl, j) : launch_fixed<5, 0>(grid, stream, B, cl, j))
-                                     : (j ? launch_fixed<3, 1>(grid, stream, B, cl, j) : launch_fixed<3, 0>(grid, stream, B, cl, j));
+  const cudaError_t e = stencil == 5 ? launch_fixed<5, false>(grid, stream, B, cl, j)
+                                     : launch_fixed<3, false>(grid, stream, B, cl, j);
   EN_CUDA(e, "batch lanczos a");
   return TDSE_OK;
 }
@@ -1893,19 +1834,20 @@ int Engine::stencil_wave() const {
   return precision == TDSE_MIXED ? sms * sched.sblocks * (kBlockJ / 32) : sms * kFxBlocksPerSM * (kFxThreads / 32);
 }
 
-// Velocity-gauge instances: the same FP64 kernel with the (A/c) p_z coupling,
+// Velocity-gauge instances: the same fixed-point walker with the (A/c) p_z coupling,
 // or the mixed register walker with it.
 int Engine::launch_a_velocity(const BatchDev &B, const ChunkList &cl, int j, const Schedule &s) {
-  const unsigned grid = (unsigned)(sms * s.sblocks);
   if (precision == TDSE_MIXED) {
+    const unsigned grid = (unsigned)(sms * s.sblocks);
     if (stencil == 5) bt_lanczos_a_mixed_vg<5><<<grid, kBlockJ, 0, stream>>>(B, cl, j);
     else bt_lanczos_a_mixed_vg<3><<<grid, kBlockJ, 0, stream>>>(B, cl, j);
     EN_CUDA(cudaGetLastError(), "batch lanczos a (mixed, velocity gauge)");
     return TDSE_OK;
   }
-  if (stencil == 5) launch_a_vg_st<5>(s.pf, grid, stream, B, cl, j);
-  else launch_a_vg_st<3>(s.pf, grid, stream, B, cl, j);
-  EN_CUDA(cudaGetLastError(), "batch lanczos a (velocity gauge)");
+  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM : kFxBlocksPerSM / 2));
+  const cudaError_t e = stencil == 5 ? launch_fixed<5, true>(grid, stream, B, cl, j)
+                                     : launch_fixed<3, true>(grid, stream, B, cl, j);
+  EN_CUDA(e, "batch lanczos a (velocity gauge)");
   return TDSE_OK;
 }
 

@@ -39,14 +39,14 @@ struct BatchInst {
   const double *rinv;    // 1/r_j (FP64 velocity gauge; null otherwise)
   const float *rinvf;    // 1/r_j (mixed velocity gauge; null otherwise)
   double2 *psi;          // (L+1) x N state, l-major
-  const double *diag;    // FP64: c0 + l(l+1)/(2 r^2) - Z/r; encoded (fx_encode_diag) in the length gauge if fx_ok
+  const double *diag;    // FP64: c0 + l(l+1)/(2 r^2) - Z/r; encoded (fx_encode_diag) if fx_ok
   const float *diagf;    // mixed: l(l+1)/(2 r^2) - Z/r (difference-form stencil)
   const double *rj, *kappa, *mask;
   const float *rjf, *kappaf;
   float2 *hi, *lo;       // mixed: split of psi
   double2 *work;         // FP64 Krylov area: slot 0 = z, slots 1..m-1 = U_j
   float2 *mwork;         // mixed Krylov area, same slots
-  double *partial;       // chunk partials of the mixed and the velocity-gauge stencil kernels
+  double *partial;       // chunk partials of the mixed stencil kernels
   double *dpart;         // 4 * nchunk_d chunk partials of the dipole, fixed-point stencil and elementwise kernels
   double2 *ref0;         // N values: the p_ground reference (1s state of the grid)
 };

@@ -1,31 +1,27 @@
 // FP64 kernels of the finite-difference TDSE path (sm_103a).
 //
-// Every stencil kernel evaluates the length-gauge Hamiltonian of Eq. (h_matrix)
+// Every stencil kernel evaluates the Hamiltonian of Eq. (h_matrix), in the length gauge
 // (arXiv 1308.1856, Sec. 2):
 //   (H x)_{l,j} = D_{l,j} x_{l,j} + c1 (x_{l,j-1} + x_{l,j+1}) [+ c2 (x_{l,j-2} + x_{l,j+2})]
 //               + E r_j (kappa_l x_{l-1,j} + kappa_{l+1} x_{l+1,j})
 // with D_{l,j} = c0 + l(l+1)/(2 r_j^2) + V(r_j) read from a table, H real and
 // symmetric, so the real and imaginary parts go through the same real operator.
 //
-// Length gauge: the fixed-point walker (tdse_walk_fixed.cuh).  An FP64
+// The operator runs in the fixed-point walker (tdse_walk_fixed.cuh).  An FP64
 // instruction of a warp takes its SM sub-partition 64 cycles, so the 15 of a
-// point's H x bounded these kernels; in fixed point the operator runs on the
-// integer pipe and only the epilogue is FP64.  The (L+1) rows of the strips of
-// kFxCols columns form one strip-major sequence of row segments; warp w of the
-// persistent grid takes a contiguous, balanced range of it (for_my_strips).  The
-// warps' numbers run across the blocks, so that the warps with one segment more
-// are spread evenly over the SMs.  What bounds it now is the integer pipe's issue
-// with the FP64 epilogue beside it.  512,000 points (8000 x 64): H x 23.5 to
-// 14.4 us a call, a Taylor stage 19.5 to 13.6, an RK4 stage 22.2 to 16.8, a
-// Lanczos-12 step 607 to 497.
+// point's H x (velocity gauge: 34) bounded these kernels; in fixed point the
+// operator runs on the integer pipe and only the epilogue is FP64.  The (L+1)
+// rows of the strips of kFxCols columns form one strip-major sequence of row
+// segments; warp w of the persistent grid takes a contiguous, balanced range of
+// it (for_my_strips).  The warps' numbers run across the blocks, so that the
+// warps with one segment more are spread evenly over the SMs.
 //
-// Velocity gauge, and Taylor and RK4 stages of grids that fit the one-launch
-// cluster path, whose states are bitwise these: all in FP64, in
-// segments of 32 radial points of one partial wave, ordered
-// radial-group-major, a contiguous balanced range for each warp (warp_range).
-// A lane owns one radial index j and walks l upwards keeping x_{l-1,j},
-// x_{l,j}, x_{l+1,j} in registers; the arithmetic is written with explicit
-// __dmul_rn / __dadd_rn / __fma_rn.
+// Taylor and RK4 stages of length-gauge grids that fit the one-launch cluster
+// path, whose states are bitwise these: all in FP64, in segments of 32 radial
+// points of one partial wave, ordered radial-group-major, a contiguous balanced
+// range for each warp (warp_range).  A lane owns one radial index j and walks l
+// upwards keeping x_{l-1,j}, x_{l,j}, x_{l+1,j} in registers; the arithmetic is
+// written with explicit __dmul_rn / __dadd_rn / __fma_rn.
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -43,7 +39,7 @@ using namespace common;
 using namespace stencil;
 
 // Visit this warp's share of the 32-point row segments (see the file header).
-template <int ST, bool SCALED = false, bool VG = false, typename F>
+template <int ST, typename F>
 __device__ __forceinline__ void for_my_segments(const StencilIn &in, F &&f) {
   const int lane = threadIdx.x & 31;
   const int Lp1 = in.L + 1;
@@ -56,25 +52,26 @@ __device__ __forceinline__ void for_my_segments(const StencilIn &in, F &&f) {
     const long long left = s_end - s;
     const int l1 = (left < (long long)(Lp1 - l0)) ? l0 + (int)left : Lp1;
     const int i = jg * 32 + lane;
-    if (i < in.N) walk_rows<ST, 0, SCALED, VG>(in, i, l0, l1, f);
+    if (i < in.N) walk_rows<ST>(in, i, l0, l1, f);
     s += l1 - l0;
   }
 }
 
-// How a stencil kernel walks the grid: in fixed point (length gauge), or in FP64.
-enum Walk { kFixed, kPlain, kPlainVG };
+// How a stencil kernel walks the grid: in fixed point (of the length or velocity
+// gauge), or in FP64 (length gauge).
+enum Walk { kFixed, kFixedVG, kPlain };
 template <int WALK>
-using OpIn = std::conditional_t<WALK == kFixed, FxIn, StencilIn>;
+using OpIn = std::conditional_t<WALK == kPlain, StencilIn, FxIn>;
 // Blocks an SM: one of 16 warps with 128 registers a thread and its rings in
 // fixed point, two of 64 registers in FP64.
 template <int WALK>
-constexpr int kOpBlocksPerSM = WALK == kFixed ? 1 : kStencilBlocksPerSM;
+constexpr int kOpBlocksPerSM = WALK == kPlain ? kStencilBlocksPerSM : 1;
 
 // Call f(idx, i, H x, x, extra values) at every point this thread owns.
-template <int ST, int WALK, int EX, bool SCALED = false, typename F>
+template <int ST, int WALK, int EX, typename F>
 __device__ __forceinline__ void for_my_points(const OpIn<WALK> &in, const FxExtra<EX> &ex, F &&f) {
-  if constexpr (WALK != kFixed) {
-    for_my_segments<ST, SCALED, WALK == kPlainVG>(in, [&](int i, size_t idx, double2 t, double2 u) {
+  if constexpr (WALK == kPlain) {
+    for_my_segments<ST>(in, [&](int i, size_t idx, double2 t, double2 u) {
       double2 e[EX > 0 ? EX : 1];
 #pragma unroll
       for (int q = 0; q < EX; ++q) e[q] = ex.p[q][idx];
@@ -82,8 +79,10 @@ __device__ __forceinline__ void for_my_points(const OpIn<WALK> &in, const FxExtr
     });
   } else {
     extern __shared__ __align__(16) unsigned char fx_smem[];
-    unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX>();
-    for_my_strips(in, [&](int j0, int l0, int l1) { walk_rows_fixed<ST, EX>(in, ex, ring, j0, l0, l1, f); });
+    unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX, WALK == kFixedVG>();
+    for_my_strips(in, [&](int j0, int l0, int l1) {
+      walk_rows_fixed<ST, WALK == kFixedVG, EX>(in, ex, ring, j0, l0, l1, f);
+    });
   }
 }
 
@@ -250,9 +249,8 @@ __global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
   double acc = 0.0;
   FxExtra<EX> ex;
   if (EX > 0) ex.p[0] = uprev;
-  if constexpr (WALK == kFixed) in.k = sc.k;
-  else in = scaled(in, sc.s);
-  for_my_points<ST, WALK, EX, true>(in, ex, [&](int idx, int, double2 t, double2 u, const double2 (&e)[1]) {
+  in.k = sc.k;
+  for_my_points<ST, WALK, EX>(in, ex, [&](int idx, int, double2 t, double2 u, const double2 (&e)[1]) {
     double2 o = t;
     if (EX > 0) {
       o.x = __fma_rn(-cprev, e[0].x, t.x);
@@ -518,11 +516,8 @@ __global__ void __launch_bounds__(kObsThreads)
 template <int WALK>
 OpIn<WALK> make_in(const Geometry &g, const OperatorView &op, double E, const double2 *x) {
   OpIn<WALK> in;
-  if constexpr (WALK != kFixed) {
+  if constexpr (WALK == kPlain) {
     in.diag = op.diag;
-    in.dscale = 1.0;
-    in.rinv = op.rinv;
-    in.d1c = (g.stencil == 5) ? 1.0 / (12.0 * g.dr) : 1.0 / (2.0 * g.dr);
   } else {
     in.diagq = op.fx_ok ? op.diagq : reinterpret_cast<const long long *>(op.diag);
     in.c1q = op.c1q;
@@ -531,6 +526,8 @@ OpIn<WALK> make_in(const Geometry &g, const OperatorView &op, double E, const do
     in.ok = op.fx_ok;
     in.k = 0;
   }
+  in.rinv = op.rinv;
+  in.d1c = (g.stencil == 5) ? 1.0 / (12.0 * g.dr) : 1.0 / (2.0 * g.dr);
   in.x = x;
   in.rj = op.rj;
   in.kappa = op.kappa;
@@ -552,7 +549,7 @@ using BC = std::integral_constant<bool, V>;
 template <bool PLAIN, typename F>
 void dispatch(const Geometry &g, bool vg, bool plain, F &&f) {
   auto go = [&](auto st) {
-    if (vg) return f(st, IC<kPlainVG>{});
+    if (vg) return f(st, IC<kFixedVG>{});
     if constexpr (PLAIN)
       if (plain) return f(st, IC<kPlain>{});
     f(st, IC<kFixed>{});
@@ -580,9 +577,10 @@ inline unsigned block_parts(const Geometry &g) {
 // the 48 KB default once per instantiation (kern is a compile-time constant).
 template <auto KERN, int WALK, int EX>
 OpLaunch op_launch(const Geometry &g) {
-  constexpr size_t bytes = WALK == kFixed ? (kBlockJ / 32) * (size_t)fx_warp_bytes<EX>() : 0;
-  const unsigned parts = WALK == kFixed ? block_parts(g) : 1u;
-  if (WALK == kFixed) {
+  constexpr size_t bytes = WALK == kPlain ? 0 : (kBlockJ / 32) * (size_t)fx_warp_bytes<EX, WALK == kFixedVG>();
+  static_assert(bytes <= 226 * 1024, "an SM's shared memory, less the kernel's own");
+  const unsigned parts = WALK == kPlain ? 1u : block_parts(g);
+  if (WALK != kPlain) {
     static const cudaError_t ready = [] {
       // one split of L1 and shared memory for all of them: a kernel that wants
       // another than its predecessor's waits for the SM to drain (Dormand-Prince

@@ -145,11 +145,11 @@ __global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistA
       double acc[1] = {0.0};
       auto phase_a = [&](auto has_prev) {
         constexpr int EX = decltype(has_prev)::value;
-        unsigned char *ring = fx_smem + (tid >> 5) * fx_warp_bytes<EX>();
+        unsigned char *ring = fx_smem + (tid >> 5) * fx_warp_bytes<EX, false>();
         FxExtra<EX> ex;
         if (EX > 0) ex.p[0] = (j == 1) ? a.psi : a.work + (size_t)(j - 1) * G;
         for_my_strips(in, [&](int j0, int l0, int l1) {
-          walk_rows_fixed<ST, EX>(in, ex, ring, j0, l0, l1,
+          walk_rows_fixed<ST, false, EX>(in, ex, ring, j0, l0, l1,
                                   [&](int idx, int, double2 t, double2 uu, const double2 (&e)[1]) {
             double2 o = t;
             if (EX > 0) {
@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistA
 
 }  // namespace
 
-constexpr int kPersistSmem = (kBlockJ / 32) * fx_warp_bytes<1>();
+constexpr int kPersistSmem = (kBlockJ / 32) * fx_warp_bytes<1, false>();
 
 bool lanczos_persistent_fits(int stencil) {
   int dev = 0, coop = 0, nb = 0;
@@ -325,6 +325,8 @@ cudaError_t launch_lanczos_persistent(const Geometry &g, const OperatorView &op,
   in.ok = op.fx_ok;
   in.k = 0;
   in.E = 0.0;
+  in.rinv = nullptr;
+  in.d1c = 0.0;
   a.psi = psi;
   a.work = work;
   a.G = (size_t)g.N * (g.L + 1);

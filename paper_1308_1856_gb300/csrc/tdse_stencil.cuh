@@ -8,7 +8,6 @@
 namespace tdse_dev {
 namespace stencil {
 
-__device__ __forceinline__ double2 ldg2(const double2 *p) { return __ldg(p); }
 // The operand's load: read-only (non-coherent) path, or CG: from L2, for a
 // kernel whose other blocks rewrite the operand between its phases (an SM's
 // L1 is not kept coherent with another SM's stores).
@@ -33,8 +32,6 @@ struct StencilIn {
   const double *__restrict__ kappa;
   int N, L;
   double c1, c2, E;  // E: the field (length gauge) or A/c (velocity gauge)
-  double dscale;   // walkers with SCALED multiply the diagonal by it (the other terms
-                   // are scaled through c1, c2 and E by the caller)
   const double *__restrict__ rinv;   // velocity gauge: 1 / r_j
   double d1c;                        // velocity gauge: 1/(12 dr) (5-point) or 1/(2 dr) (3-point)
 };
@@ -45,27 +42,16 @@ struct StencilIn {
 template <int ST>
 __device__ __forceinline__ double2 d1_point(const StencilIn &in, const double2 *row, int i) {
   const double2 z = make_double2(0.0, 0.0);
-  const double2 m1 = (i >= 1) ? ldg2(row + i - 1) : z;
-  const double2 p1 = (i + 1 < in.N) ? ldg2(row + i + 1) : z;
+  const double2 m1 = (i >= 1) ? __ldcg(row + i - 1) : z;
+  const double2 p1 = (i + 1 < in.N) ? __ldcg(row + i + 1) : z;
   if (ST == 5) {
-    const double2 m2 = (i >= 2) ? ldg2(row + i - 2) : z;
-    const double2 p2 = (i + 2 < in.N) ? ldg2(row + i + 2) : z;
+    const double2 m2 = (i >= 2) ? __ldcg(row + i - 2) : z;
+    const double2 p2 = (i + 2 < in.N) ? __ldcg(row + i + 2) : z;
     return make_double2(
         __dmul_rn(in.d1c, __fma_rn(8.0, __dsub_rn(p1.x, m1.x), __dsub_rn(m2.x, p2.x))),
         __dmul_rn(in.d1c, __fma_rn(8.0, __dsub_rn(p1.y, m1.y), __dsub_rn(m2.y, p2.y))));
   }
   return make_double2(__dmul_rn(in.d1c, __dsub_rn(p1.x, m1.x)), __dmul_rn(in.d1c, __dsub_rn(p1.y, m1.y)));
-}
-
-// The operator scaled by s: every coefficient that multiplies the operand is
-// multiplied by s once (c1, c2, E here, the diagonal point by point by the
-// SCALED walker), so s H x costs one FP64 multiply per point instead of two.
-__device__ __forceinline__ StencilIn scaled(StencilIn in, double s) {
-  in.c1 = __dmul_rn(s, in.c1);
-  in.c2 = __dmul_rn(s, in.c2);
-  in.E = __dmul_rn(s, in.E);
-  in.dscale = s;
-  return in;
 }
 
 // (H x) at (l, i) from the register window; 15 FP64 instructions (5-point).
@@ -188,60 +174,47 @@ __device__ __forceinline__ void split2(double2 v, float2 &h, float2 &lo) {
   lo = make_float2(__double2float_rn(v.x - (double)h.x), __double2float_rn(v.y - (double)h.y));
 }
 
-// Walk rows [l0, l1) of column i and call f(i, idx, Hx, x_center).  PF > 0
-// asks L2 for the operand and diagonal rows PF rows ahead.
-// VG: velocity gauge, (A/c) p_z with p_z = -i [ (d/dr - l/r) kappa_l f_{l-1}
-// + (d/dr + (l+1)/r) kappa_{l+1} f_{l+1} ] (the partial-wave form of -i d/dz;
-// the paper prints the l/r terms with the opposite signs) in place of r E kappa.
-// CG: the operand's loads go to L2 (see ldx).
-template <int ST, int PF = 0, bool SCALED = false, bool VG = false, bool CG = false, typename F>
+// Walk rows [l0, l1) of column i (length gauge) and call f(i, idx, Hx, x_center).
+template <int ST, typename F>
 __device__ __forceinline__ void walk_rows(const StencilIn &in, int i, int l0, int l1, F &&f) {
-  static_assert(!(VG && CG), "the velocity gauge's first derivatives read through the read-only path");
   const int N = in.N, L = in.L;
   const double2 z = make_double2(0.0, 0.0);
   const double Er = __dmul_rn(in.E, in.rj[i]);
-  double2 prev = (l0 > 0) ? ldx<CG>(in.x + (size_t)(l0 - 1) * N + i) : z;
-  double2 cur = ldx<CG>(in.x + (size_t)l0 * N + i);
+  double2 prev = (l0 > 0) ? ldx<false>(in.x + (size_t)(l0 - 1) * N + i) : z;
+  double2 cur = ldx<false>(in.x + (size_t)l0 * N + i);
   double a_cur = __dmul_rn(in.kappa[l0], Er);
-  if (PF > 0)
-    for (int q = 1; q < PF && l0 + q < l1; ++q) {
-      prefetch_l2(in.x + (size_t)(l0 + q) * N + i);
-      prefetch_l2(in.diag + (size_t)(l0 + q) * N + i);
-    }
   for (int l = l0; l < l1; ++l) {
     const size_t idx = (size_t)l * N + i;
-    if (PF > 0 && l + PF < l1) {
-      prefetch_l2(in.x + idx + (size_t)PF * N);
-      prefetch_l2(in.diag + idx + (size_t)PF * N);
-    }
-    const double2 next = (l < L) ? ldx<CG>(in.x + idx + N) : z;
+    const double2 next = (l < L) ? ldx<false>(in.x + idx + N) : z;
     const double a_next = __dmul_rn(in.kappa[l + 1], Er);
-    const double d = SCALED ? __dmul_rn(in.dscale, __ldg(in.diag + idx)) : __ldg(in.diag + idx);
-    double2 t = h_point<ST, !VG, CG>(in, in.x + (size_t)l * N, i, d, prev, cur, next, a_cur, a_next);
-    if (VG) {
-      const double ri = __ldg(in.rinv + i);
-      double wx = 0.0, wy = 0.0;
-      if (l > 0) {
-        const double2 dp = d1_point<ST>(in, in.x + (size_t)(l - 1) * N, i);
-        const double k = in.kappa[l], lr = __dmul_rn((double)l, ri);
-        wx = __dmul_rn(k, __fma_rn(-lr, prev.x, dp.x));
-        wy = __dmul_rn(k, __fma_rn(-lr, prev.y, dp.y));
-      }
-      if (l < L) {
-        const double2 dn = d1_point<ST>(in, in.x + (size_t)(l + 1) * N, i);
-        const double k = in.kappa[l + 1], lr = __dmul_rn((double)(l + 1), ri);
-        wx = __fma_rn(k, __fma_rn(lr, next.x, dn.x), wx);
-        wy = __fma_rn(k, __fma_rn(lr, next.y, dn.y), wy);
-      }
-      // -i (A/c) w
-      t.x = __fma_rn(in.E, wy, t.x);
-      t.y = __fma_rn(-in.E, wx, t.y);
-    }
+    const double2 t = h_point<ST>(in, in.x + (size_t)l * N, i, __ldg(in.diag + idx), prev, cur, next, a_cur, a_next);
     f(i, idx, t, cur);
     prev = cur;
     cur = next;
     a_cur = a_next;
   }
+}
+
+// The velocity gauge's coupling at (l, i): (A/c) p_z with p_z = -i [ (d/dr - l/r)
+// kappa_l f_{l-1} + (d/dr + (l+1)/r) kappa_{l+1} f_{l+1} ] (the partial-wave form
+// of -i d/dz; the paper prints the l/r terms with the opposite signs).
+template <int ST>
+__device__ __forceinline__ double2 velocity_point(const StencilIn &in, int l, int i, double2 prev, double2 next) {
+  const double ri = __ldg(in.rinv + i);
+  double wx = 0.0, wy = 0.0;
+  if (l > 0) {
+    const double2 dp = d1_point<ST>(in, in.x + (size_t)(l - 1) * in.N, i);
+    const double k = in.kappa[l], lr = __dmul_rn((double)l, ri);
+    wx = __dmul_rn(k, __fma_rn(-lr, prev.x, dp.x));
+    wy = __dmul_rn(k, __fma_rn(-lr, prev.y, dp.y));
+  }
+  if (l < in.L) {
+    const double2 dn = d1_point<ST>(in, in.x + (size_t)(l + 1) * in.N, i);
+    const double k = in.kappa[l + 1], lr = __dmul_rn((double)(l + 1), ri);
+    wx = __fma_rn(k, __fma_rn(lr, next.x, dn.x), wx);
+    wy = __fma_rn(k, __fma_rn(lr, next.y, dn.y), wy);
+  }
+  return make_double2(__dmul_rn(in.E, wy), __dmul_rn(-in.E, wx));   // -i (A/c) w
 }
 
 // First derivative of the mixed operand's row starting at element `row`, at

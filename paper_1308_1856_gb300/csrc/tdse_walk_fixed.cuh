@@ -1,5 +1,5 @@
-// The FP64 operator's row walker in fixed point (tdse_fixed.cuh): H x of the
-// length gauge with the operand and the result in FP64.
+// The FP64 operator's row walker in fixed point (tdse_fixed.cuh): H x of either
+// gauge with the operand and the result in FP64.
 //
 // A warp owns a strip of kFxCols radial columns and walks it up the partial
 // waves.  Lane k holds columns j0 - 2 + 2k and the one after it, so lanes 0
@@ -17,6 +17,13 @@
 // errors relative to that value, put into the stiff centrifugal points, are
 // multiplied by the largest energies of the grid in every Krylov iteration
 // (measured: 3e-12 after one step where FP64 gives 6e-16).
+//
+// The velocity gauge couples the rows l -+ 1 through their first derivatives and
+// l/r terms: four products a part in place of two, of the derivative's integer
+// difference D and of the values, and the parts cross (-i).  D of a row is formed
+// once, when the row is converted, and kept in the lane's shared memory until
+// the row after next.  The length gauge's bound on the sums becomes
+// |mm| < (3.8 + 2 1.08 + 2 0.72) 2^60 < 2^63: D is held to 2^58.2.
 //
 // Blocks near the limits of FP64 (subnormal values, results that under- or
 // overflow) take separate conversions.  A row with an Inf or NaN in reach is
@@ -44,11 +51,13 @@ struct FxIn {
   const double *__restrict__ rj;
   const double *__restrict__ kappa;
   int N, L;
-  double c1, c2, E;
+  double c1, c2, E;                      // E: the field (length gauge) or A/c (velocity gauge)
   long long c1q, c2q;                    // c1, c2 against 2^ec
   int ec;
   int ok;                                // 0: the grid's coefficients do not fit, every row runs in FP64
   int k;                                 // the result is 2^k H x
+  const double *__restrict__ rinv;       // velocity gauge: 1 / r_j
+  double d1c;                            // velocity gauge: 1/(12 dr) (5-point) or 1/(2 dr) (3-point)
 };
 
 __device__ __forceinline__ double fx_double(uint64_t b) { return __longlong_as_double((long long)b); }
@@ -59,7 +68,7 @@ __device__ __forceinline__ double fx_diag_double(const FxIn &in, long long q) {
 }
 
 // 2^k (H x)(l, i) in FP64, from global memory (the rare rows; one point per call).
-template <int ST>
+template <int ST, bool VG>
 __device__ __noinline__ double2 h_point_fp64(const FxIn &in, int l, int i) {
   const double2 z = make_double2(0.0, 0.0);
   const size_t idx = (size_t)l * in.N + i;
@@ -69,13 +78,20 @@ __device__ __noinline__ double2 h_point_fp64(const FxIn &in, int l, int i) {
   s.L = in.L;
   s.c1 = in.c1;
   s.c2 = in.c2;
-  const double Er = __dmul_rn(in.E, in.rj[i]);
-  constexpr bool CG = true;
-  const double2 prev = l > 0 ? ldx<CG>(in.x + idx - in.N) : z;
-  const double2 next = l < in.L ? ldx<CG>(in.x + idx + in.N) : z;
-  const double2 t = h_point<ST, true, CG>(s, in.x + (size_t)l * in.N, i, fx_diag_double(in, in.diagq[idx]), prev,
-                                          ldx<CG>(in.x + idx), next, __dmul_rn(in.kappa[l], Er),
-                                          __dmul_rn(in.kappa[l + 1], Er));
+  s.E = in.E;
+  s.kappa = in.kappa;
+  s.rinv = in.rinv;
+  s.d1c = in.d1c;
+  const double Er = VG ? 0.0 : __dmul_rn(in.E, in.rj[i]);
+  const double2 prev = l > 0 ? __ldcg(in.x + idx - in.N) : z;
+  const double2 next = l < in.L ? __ldcg(in.x + idx + in.N) : z;
+  double2 t = h_point<ST, !VG, true>(s, in.x + (size_t)l * in.N, i, fx_diag_double(in, in.diagq[idx]), prev,
+                               __ldcg(in.x + idx), next, __dmul_rn(in.kappa[l], Er), __dmul_rn(in.kappa[l + 1], Er));
+  if (VG) {
+    const double2 v = velocity_point<ST>(s, l, i, prev, next);
+    t.x += v.x;
+    t.y += v.y;
+  }
   return make_double2(ldexp(t.x, in.k), ldexp(t.y, in.k));
 }
 
@@ -86,11 +102,12 @@ __device__ __noinline__ double2 h_point_fp64(const FxIn &in, int l, int i) {
 // also the diagonal and EX further vectors (the epilogue's).  While row l is
 // computed row l + 2 is in flight.  Register double buffering of the operand
 // alone left the epilogue's loads exposed (the top stall) and spilled.
+// In the velocity gauge a slot also keeps the row's D.
 constexpr int kFxSlots = 3;
-template <int EX>
-constexpr int fx_slot_bytes() { return (2 + 2 * EX + 1) * 32 * 16; }
-template <int EX>
-constexpr int fx_warp_bytes() { return kFxSlots * fx_slot_bytes<EX>(); }
+template <int EX, bool VG>
+constexpr int fx_slot_bytes() { return (2 + 2 * EX + 1 + (VG ? 2 : 0)) * 32 * 16; }
+template <int EX, bool VG>
+constexpr int fx_warp_bytes() { return kFxSlots * fx_slot_bytes<EX, VG>(); }
 
 template <int EX>
 struct FxExtra {
@@ -113,7 +130,9 @@ struct FxRow {
   int64_t X[2][2];   // [column][re, im]
   int e;             // their exponent field (0: zero)
   bool ok;           // every value of the strip finite (uniform)
+  int eD;            // velocity gauge: the exponent field of D (0: zero)
 };
+constexpr int kDShift = 6;   // D = (8 (x_{j+1} - x_{j-1}) - (x_{j+2} - x_{j-2})) / 2^6
 
 __device__ __forceinline__ uint32_t fx_field(double v) { return (uint32_t)__double2hiint(v) & kExpMask; }
 __device__ __forceinline__ int64_t fx_word(double v, uint32_t m) {
@@ -127,6 +146,7 @@ __device__ __forceinline__ void fx_convert(const double2 &v0, const double2 &v1,
   const uint32_t m = max(max(fx_field(v0.x), fx_field(v0.y)), max(fx_field(v1.x), fx_field(v1.y)));
   r.e = (int)(m >> 20);
   r.ok = true;
+  r.eD = 0;
   constexpr uint32_t kLo = (uint32_t)kExpSmall << 20;
   if (__all_sync(0xffffffffu, m - kLo < kExpMask - kLo)) {   // kLo <= m < kExpMask
     r.X[0][0] = fx_word(v0.x, m);
@@ -156,9 +176,9 @@ __device__ __forceinline__ int64_t fx_shfl_down(int64_t v) { return __shfl_down_
 
 // Walk rows [l0, l1) of the strip whose first output column is j0: calls
 // f(idx, column, 2^k (H x), x, extra values) for every output point.  Every lane of the
-// warp calls it with the same j0, l0, l1; ring: the warp's fx_warp_bytes<EX>()
+// warp calls it with the same j0, l0, l1; ring: the warp's fx_warp_bytes<EX, VG>()
 // of shared memory.  The operand and the extra vectors are read through L2.
-template <int ST, int EX, typename F>
+template <int ST, bool VG, int EX, typename F>
 __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX> &ex, unsigned char *ring, int j0,
                                                 int l0, int l1, F &&f) {
   const int N = in.N, L = in.L;
@@ -170,7 +190,7 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
   // the lane's parts of a slot: 16-byte columns x0, x1, extras, diagonal pair
   unsigned char *mine = ring + lane * 16;
   const unsigned smine = (unsigned)__cvta_generic_to_shared(mine);
-  constexpr int kSlot = fx_slot_bytes<EX>();
+  constexpr int kSlot = fx_slot_bytes<EX, VG>();
   int so = (l0 - 1) * N + j;                               // the lane's element of the next row to stage
   auto stage = [&](int r, int slot) {
     const unsigned d = smine + slot * kSlot;
@@ -200,50 +220,99 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
 #pragma unroll
         for (int q = 0; q < EX; ++q)
           e[q] = *reinterpret_cast<const double2 *>(mine + slot * kSlot + 1024 + 1024 * q + 512 * c);
-        f(l * N + j + c, j + c, h_point_fp64<ST>(in, l, j + c), slot_x(slot, c), e);
+        f(l * N + j + c, j + c, h_point_fp64<ST, VG>(in, l, j + c), slot_x(slot, c), e);
       }
   };
   // the tables' first entries are asked for before the rows, so that their
   // latencies overlap: a warp's share is often a single row
-  const double rj0 = have0 ? in.rj[j] : 0.0, rj1 = have1 ? in.rj[j + 1] : 0.0;
+  const double *rw = VG ? in.rinv : in.rj;
+  const double rj0 = have0 ? rw[j] : 0.0, rj1 = have1 ? rw[j + 1] : 0.0;
   const double kap0 = __ldg(in.kappa + l0);
   double kap = __ldg(in.kappa + l0 + 1);                   // kappa of the next row
   stage(l0 - 1, 0);
   stage(l0, 1);
   stage(l0 + 1, 2);
-  // the coupling w_j = E r_j of the lane's columns
+  // the coupling w_j = E r_j (velocity gauge: E / r_j) of the lane's columns
   const double w0 = __dmul_rn(in.E, rj0), w1 = __dmul_rn(in.E, rj1);
+  const double wd = VG ? __dmul_rn(in.E, in.d1c) : 0.0;    // velocity gauge: the derivative's coefficient
   const uint32_t wm = max(fx_field(w0), fx_field(w1));
-  const bool all_ok = in.ok && __all_sync(0xffffffffu, wm != kExpMask) != 0;
+  const bool all_ok = in.ok && __all_sync(0xffffffffu, max(wm, fx_field(wd)) != kExpMask) != 0;
   const int we = max((int)(wm >> 20), 1), ew = we - 1022;  // w = W 2^(ew - 60)
   const Limb W[2] = {fx_limbs(fx_small(w0, we)), fx_limbs(fx_small(w1, we))};
   const bool has_w = (W[0].h | W[0].l | W[1].h | W[1].l) != 0;
-  auto coupling = [&](double kappa, Limb (&a)[2]) {        // a = kappa_l w = A 2^(ew - 61)
-    const Limb kp = fx_limbs(fx_coef((uint64_t)__double_as_longlong(kappa), 0));
-    a[0] = fx_limbs(fx_coef_product(kp, W[0]));
-    a[1] = fx_limbs(fx_coef_product(kp, W[1]));
+  // length gauge: a = kappa_l w = A 2^(ew - 61); velocity gauge: a = kappa_l l w =
+  // A 2^(ew + el - 61) with 2^el > l, and d = kappa_l E d1c = D 2^(ed - 61)
+  const int wde = max((int)(fx_field(wd) >> 20), 1), ed = wde - 1022;
+  const Limb WD = fx_limbs(VG ? fx_small(wd, wde) : 0);
+  const bool has_d = (WD.h | WD.l) != 0;
+  auto coupling = [&](int l, double kappa, Limb (&a)[2], Limb &d, int &el) {
+    const int64_t K = fx_coef((uint64_t)__double_as_longlong(kappa), 0);
+    Limb kp = fx_limbs(K);
+    if (VG) {
+      d = fx_limbs(fx_coef_product(kp, WD));
+      el = 32 - __clz(l | 1);
+      // K l / 2^el, odd: no limb is -2^31, so that the next row can negate it
+      kp = fx_limbs((int64_t)(__umul64hi((uint64_t)K << 2, (uint64_t)l << (64 - el)) >> 2));
+    }
+#pragma unroll
+    for (int c = 0; c < 2; ++c) a[c] = fx_limbs(fx_coef_product(kp, W[c]) | (VG ? 1 : 0));
+  };
+  // velocity gauge: the differences D of a row, against the largest exponent of
+  // the lane's and its neighbours' columns, into the slot
+  auto differences = [&](FxRow &r, int slot) {
+    const int eU = __shfl_up_sync(0xffffffffu, r.e, 1), eD = __shfl_down_sync(0xffffffffu, r.e, 1);
+    r.eD = max(r.e, max(eU, eD));
+    const int sC = min(r.eD - r.e, 63), sU = min(r.eD - eU, 63), sD = min(r.eD - eD, 63);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const int64_t lB = fx_shfl_up(r.X[1][p]) >> sU, rA = fx_shfl_down(r.X[0][p]) >> sD;
+      const int64_t A = r.X[0][p] >> sC, B = r.X[1][p] >> sC;
+      longlong2 D;
+      constexpr int64_t half = (int64_t)1 << (kDShift - 1);
+      if (ST == 5) {
+        const int64_t lA = fx_shfl_up(r.X[0][p]) >> sU, rB = fx_shfl_down(r.X[1][p]) >> sD;
+        D.x = (B - lB - ((rA - lA) >> 3) + half / 8) >> (kDShift - 3);
+        D.y = (rA - A - ((rB - lB) >> 3) + half / 8) >> (kDShift - 3);
+      } else {
+        D.x = (B - lB + half) >> kDShift;
+        D.y = (rA - A + half) >> kDShift;
+      }
+      *reinterpret_cast<longlong2 *>(mine + slot * kSlot + kSlot - 1024 + 512 * p) = D;
+    }
   };
   const Limb k1 = fx_limbs(in.c1q), k2 = fx_limbs(in.c2q);
-  Limb acur[2], anext[2];
-  coupling(kap0, acur);
+  Limb acur[2], anext[2], dcur = {0, 0}, dnext = {0, 0};
+  int lcur = 0, lnext = 0;
+  coupling(l0, kap0, acur, dcur, lcur);
+  if (VG)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) acur[c] = Limb{-acur[c].h, -acur[c].l};
   FxRow prev, cur, next;
   cp_async_wait<1>();
   fx_convert(slot_x(0, 0), slot_x(0, 1), prev);
   fx_convert(slot_x(1, 0), slot_x(1, 1), cur);
+  if (VG) {
+    differences(prev, 0);
+    differences(cur, 1);
+  }
   stage(l0 + 2, 0);
   int s0 = 1, s1 = 2;                                      // slots of rows l and l + 1
 #pragma unroll 1
   for (int l = l0; l < l1; ++l) {
     cp_async_wait<1>();
     fx_convert(slot_x(s1, 0), slot_x(s1, 1), next);
-    coupling(kap, anext);
+    if (VG) differences(next, s1);
+    coupling(l + 1, kap, anext, dnext, lnext);
     if (l + 1 < l1) kap = __ldg(in.kappa + l + 2);
     const int eU = __shfl_up_sync(0xffffffffu, cur.e, 1), eD = __shfl_down_sync(0xffffffffu, cur.e, 1);
     // exponent of the point's sum: the largest of its terms', coefficients included
     const int eb = max(cur.e, max(eU, eD));
-    const int EP = (prev.e && has_w) ? prev.e + ew : kNone;
-    const int EN = (next.e && has_w) ? next.e + ew : kNone;
-    const int Em = max(eb ? eb + in.ec : kNone, max(EP, EN));
+    const int EP = (prev.e && has_w) ? prev.e + ew + lcur : kNone;
+    const int EN = (next.e && has_w) ? next.e + ew + lnext : kNone;
+    int Em = max(eb ? eb + in.ec : kNone, max(EP, EN));
+    const int EPD = (VG && prev.eD && has_d) ? prev.eD + ed + kDShift : kNone;
+    const int END = (VG && next.eD && has_d) ? next.eD + ed + kDShift : kNone;
+    if (VG) Em = max(Em, max(EPD, END));
     if (all_ok && prev.ok && cur.ok && next.ok) {
       const unsigned char *body = mine + s0 * kSlot;
       const longlong2 dq = *reinterpret_cast<const longlong2 *>(body + 1024 + 1024 * EX);
@@ -251,6 +320,8 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
       const int eL = Em == kNone ? 0 : Em - in.ec;
       const int sC = min(eL - cur.e, 63), sU = min(eL - eU, 63), sD = min(eL - eD, 63);
       const int sP = min(Em - EP, 63), sN = min(Em - EN, 63);
+      const int sPD = min(Em - EPD, 63), sND = min(Em - END, 63);
+      const unsigned char *pd = mine + (kFxSlots - s0 - s1) * kSlot + kSlot - 1024, *nd = mine + s1 * kSlot + kSlot - 1024;
       const int E = Em + in.k;
       int64_t V[2][2];
       // the sums without (D = false) or with the diagonal's term
@@ -269,8 +340,20 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
             int64_t hh = 0, mm = kHalf;
             fx_mac(fx_limbs(c == 0 ? lB + B : A + rA), k1, hh, mm);
             if (ST == 5) fx_mac(fx_limbs(c == 0 ? lA + rA : lB + rB), k2, hh, mm);
-            fx_mac(fx_limbs(prev.X[c][p] >> sP), acur[c], hh, mm);
-            fx_mac(fx_limbs(next.X[c][p] >> sN), anext[c], hh, mm);
+            if (!VG) {
+              fx_mac(fx_limbs(prev.X[c][p] >> sP), acur[c], hh, mm);
+              fx_mac(fx_limbs(next.X[c][p] >> sN), anext[c], hh, mm);
+            } else {   // -i (A/c) w: the real part takes +w's imaginary part, the imaginary part -w's real part
+              int64_t ch = 0, cm = 0;
+              const int64_t *dp = reinterpret_cast<const int64_t *>(pd + 512 * (1 - p)) + c;
+              const int64_t *dn = reinterpret_cast<const int64_t *>(nd + 512 * (1 - p)) + c;
+              fx_mac(fx_limbs(prev.X[c][1 - p] >> sP), acur[c], ch, cm);
+              fx_mac(fx_limbs(next.X[c][1 - p] >> sN), anext[c], ch, cm);
+              fx_mac(fx_limbs(*dp >> sPD), dcur, ch, cm);
+              fx_mac(fx_limbs(*dn >> sND), dnext, ch, cm);
+              hh = p == 0 ? hh + ch : hh - ch;
+              mm = p == 0 ? mm + cm : mm - cm;
+            }
             if (decltype(with_d)::value) fx_mac(fx_limbs(c == 0 ? A : B), fx_limbs(c == 0 ? dq.x : dq.y), hh, mm);
             V[c][p] = fx_value(hh, mm);
           }
@@ -324,8 +407,10 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
     s1 = s2;
     prev = cur;
     cur = next;
-    acur[0] = anext[0];
-    acur[1] = anext[1];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) acur[c] = VG ? Limb{-anext[c].h, -anext[c].l} : anext[c];
+    dcur = dnext;
+    lcur = lnext;
   }
   cp_async_wait<0>();   // the ring is free for the next call
 }
