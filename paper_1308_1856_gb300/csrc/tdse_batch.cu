@@ -34,6 +34,7 @@
 #include "tdse_internal.cuh"
 #include "tdse_stencil.cuh"
 #include "tdse_walk_fixed.cuh"
+#include "tdse_combine_fixed.cuh"
 
 namespace tdse_dev {
 namespace {
@@ -58,7 +59,6 @@ constexpr int kChunkPts = 512;
 constexpr int kFxThreads = 128;              // threads of a block of the fixed-point stencil kernel
 constexpr int kFxBlocksPerSM = 4;            // 128 registers a thread
 constexpr int kFxMaxRows = 32;               // segments of a chunk at most (16: 5% slower on large batches)
-constexpr int kCombinePts = 2;               // points per lane whose Krylov loads the combines overlap
 constexpr int kMixedCombinePts = 2;          // the same for the mixed combine, two vectors per round
 
 __device__ __forceinline__ double field_of(const BatchDev &B, int inst) {
@@ -442,66 +442,41 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
 }
 
 // psi_new = sum_{j<k} coef_j U_j, mask (unless mask_on is 0: imaginary
-// time), ||psi_new|| (FP64).
-__global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
-    bt_combine_fp64(BatchDev B, ChunkList cl, int mask_on) {
-  // the chunk's coefficients, one copy per warp
-  __shared__ double2 wcoef[kElemThreads / 32][kMaxKrylov];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+// time), ||psi_new|| (FP64).  The sum in fixed point (tdse_combine_fixed.cuh), 128
+// registers a thread for its loads in flight.
+__global__ void __launch_bounds__(kElemThreads, 1) bt_combine_fp64(BatchDev B, ChunkList cl, int mask_on) {
+  __shared__ CbTable tabs[kElemThreads / 32];   // the instance's coefficients, one copy per warp
+  const int lane = threadIdx.x & 31;
+  CbTable &tab = tabs[threadIdx.x >> 5];
   for_elem_chunks(B, cl, [&](int inst, const BatchInst &I, int ci, int n, ChunkSums &sums) {
-    LanczosScalars *ls = B.ls + inst;
-    const long long G = (long long)I.N * (I.L + 1);
+    const unsigned N = (unsigned)I.N, G = N * (unsigned)(I.L + 1);
     double2 *psi = I.psi;
     const double2 *U1 = I.work + G;
-    const double *mask = I.mask;
-    const int k = ls->kdim;
     __syncwarp();
-    if (lane < k) wcoef[wib][lane] = ls->coef[lane];
-    __syncwarp();
-    const double2 c0 = wcoef[wib][0];
+    cb_setup(tab, B.ls + inst);
     for (int q = 0; q < n; ++q) {
       double acc = 0.0;
-      // kCombinePts points at a time, Krylov vector by Krylov vector
-      chunk_groups_of<kCombinePts>(I, ci + q, [&](const size_t (&ix)[kCombinePts], const int (&iq)[kCombinePts], int nq) {
-        double ox[kCombinePts], oy[kCombinePts];
-#pragma unroll
-        for (int q = 0; q < kCombinePts; ++q) {
-          if (q < nq) {
-            const double2 u0 = psi[ix[q]];
-            ox[q] = __fma_rn(c0.x, u0.x, __dmul_rn(-c0.y, u0.y));
-            oy[q] = __fma_rn(c0.x, u0.y, __dmul_rn(c0.y, u0.x));
+      const unsigned base = (unsigned)(ci + q) * kChunkPts, end = min(G, base + kChunkPts);
+      unsigned i = (base + lane) % N;
+      for (unsigned first = base; first < end; first += 32) {
+        const unsigned idx = first + lane;
+        const bool ok = idx < end;
+        double2 o = cb_sum(tab, [&](int j) {
+          return ok ? (j == 0 ? psi[idx] : U1[(size_t)(j - 1) * G + idx]) : make_double2(0.0, 0.0);
+        });
+        if (ok) {
+          if (mask_on && (int)i >= I.mask_start) {
+            const double mv = I.mask[i];
+            o.x = __dmul_rn(mv, o.x);
+            o.y = __dmul_rn(mv, o.y);
           }
+          psi[idx] = o;
+          acc = __fma_rn(o.x, o.x, acc);
+          acc = __fma_rn(o.y, o.y, acc);
         }
-        for (int jj = 1; jj < k; ++jj) {
-          double2 u[kCombinePts];
-#pragma unroll
-          for (int q = 0; q < kCombinePts; ++q)
-            if (q < nq) u[q] = U1[(size_t)(jj - 1) * G + ix[q]];
-          const double2 c = wcoef[wib][jj];
-#pragma unroll
-          for (int q = 0; q < kCombinePts; ++q) {
-            if (q < nq) {
-              ox[q] = __fma_rn(c.x, u[q].x, ox[q]);
-              ox[q] = __fma_rn(-c.y, u[q].y, ox[q]);
-              oy[q] = __fma_rn(c.x, u[q].y, oy[q]);
-              oy[q] = __fma_rn(c.y, u[q].x, oy[q]);
-            }
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < kCombinePts; ++q) {
-          if (q < nq) {
-            if (mask_on && iq[q] >= I.mask_start) {
-              const double mv = mask[iq[q]];
-              ox[q] = __dmul_rn(mv, ox[q]);
-              oy[q] = __dmul_rn(mv, oy[q]);
-            }
-            psi[ix[q]] = make_double2(ox[q], oy[q]);
-            acc = __fma_rn(ox[q], ox[q], acc);
-            acc = __fma_rn(oy[q], oy[q], acc);
-          }
-        }
-      });
+        i += 32;
+        while (i >= N) i -= N;
+      }
       sums.set(q, acc);
     }
   }, [&](int inst, double s) {
@@ -1903,7 +1878,7 @@ int Engine::enqueue_step(const BatchDev &B, const Segment &sg, int &count) {
     if (steps_tab()) bt_combine_mixed<true><<<egrid, kElemThreads, 0, stream>>>(B, all);   // per-step observables read psi
     else bt_combine_mixed<false><<<egrid, kElemThreads, 0, stream>>>(B, all);
   }
-  else bt_combine_fp64<<<egrid, kElemThreads, 0, stream>>>(B, all, run_imag ? 0 : 1);
+  else bt_combine_fp64<<<(unsigned)sms, kElemThreads, 0, stream>>>(B, all, run_imag ? 0 : 1);
   prof_end(pc);
   ++count;
   EN_CUDA(cudaGetLastError(), "batch combine");

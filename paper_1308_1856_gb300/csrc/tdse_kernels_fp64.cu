@@ -29,6 +29,7 @@
 #include "tdse_device_common.cuh"
 #include "tdse_stencil.cuh"
 #include "tdse_walk_fixed.cuh"
+#include "tdse_combine_fixed.cuh"
 #include "tdse_internal.cuh"
 
 namespace tdse_dev {
@@ -378,41 +379,38 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
 
 // psi_new = sum_{j<k} coef_j U_j  (U_0 = psi, read and written in place by
 // the same thread), then the absorber mask and ||psi_new||^2 for the next step.
-__global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
+// The sum in fixed point (tdse_combine_fixed.cuh), 128 registers a thread for
+// its loads in flight.
+__global__ void __launch_bounds__(kElemThreads, 1)
     lanczos_combine_kernel(size_t G, int N, double2 *psi, const double2 *__restrict__ work,
                            size_t stride, const double *__restrict__ mask, int mask_start,
                            Reduction *red, LanczosScalars *ls, int *status) {
   __shared__ double sh[kElemThreads / 32 + 1];
-  __shared__ double2 coef[kMaxKrylov];
-  __shared__ int s_k;
+  __shared__ CbTable tab;
   pdl_wait();
-  if (threadIdx.x < kMaxKrylov) coef[threadIdx.x] = ls->coef[threadIdx.x];
-  if (threadIdx.x == 0) s_k = ls->kdim;
+  if (threadIdx.x < 32) cb_setup(tab, ls);
   __syncthreads();
-  const int k = s_k;
   double acc = 0.0;
-  for_my_groups(G, [&](size_t idx) {
-    const double2 u0 = psi[idx];
-    double ox = __fma_rn(coef[0].x, u0.x, __dmul_rn(-coef[0].y, u0.y));
-    double oy = __fma_rn(coef[0].x, u0.y, __dmul_rn(coef[0].y, u0.x));
-    for (int jj = 1; jj < k; ++jj) {
-      const double2 u = work[(size_t)(jj - 1) * stride + idx];
-      const double2 c = coef[jj];
-      ox = __fma_rn(c.x, u.x, ox);
-      ox = __fma_rn(-c.y, u.y, ox);
-      oy = __fma_rn(c.x, u.y, oy);
-      oy = __fma_rn(c.y, u.x, oy);
-    }
+  const int lane = threadIdx.x & 31;
+  long long g0, g1;
+  warp_range((long long)((G + 31) >> 5), g0, g1);
+  for (long long gi = g0; gi < g1; ++gi) {
+    const size_t idx = (size_t)gi * 32 + lane;
+    const bool ok = idx < G;
+    double2 o = cb_sum(tab, [&](int j) {
+      return ok ? (j == 0 ? psi[idx] : work[(size_t)(j - 1) * stride + idx]) : make_double2(0.0, 0.0);
+    });
+    if (!ok) continue;
     const int jr = (int)((unsigned)idx % (unsigned)N);
     if (jr >= mask_start) {
       const double mv = mask[jr];
-      ox = __dmul_rn(mv, ox);
-      oy = __dmul_rn(mv, oy);
+      o.x = __dmul_rn(mv, o.x);
+      o.y = __dmul_rn(mv, o.y);
     }
-    psi[idx] = make_double2(ox, oy);
-    acc = __fma_rn(ox, ox, acc);
-    acc = __fma_rn(oy, oy, acc);
-  });
+    psi[idx] = o;
+    acc = __fma_rn(o.x, o.x, acc);
+    acc = __fma_rn(o.y, o.y, acc);
+  }
   pdl_trigger();
   if (publish_block_partial(acc, red, sh)) {
     const double s = reduce_partials(red, gridDim.x, sh);
@@ -766,7 +764,7 @@ cudaError_t launch_lanczos_combine(const Geometry &g, const OperatorView &op, in
                                    cudaStream_t st) {
   (void)m;
   const size_t G = (size_t)g.N * (g.L + 1);
-  const cudaError_t e = launch_pdl(lanczos_combine_kernel, elem_blocks(g), kElemThreads, 0, st, G, g.N, psi, work,
+  const cudaError_t e = launch_pdl(lanczos_combine_kernel, (unsigned)g.sms, kElemThreads, 0, st, G, g.N, psi, work,
                                    stride, op.mask, op.mask_start, red, ls, status);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -33,6 +33,7 @@
 #include "tdse_small_expm.cuh"
 #include "tdse_stencil.cuh"
 #include "tdse_walk_fixed.cuh"
+#include "tdse_combine_fixed.cuh"
 
 namespace tdse_dev {
 namespace {
@@ -119,8 +120,7 @@ __global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistA
   __shared__ double sh[kBlockJ / 32 + 1];
   __shared__ double s_sigma[kMaxKrylov + 1], s_ratio[kMaxKrylov + 1], s_acoef[kMaxKrylov];
   __shared__ double s_g[kMaxKrylov];   // step_scale's g_j
-  __shared__ double2 s_coef[kMaxKrylov];
-  __shared__ int s_k;
+  __shared__ CbTable tab;
   extern __shared__ __align__(16) unsigned char fx_smem[];
   constexpr int V = kElemBlocksPerSM;
   static_assert(kElemThreads == kBlockJ, "a block stands for whole elementwise blocks");
@@ -228,44 +228,32 @@ __global__ void __launch_bounds__(kBlockJ, 1) lanczos_persistent_kernel(PersistA
     // ---- the small exponential: block 0's first kEx threads
     if (lead && tid < kEx) expm_body(a.m, a.dt, a.ls, false, ExNamedSync{});
     grid_sync(a.bar, gridDim.x, a.status);
-    if (tid < kMaxKrylov) s_coef[tid] = __ldcg(&a.ls->coef[tid]);
-    if (tid == 0) s_k = __ldcg(&a.ls->kdim);
+    if (tid < 32) cb_setup(tab, a.ls);
     __syncthreads();
     // ---- the combine (the lanczos_combine kernel's arithmetic and work split)
-    const int k = s_k;
     const int N = a.in.N;
     const double2 *U1 = a.work + G;
-    double accn[V];
-#pragma unroll 1
-    for (int q = 0; q < V; ++q) {
-      double acc = 0.0;
+    double accn[1] = {0.0};
+    {
       long long g0, g1;
-      elem_range<V>(q, (long long)((G + 31) >> 5), g0, g1);
+      elem_range<1>(0, (long long)((G + 31) >> 5), g0, g1);
       for (long long gi = g0; gi < g1; ++gi) {
         const size_t idx = (size_t)gi * 32 + lane;
-        if (idx >= G) continue;
-        const double2 u0 = __ldcg(a.psi + idx);
-        double ox = __fma_rn(s_coef[0].x, u0.x, __dmul_rn(-s_coef[0].y, u0.y));
-        double oy = __fma_rn(s_coef[0].x, u0.y, __dmul_rn(s_coef[0].y, u0.x));
-        for (int jj = 1; jj < k; ++jj) {
-          const double2 v = __ldcg(U1 + (size_t)(jj - 1) * G + idx);
-          const double2 cc = s_coef[jj];
-          ox = __fma_rn(cc.x, v.x, ox);
-          ox = __fma_rn(-cc.y, v.y, ox);
-          oy = __fma_rn(cc.x, v.y, oy);
-          oy = __fma_rn(cc.y, v.x, oy);
-        }
+        const bool ok = idx < G;
+        double2 o = cb_sum(tab, [&](int j) {
+          return ok ? __ldcg(j == 0 ? a.psi + idx : U1 + (size_t)(j - 1) * G + idx) : make_double2(0.0, 0.0);
+        });
+        if (!ok) continue;
         const int jr = (int)((unsigned)idx % (unsigned)N);
         if (jr >= a.mask_start) {
           const double mv = a.mask[jr];
-          ox = __dmul_rn(mv, ox);
-          oy = __dmul_rn(mv, oy);
+          o.x = __dmul_rn(mv, o.x);
+          o.y = __dmul_rn(mv, o.y);
         }
-        a.psi[idx] = make_double2(ox, oy);
-        acc = __fma_rn(ox, ox, acc);
-        acc = __fma_rn(oy, oy, acc);
+        a.psi[idx] = o;
+        accn[0] = __fma_rn(o.x, o.x, accn[0]);
+        accn[0] = __fma_rn(o.y, o.y, accn[0]);
       }
-      accn[q] = acc;
     }
     const double sn2 = grid_reduce(accn, a.rp + par, sh, a);
     par ^= 1;
