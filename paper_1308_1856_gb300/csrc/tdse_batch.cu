@@ -1593,8 +1593,7 @@ constexpr size_t kGraphCache = 8;    // captured step graphs kept across runs
 template <int ST, bool VG, int EX>
 cudaError_t launch_fixed_ex(unsigned grid, cudaStream_t st, const BatchDev &B, const ChunkList &cl, int j) {
   constexpr int bytes = (kFxThreads / 32) * fx_warp_bytes<EX, VG>();
-  static const cudaError_t ready = cudaFuncSetAttribute(bt_lanczos_a_fixed<ST, VG, EX>,
-                                                        cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const cudaError_t ready = kernel_ready<bt_lanczos_a_fixed<ST, VG, EX>>(bytes);
   if (ready != cudaSuccess) return ready;
   bt_lanczos_a_fixed<ST, VG, EX><<<grid, kFxThreads, bytes, st>>>(B, cl, j);
   return cudaGetLastError();

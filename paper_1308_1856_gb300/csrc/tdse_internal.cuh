@@ -13,6 +13,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -253,6 +254,22 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
+}
+
+// The largest dynamic shared memory of a kernel (and its split of L1 and shared
+// memory, if given) set once per kernel and device.
+template <auto KERN>
+cudaError_t kernel_ready(int bytes, int carveout = -1) {
+  static std::atomic<unsigned long long> set{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0;
+  if (set.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  if (carveout >= 0) e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout, carveout);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) set.fetch_or(bit, std::memory_order_release);
+  return e;
 }
 
 // A kernel's launch shape, or why it could not be set up.

@@ -572,21 +572,17 @@ inline unsigned block_parts(const Geometry &g) {
 }
 
 // A stencil kernel's launch: its rings are dynamic shared memory, raised above
-// the 48 KB default once per instantiation (kern is a compile-time constant).
+// the 48 KB default once per instantiation and device.
 template <auto KERN, int WALK, int EX>
 OpLaunch op_launch(const Geometry &g) {
   constexpr size_t bytes = WALK == kPlain ? 0 : (kBlockJ / 32) * (size_t)fx_warp_bytes<EX, WALK == kFixedVG>();
   static_assert(bytes <= 226 * 1024, "an SM's shared memory, less the kernel's own");
   const unsigned parts = WALK == kPlain ? 1u : block_parts(g);
   if (WALK != kPlain) {
-    static const cudaError_t ready = [] {
-      // one split of L1 and shared memory for all of them: a kernel that wants
-      // another than its predecessor's waits for the SM to drain (Dormand-Prince
-      // on 50,000 points: 279 us for four steps, 233 with one split)
-      const cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                                 cudaSharedmemCarveoutMaxShared);
-      return e != cudaSuccess ? e : cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    }();
+    // one split of L1 and shared memory for all of them: a kernel that wants
+    // another than its predecessor's waits for the SM to drain (Dormand-Prince
+    // on 50,000 points: 279 us for four steps, 233 with one split)
+    const cudaError_t ready = kernel_ready<KERN>((int)bytes, cudaSharedmemCarveoutMaxShared);
     if (ready != cudaSuccess) return OpLaunch{0, 0, 0, ready};
   }
   return OpLaunch{stencil_blocks<WALK>(g), kBlockJ / parts, bytes / parts, cudaSuccess};
