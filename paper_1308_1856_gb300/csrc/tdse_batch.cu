@@ -14,8 +14,8 @@
 //
 // Algorithm per instance: the Lanczos propagator of the single-instance path
 // (Appendix "Lanczos methods" of arXiv 1308.1856): U_0 = psi,
-// z = sigma_j H U_j - ratio_j U_{j-1}, alpha_j = sigma_j Re<U_j, z>,
-// U_{j+1} = z - alpha_j sigma_j U_j, beta_j = ||U_{j+1}||, then
+// z = s_j H U_j - ratio_j U_{j-1} with s_j near sigma_j (step_scale), alpha_j from Re<U_j, z>,
+// U_{j+1} = z - alpha_j s_j U_j, beta_j from ||U_{j+1}||, then
 // c = exp(-i T dt) e_1 and psi_new = sum_j coef_j U_j, mask, ||psi_new||.
 #include <cuda_runtime.h>
 
