@@ -736,10 +736,10 @@ int rk4_steps(tdse *h, double dt, long nsteps) {
 // (lanczos_persistent_kernel), bitwise the multi-launch path's result.
 int persistent_steps(tdse *h, int m, double dt, long nsteps, bool *done) {
   *done = false;
-  // AUTO keeps the multi-launch path: measured on the at-scale grid, one
-  // cooperative launch per call is slower (a Lanczos-12 step 0.711 ms against
-  // 0.656 ms), its phases reading the Krylov vectors from L2 rather than L1
-  // and its 2m + 1 grid barriers costing about what the launches did
+  // AUTO keeps the multi-launch path: measured on 512,000 points, one
+  // cooperative launch per call is slower (a Lanczos-12 step 0.384 ms against
+  // 0.369 ms), its 2m + 1 grid barriers costing about what the launches do and
+  // its elementwise phases running on half the warps
   if (h->persist_mode != TDSE_SMALL_GRID_FORCE || nsteps < 1 || hooks_on(h) || h->opts.precision != TDSE_FP64 ||
       h->g.gauge != 0)
     return TDSE_OK;
