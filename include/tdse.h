@@ -278,6 +278,15 @@ int tdse_flux_read(tdse_t *h, double *flux, double *yield, double *density, doub
 int tdse_check_guards(tdse_t *h);
 
 /*
+ * Debug: a failing allocation.  When the environment variable TDSE_FAIL_ALLOC
+ * names a buffer of the handle at tdse_create ("work", "dip_partials", ...),
+ * the first allocation of it is reported as out of memory, once.  Where the
+ * handle can give memory back (the fixed-point copy of its diagonal, 8 bytes a
+ * point, without which the FP64 operator runs in FP64) it does and tries
+ * again; otherwise the call returns TDSE_ERR_OOM.
+ */
+
+/*
  * Checkpoint and resume.  A checkpoint holds the state, the time, the cached
  * norm the next Lanczos step starts from and, if the flux is set up, its
  * current values and time integrals: loading it into a handle of the same

@@ -69,6 +69,7 @@ struct tdse {
   // debug guard bands (TDSE_GUARD_BYTES at create): every device buffer of the
   // handle sits between two bands of 0xff bytes that tdse_check_guards verifies
   size_t guard = 0;
+  std::string fail_alloc;   // debug (TDSE_FAIL_ALLOC at create): the buffer whose next allocation fails once
   struct Alloc { char *base; void *user; size_t bytes; const char *name; };
   std::vector<Alloc> allocs;
   // bookkeeping
@@ -156,7 +157,9 @@ int check_usable(tdse *h) {
   return TDSE_OK;
 }
 
-OperatorView view(const tdse *h) {
+// Taken anew for every launch: an allocation between two launches may give the
+// encoded diagonal's memory back (dmalloc).
+OperatorView view(const tdse *h, bool plain = false) {
   OperatorView op;
   op.diag = h->diag;
   op.rj = h->rj;
@@ -169,6 +172,7 @@ OperatorView view(const tdse *h) {
   op.c2q = h->c2q;
   op.fx_ec = h->fx_ec;
   op.fx_ok = h->diagq ? 1 : 0;
+  op.plain = plain;
   return op;
 }
 
@@ -198,8 +202,10 @@ template <typename T>
 cudaError_t dmalloc(tdse *h, T **p, size_t bytes, const char *name) {
   char *base = nullptr;
   const size_t g = h->guard;
-  cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&base), bytes + 2 * g);
-  if (e != cudaSuccess && h->diagq) {   // memory is short: the encoded diagonal is a copy the handle can do without
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (h->fail_alloc == name) h->fail_alloc.clear();
+  else e = cudaMalloc(reinterpret_cast<void **>(&base), bytes + 2 * g);
+  if (e == cudaErrorMemoryAllocation && h->diagq) {   // memory is short: the encoded diagonal is a copy the handle can do without
     cudaGetLastError();
     dfree(h, h->diagq);
     h->diagq = nullptr;
@@ -512,7 +518,6 @@ int mx_taylor_steps(tdse *h, int P, double dt, long nsteps) {
   if (rc) return rc;
   rc = refresh_split(h, false);
   if (rc) return rc;
-  const OperatorView op = view(h);
   const MixedView mv = mview(h);
   const size_t G = npts(h);
   float2 *wb[2] = {h->mwork, h->mwork + G};
@@ -525,7 +530,7 @@ int mx_taylor_steps(tdse *h, int P, double dt, long nsteps) {
       const bool last = (k == 1);
       float2 *w_out = last ? nullptr : wb[(P - k) & 1];
       TDSE_LAUNCH(h, TDSE_K_TAYLOR_STAGE,
-                  launch_mx_taylor_stage(h->g, mv, op, E, dt / (double)k, split_hi(h, cur), split_lo(h, cur),
+                  launch_mx_taylor_stage(h->g, mv, view(h), E, dt / (double)k, split_hi(h, cur), split_lo(h, cur),
                                          w_in, w_out, last, h->psi, split_hi(h, nxt), split_lo(h, nxt),
                                          h->stream),
                   "mixed taylor stage");
@@ -544,7 +549,6 @@ int mx_rk4_steps(tdse *h, double dt, long nsteps) {
   if (rc) return rc;
   rc = refresh_split(h, false);
   if (rc) return rc;
-  const OperatorView op = view(h);
   const MixedView mv = mview(h);
   const size_t G = npts(h);
   float2 *ka = h->mwork, *kb = h->mwork + G, *ahi = h->mwork + 2 * G, *alo = h->mwork + 3 * G;
@@ -554,10 +558,10 @@ int mx_rk4_steps(tdse *h, double dt, long nsteps) {
     const double E1 = coupling_at(h, tn), E2 = coupling_at(h, tn + 0.5 * dt), E4 = coupling_at(h, tn + dt);
     const int cur = h->split_cur, nxt = 1 - cur;
     float2 *hi = split_hi(h, cur), *lo = split_lo(h, cur);
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, op, E1, 1, dt, hi, lo, nullptr, ka, ahi, alo, h->psi, nullptr, nullptr, h->stream), "mixed rk 1");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, op, E2, 2, dt, hi, lo, ka, kb, ahi, alo, h->psi, nullptr, nullptr, h->stream), "mixed rk 2");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, op, E2, 3, dt, hi, lo, kb, ka, ahi, alo, h->psi, nullptr, nullptr, h->stream), "mixed rk 3");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, op, E4, 4, dt, hi, lo, ka, nullptr, ahi, alo, h->psi, split_hi(h, nxt), split_lo(h, nxt), h->stream), "mixed rk 4");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, view(h), E1, 1, dt, hi, lo, nullptr, ka, ahi, alo, h->psi, nullptr, nullptr, h->stream), "mixed rk 1");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, view(h), E2, 2, dt, hi, lo, ka, kb, ahi, alo, h->psi, nullptr, nullptr, h->stream), "mixed rk 2");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, view(h), E2, 3, dt, hi, lo, kb, ka, ahi, alo, h->psi, nullptr, nullptr, h->stream), "mixed rk 3");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_mx_rk_stage(h->g, mv, view(h), E4, 4, dt, hi, lo, ka, nullptr, ahi, alo, h->psi, split_hi(h, nxt), split_lo(h, nxt), h->stream), "mixed rk 4");
     h->split_cur = nxt;
     TDSE_HOOK(h, t0 + (double)(n + 1) * dt, dt);
   }
@@ -571,7 +575,6 @@ int mx_lanczos_steps(tdse *h, int m, double dt, long nsteps) {
   if (rc) return rc;
   rc = refresh_split(h, true);
   if (rc) return rc;
-  const OperatorView op = view(h);
   const MixedView mv = mview(h);
   const size_t G = npts(h);
   float2 *z = h->mwork;
@@ -593,7 +596,7 @@ int mx_lanczos_steps(tdse *h, int m, double dt, long nsteps) {
     }
     TDSE_LAUNCH(h, TDSE_K_LANCZOS_EXPM, launch_lanczos_expm(m, dt, h->ls, h->stream), "lanczos expm");
     TDSE_LAUNCH(h, TDSE_K_LANCZOS_COMBINE,
-                launch_mx_lanczos_combine(h->g, op, h->psi, hi, lo, h->mwork + G, G, h->red, h->ls,
+                launch_mx_lanczos_combine(h->g, view(h), h->psi, hi, lo, h->mwork + G, G, h->red, h->ls,
                                           h->status, h->stream),
                 "mixed lanczos combine");
     TDSE_HOOK(h, t0 + (double)(n + 1) * dt, dt);
@@ -685,8 +688,7 @@ int taylor_steps(tdse *h, int P, double dt, long nsteps) {
   if (rc || done) return rc;
   rc = ensure_work(h, 2);
   if (rc) return rc;
-  OperatorView op = view(h);
-  op.plain = fits_cluster(h, TDSE_TAYLOR, P);
+  const bool plain = fits_cluster(h, TDSE_TAYLOR, P);
   const size_t G = npts(h);
   double2 *buf[2] = {h->work, h->work + G};
   const double t0 = h->t;
@@ -696,7 +698,7 @@ int taylor_steps(tdse *h, int P, double dt, long nsteps) {
     for (int k = P; k >= 1; --k) {
       const bool last = (k == 1);
       double2 *out = last ? ((P == 1) ? buf[0] : h->psi) : buf[(P - k) & 1];
-      TDSE_LAUNCH(h, TDSE_K_TAYLOR_STAGE, launch_taylor_stage(h->g, op, E, dt / (double)k, in, h->psi, out, last, h->stream),
+      TDSE_LAUNCH(h, TDSE_K_TAYLOR_STAGE, launch_taylor_stage(h->g, view(h, plain), E, dt / (double)k, in, h->psi, out, last, h->stream),
                   "taylor stage");
       in = out;
     }
@@ -714,18 +716,17 @@ int rk4_steps(tdse *h, double dt, long nsteps) {
   if (rc || done) return rc;
   rc = ensure_work(h, 3);
   if (rc) return rc;
-  OperatorView op = view(h);
-  op.plain = fits_cluster(h, TDSE_RK4, 4);
+  const bool plain = fits_cluster(h, TDSE_RK4, 4);
   const size_t G = npts(h);
   double2 *ga = h->work, *gb = h->work + G, *acc = h->work + 2 * G;
   const double t0 = h->t;
   for (long n = 0; n < nsteps; ++n) {
     const double tn = t0 + (double)n * dt;
     const double E1 = coupling_at(h, tn), E2 = coupling_at(h, tn + 0.5 * dt), E4 = coupling_at(h, tn + dt);
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E1, 1, dt, h->psi, h->psi, acc, ga, nullptr, h->stream), "rk stage 1");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E2, 2, dt, ga, h->psi, acc, gb, nullptr, h->stream), "rk stage 2");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E2, 3, dt, gb, h->psi, acc, ga, nullptr, h->stream), "rk stage 3");
-    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, E4, 4, dt, ga, h->psi, acc, nullptr, h->psi, h->stream), "rk stage 4");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h, plain), E1, 1, dt, h->psi, h->psi, acc, ga, nullptr, h->stream), "rk stage 1");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h, plain), E2, 2, dt, ga, h->psi, acc, gb, nullptr, h->stream), "rk stage 2");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h, plain), E2, 3, dt, gb, h->psi, acc, ga, nullptr, h->stream), "rk stage 3");
+    TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h, plain), E4, 4, dt, ga, h->psi, acc, nullptr, h->psi, h->stream), "rk stage 4");
     TDSE_HOOK(h, t0 + (double)(n + 1) * dt, dt);
   }
   return TDSE_OK;
@@ -776,7 +777,6 @@ int lanczos_steps(tdse *h, int m, double dt, long nsteps) {
   // work slot 0: z; slots 1..m-1: U_1..U_{m-1} (U_0 is psi itself)
   rc = ensure_work(h, (size_t)(m > 1 ? m : 1));
   if (rc) return rc;
-  const OperatorView op = view(h);
   const size_t G = npts(h);
   double2 *z = h->work;
   auto U = [&](int j) -> double2 * { return j == 0 ? h->psi : h->work + (size_t)j * G; };
@@ -786,13 +786,13 @@ int lanczos_steps(tdse *h, int m, double dt, long nsteps) {
   for (long n = 0; n < nsteps; ++n) {
     const double E = coupling_at(h, t0 + (double)n * dt + 0.5 * dt);
     for (int j = 0; j < m; ++j) {
-      TDSE_LAUNCH(h, TDSE_K_LANCZOS_A, launch_lanczos_a(h->g, op, E, j, U(j), j > 0 ? U(j - 1) : nullptr, z, h->red, h->ls, h->stream),
+      TDSE_LAUNCH(h, TDSE_K_LANCZOS_A, launch_lanczos_a(h->g, view(h), E, j, U(j), j > 0 ? U(j - 1) : nullptr, z, h->red, h->ls, h->stream),
                   "lanczos a");
       if (j + 1 < m)
         TDSE_LAUNCH(h, TDSE_K_LANCZOS_B, launch_lanczos_b(h->g, j, z, U(j), U(j + 1), h->red, h->ls, h->stream), "lanczos b");
     }
     TDSE_LAUNCH(h, TDSE_K_LANCZOS_EXPM, launch_lanczos_expm(m, dt, h->ls, h->stream), "lanczos expm");
-    TDSE_LAUNCH(h, TDSE_K_LANCZOS_COMBINE, launch_lanczos_combine(h->g, op, m, h->psi, h->work + G, G, h->red, h->ls, h->status, h->stream),
+    TDSE_LAUNCH(h, TDSE_K_LANCZOS_COMBINE, launch_lanczos_combine(h->g, view(h), m, h->psi, h->work + G, G, h->red, h->ls, h->status, h->stream),
                 "lanczos combine");
     TDSE_HOOK(h, t0 + (double)(n + 1) * dt, dt);
   }
@@ -874,7 +874,6 @@ int rk_general_steps(tdse *h, int id, double dt, long nsteps, double *sigma) {
     return fail(h, TDSE_ERR_OOM, "RK error-estimate scalar");
   }
   TDSE_CUDA(h, cudaMemsetAsync(h->rk_sigma, 0, sizeof(double), h->stream), "clear sigma");
-  const OperatorView op = view(h);
   const size_t G = npts(h);
   double2 *gbuf[2] = {h->work, h->work + G};
   auto kbuf = [&](int j) { return h->work + (size_t)(2 + j) * G; };
@@ -907,7 +906,7 @@ int rk_general_steps(tdse *h, int id, double dt, long nsteps, double *sigma) {
         a.psi_out = (i == 0) ? gbuf[0] : h->psi;
       }
       const double E = coupling_at(h, tn + tb.c[i] * dt);
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_general_stage(h->g, op, E, gin, h->psi, a, h->red, h->stream),
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_general_stage(h->g, view(h), E, gin, h->psi, a, h->red, h->stream),
                   "rk stage");
     }
     if (s == 1)
@@ -933,10 +932,13 @@ int imag_steps(tdse *h, int method, int order, double dt, long nsteps, double *e
     return fail(h, TDSE_ERR_OOM, "imaginary-time scalars");
   }
   const size_t G = npts(h);
-  OperatorView op = view(h);
-  op.mask_start = h->g.N;   // no absorber in imaginary time
   int rc = ensure_work(h, method == TDSE_LANCZOS ? (size_t)(order > 1 ? order : 1) : (method == TDSE_RK4 ? 3 : 2));
   if (rc) return rc;
+  auto unmasked = [&] {   // no absorber in imaginary time
+    OperatorView op = view(h);
+    op.mask_start = h->g.N;
+    return op;
+  };
   for (long n = 0; n < nsteps; ++n) {
     TDSE_LAUNCH(h, TDSE_K_NORM, launch_norm(h->g, h->psi, h->red, h->ls, h->status, h->stream), "norm");
     TDSE_CUDA(h, launch_imag_begin(h->red, h->g.dr, h->imag, h->stream), "imaginary-time norm");
@@ -947,7 +949,7 @@ int imag_steps(tdse *h, int method, int order, double dt, long nsteps, double *e
         const bool last = (k == 1);
         double2 *out = last ? ((order == 1) ? buf[0] : h->psi) : buf[(order - k) & 1];
         TDSE_LAUNCH(h, TDSE_K_TAYLOR_STAGE,
-                    launch_taylor_stage(h->g, op, 0.0, dt / (double)k, in, h->psi, out, last, h->stream, true),
+                    launch_taylor_stage(h->g, view(h), 0.0, dt / (double)k, in, h->psi, out, last, h->stream, true),
                     "taylor stage");
         in = out;
       }
@@ -956,22 +958,22 @@ int imag_steps(tdse *h, int method, int order, double dt, long nsteps, double *e
                   "taylor copy");
     } else if (method == TDSE_RK4) {
       double2 *ga = h->work, *gb = h->work + G, *acc = h->work + 2 * G;
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 1, dt, h->psi, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 1");
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 2, dt, ga, h->psi, acc, gb, nullptr, h->stream, true), "rk stage 2");
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 3, dt, gb, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 3");
-      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, op, 0.0, 4, dt, ga, h->psi, acc, nullptr, h->psi, h->stream, true), "rk stage 4");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h), 0.0, 1, dt, h->psi, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 1");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h), 0.0, 2, dt, ga, h->psi, acc, gb, nullptr, h->stream, true), "rk stage 2");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h), 0.0, 3, dt, gb, h->psi, acc, ga, nullptr, h->stream, true), "rk stage 3");
+      TDSE_LAUNCH(h, TDSE_K_RK_STAGE, launch_rk_stage(h->g, view(h), 0.0, 4, dt, ga, h->psi, acc, nullptr, h->psi, h->stream, true), "rk stage 4");
     } else {
       const int m = order;
       double2 *z = h->work;
       auto U = [&](int j) -> double2 * { return j == 0 ? h->psi : h->work + (size_t)j * G; };
       for (int j = 0; j < m; ++j) {
-        TDSE_LAUNCH(h, TDSE_K_LANCZOS_A, launch_lanczos_a(h->g, op, 0.0, j, U(j), j > 0 ? U(j - 1) : nullptr, z, h->red, h->ls, h->stream),
+        TDSE_LAUNCH(h, TDSE_K_LANCZOS_A, launch_lanczos_a(h->g, view(h), 0.0, j, U(j), j > 0 ? U(j - 1) : nullptr, z, h->red, h->ls, h->stream),
                     "lanczos a");
         if (j + 1 < m)
           TDSE_LAUNCH(h, TDSE_K_LANCZOS_B, launch_lanczos_b(h->g, j, z, U(j), U(j + 1), h->red, h->ls, h->stream), "lanczos b");
       }
       TDSE_LAUNCH(h, TDSE_K_LANCZOS_EXPM, launch_lanczos_expm(m, dt, h->ls, h->stream, true), "lanczos expm");
-      TDSE_LAUNCH(h, TDSE_K_LANCZOS_COMBINE, launch_lanczos_combine(h->g, op, m, h->psi, h->work + G, G, h->red, h->ls, h->status, h->stream),
+      TDSE_LAUNCH(h, TDSE_K_LANCZOS_COMBINE, launch_lanczos_combine(h->g, unmasked(), m, h->psi, h->work + G, G, h->red, h->ls, h->status, h->stream),
                   "lanczos combine");
     }
     TDSE_LAUNCH(h, TDSE_K_NORM, launch_norm(h->g, h->psi, h->red, h->ls, h->status, h->stream), "norm");
@@ -1057,6 +1059,7 @@ int tdse_create(int N, double dr, int lmax, int stencil, double Z, const double 
     const long v = std::strtol(gb, nullptr, 10);
     if (v > 0) h->guard = ((size_t)v + 255) / 256 * 256;   // keeps every buffer 256-byte aligned
   }
+  if (const char *fa = std::getenv("TDSE_FAIL_ALLOC")) h->fail_alloc = fa;
   const int nbx = observables_blocks(h->g);
   const size_t obs_n = (size_t)5 * nbx * (lmax + 1) + 2;
   bool ok = DMALLOC(h, psi, sizeof(double2) * G) == cudaSuccess &&
