@@ -402,7 +402,8 @@ int tdse_small_grid_path_used(const tdse_t *h);
 /*
  * Larger grids: every FP64 length-gauge Lanczos step of a tdse_propagate call
  * in one cooperative launch (Appendix "Lanczos methods"), when no per-step
- * observables are set up.  The multi-launch path issues 2 order + 1 launches
+ * observables are set up and the handle holds the fixed-point form of its
+ * operator (tdse_create: not with potentials or spacings outside its range).  The multi-launch path issues 2 order + 1 launches
  * per step; here one grid of one block of 512 threads per SM stays resident,
  * separates the phases by grid-wide barriers (bounded waits) and has every
  * block add each reduction's block partials in the multi-launch path's fixed

@@ -172,7 +172,7 @@ OperatorView view(const tdse *h, bool plain = false) {
   op.c2q = h->c2q;
   op.fx_ec = h->fx_ec;
   op.fx_ok = h->diagq ? 1 : 0;
-  op.plain = plain;
+  op.plain = plain || !h->diagq;
   return op;
 }
 
@@ -232,8 +232,7 @@ cudaError_t dmalloc(tdse *h, T **p, size_t bytes, const char *name) {
 #define DMALLOC(h, field, bytes) dmalloc(h, &(h)->field, bytes, #field)
 
 // The fixed-point walker's form of the operator, from the FP64 diagonal on the
-// device; dmax bounds its magnitude.  Left out (the walker then runs in FP64
-// point by point) where the coefficients do not fit the encoding, and where
+// device; dmax bounds its magnitude.  Left out (the kernels then run in FP64) where the coefficients do not fit the encoding, and where
 // there is no memory for the table.
 int build_fixed(tdse *h, double dmax) {
   if (!(tdse_fx::fx_scale(h->g.c0, h->fx_ec) && tdse_fx::fx_diag_fits(dmax, h->fx_ec))) {
@@ -757,6 +756,7 @@ int persistent_steps(tdse *h, int m, double dt, long nsteps, bool *done) {
     }
   }
   if ((rc = upload_etab(h, TDSE_LANCZOS, dt, nsteps))) return rc;
+  if (!h->diagq) return TDSE_OK;   // (the allocations above may have given it back)
   if (!h->lanczos_norm_valid)
     TDSE_LAUNCH(h, TDSE_K_NORM, launch_norm(h->g, h->psi, h->red, h->ls, h->status, h->stream), "norm");
   TDSE_LAUNCH(h, TDSE_K_PERSISTENT,

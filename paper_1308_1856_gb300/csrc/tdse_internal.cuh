@@ -81,7 +81,7 @@ struct OperatorView {
   const long long *diagq = nullptr;
   long long c1q = 0, c2q = 0;
   int fx_ec = 0, fx_ok = 0;
-  bool plain = false;             // length gauge: Taylor and RK4 stages in FP64 (see launch_taylor_stage)
+  bool plain = false;             // all in FP64 (where fx_ok is 0, and where the cluster path's bits are wanted)
 };
 
 // diagq = diag in the fixed-point walker's encoding (fx_encode_diag).
@@ -89,7 +89,7 @@ cudaError_t launch_fx_diag(const double *diag, size_t G, int ec, long long *diag
 
 cudaError_t launch_apply_h(const Geometry &g, const OperatorView &op, double E,
                            const double2 *x, double2 *y, cudaStream_t s);
-// op.plain: all in FP64, bitwise the cluster path's arithmetic.
+// op.plain, length gauge: bitwise the cluster path's arithmetic.
 // imag: the stage of exp(-H dt) (imaginary time: -H instead of -i H, no mask).
 cudaError_t launch_taylor_stage(const Geometry &g, const OperatorView &op, double E, double s,
                                 const double2 *v_in, const double2 *psi, double2 *v_out,

@@ -16,12 +16,17 @@
 // it (for_my_strips).  The warps' numbers run across the blocks, so that the
 // warps with one segment more are spread evenly over the SMs.
 //
-// Taylor and RK4 stages of length-gauge grids that fit the one-launch cluster
-// path, whose states are bitwise these: all in FP64, in segments of 32 radial
+// All in FP64 run the Taylor and RK4 stages of length-gauge grids that fit the
+// one-launch cluster path, whose states are bitwise these, and every kernel of a
+// grid without the fixed-point form (coefficients that do not fit, or no memory
+// for its diagonal; OperatorView::plain): in segments of 32 radial
 // points of one partial wave, ordered radial-group-major, a contiguous balanced
 // range for each warp (warp_range).  A lane owns one radial index j and walks l
 // upwards keeping x_{l-1,j}, x_{l,j}, x_{l+1,j} in registers; the arithmetic is
 // written with explicit __dmul_rn / __dadd_rn / __fma_rn.
+// H x of 512,000 points on a grid whose potential does not fit: 19 us in these
+// registers, velocity gauge 45 us; point by point from L2 in the fixed-point walker 35
+// and 62 us.
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -40,7 +45,7 @@ using namespace common;
 using namespace stencil;
 
 // Visit this warp's share of the 32-point row segments (see the file header).
-template <int ST, typename F>
+template <int ST, bool VG, typename F>
 __device__ __forceinline__ void for_my_segments(const StencilIn &in, F &&f) {
   const int lane = threadIdx.x & 31;
   const int Lp1 = in.L + 1;
@@ -53,26 +58,27 @@ __device__ __forceinline__ void for_my_segments(const StencilIn &in, F &&f) {
     const long long left = s_end - s;
     const int l1 = (left < (long long)(Lp1 - l0)) ? l0 + (int)left : Lp1;
     const int i = jg * 32 + lane;
-    if (i < in.N) walk_rows<ST>(in, i, l0, l1, f);
+    if (i < in.N) walk_rows<ST, VG>(in, i, l0, l1, f);
     s += l1 - l0;
   }
 }
 
-// How a stencil kernel walks the grid: in fixed point (of the length or velocity
-// gauge), or in FP64 (length gauge).
-enum Walk { kFixed, kFixedVG, kPlain };
+// How a stencil kernel walks the grid: in fixed point or in FP64, in the length or
+// the velocity gauge.
+enum Walk { kFixed, kFixedVG, kPlain, kPlainVG };
+constexpr bool is_plain(int walk) { return walk == kPlain || walk == kPlainVG; }
 template <int WALK>
-using OpIn = std::conditional_t<WALK == kPlain, StencilIn, FxIn>;
+using OpIn = std::conditional_t<is_plain(WALK), StencilIn, FxIn>;
 // Blocks an SM: one of 16 warps with 128 registers a thread and its rings in
 // fixed point, two of 64 registers in FP64.
 template <int WALK>
-constexpr int kOpBlocksPerSM = WALK == kPlain ? kStencilBlocksPerSM : 1;
+constexpr int kOpBlocksPerSM = is_plain(WALK) ? kStencilBlocksPerSM : 1;
 
 // Call f(idx, i, H x, x, extra values) at every point this thread owns.
 template <int ST, int WALK, int EX, typename F>
 __device__ __forceinline__ void for_my_points(const OpIn<WALK> &in, const FxExtra<EX> &ex, F &&f) {
-  if constexpr (WALK == kPlain) {
-    for_my_segments<ST>(in, [&](int i, size_t idx, double2 t, double2 u) {
+  if constexpr (is_plain(WALK)) {
+    for_my_segments<ST, WALK == kPlainVG>(in, [&](int i, size_t idx, double2 t, double2 u) {
       double2 e[EX > 0 ? EX : 1];
 #pragma unroll
       for (int q = 0; q < EX; ++q) e[q] = ex.p[q][idx];
@@ -250,8 +256,9 @@ __global__ void __launch_bounds__(kBlockJ, kOpBlocksPerSM<WALK>)
   double acc = 0.0;
   FxExtra<EX> ex;
   if (EX > 0) ex.p[0] = uprev;
-  in.k = sc.k;
+  if constexpr (!is_plain(WALK)) in.k = sc.k;
   for_my_points<ST, WALK, EX>(in, ex, [&](int idx, int, double2 t, double2 u, const double2 (&e)[1]) {
+    if (is_plain(WALK)) t = make_double2(__dmul_rn(sc.s, t.x), __dmul_rn(sc.s, t.y));
     double2 o = t;
     if (EX > 0) {
       o.x = __fma_rn(-cprev, e[0].x, t.x);
@@ -514,14 +521,14 @@ __global__ void __launch_bounds__(kObsThreads)
 template <int WALK>
 OpIn<WALK> make_in(const Geometry &g, const OperatorView &op, double E, const double2 *x) {
   OpIn<WALK> in;
-  if constexpr (WALK == kPlain) {
+  if constexpr (is_plain(WALK)) {
     in.diag = op.diag;
   } else {
-    in.diagq = op.fx_ok ? op.diagq : reinterpret_cast<const long long *>(op.diag);
+    in.diagq = op.diagq;
     in.c1q = op.c1q;
     in.c2q = op.c2q;
     in.ec = op.fx_ec;
-    in.ok = op.fx_ok;
+    in.ok = 1;
     in.k = 0;
   }
   in.rinv = op.rinv;
@@ -542,15 +549,14 @@ using IC = std::integral_constant<int, V>;
 template <bool V>
 using BC = std::integral_constant<bool, V>;
 
-// f(stencil, walk) with both as compile-time constants.  PLAIN: whether the
-// caller has a use for the length gauge's FP64 walk, taken where `plain` says so.
-template <bool PLAIN, typename F>
+// f(stencil, walk) with both as compile-time constants.
+template <typename F>
 void dispatch(const Geometry &g, bool vg, bool plain, F &&f) {
   auto go = [&](auto st) {
-    if (vg) return f(st, IC<kFixedVG>{});
-    if constexpr (PLAIN)
-      if (plain) return f(st, IC<kPlain>{});
-    f(st, IC<kFixed>{});
+    if (plain && vg) f(st, IC<kPlainVG>{});
+    else if (plain) f(st, IC<kPlain>{});
+    else if (vg) f(st, IC<kFixedVG>{});
+    else f(st, IC<kFixed>{});
   };
   if (g.stencil == 5) go(IC<5>{});
   else go(IC<3>{});
@@ -575,10 +581,10 @@ inline unsigned block_parts(const Geometry &g) {
 // the 48 KB default once per instantiation and device.
 template <auto KERN, int WALK, int EX>
 OpLaunch op_launch(const Geometry &g) {
-  constexpr size_t bytes = WALK == kPlain ? 0 : (kBlockJ / 32) * (size_t)fx_warp_bytes<EX, WALK == kFixedVG>();
+  constexpr size_t bytes = is_plain(WALK) ? 0 : (kBlockJ / 32) * (size_t)fx_warp_bytes<EX, WALK == kFixedVG>();
   static_assert(bytes <= 226 * 1024, "an SM's shared memory, less the kernel's own");
-  const unsigned parts = WALK == kPlain ? 1u : block_parts(g);
-  if (WALK != kPlain) {
+  const unsigned parts = is_plain(WALK) ? 1u : block_parts(g);
+  if (!is_plain(WALK)) {
     // one split of L1 and shared memory for all of them: a kernel that wants
     // another than its predecessor's waits for the SM to drain (Dormand-Prince
     // on 50,000 points: 279 us for four steps, 233 with one split)
@@ -599,7 +605,7 @@ cudaError_t launch_fx_diag(const double *diag, size_t G, int ec, long long *diag
 cudaError_t launch_apply_h(const Geometry &g, const OperatorView &op, double E,
                            const double2 *x, double2 *y, cudaStream_t s) {
   cudaError_t e = cudaSuccess;
-  dispatch<false>(g, g.gauge == 1, false, [&](auto st, auto walk) {
+  dispatch(g, g.gauge == 1, op.plain, [&](auto st, auto walk) {
     constexpr int ST = decltype(st)::value;
     constexpr int WALK = decltype(walk)::value;
     const OpLaunch o = op_launch<apply_h_kernel<ST, WALK>, WALK, 0>(g);
@@ -615,14 +621,14 @@ cudaError_t launch_taylor_stage(const Geometry &g, const OperatorView &op, doubl
                                 bool final_stage, cudaStream_t st, bool imag) {
   const int mstart = op.mask_start;
   cudaError_t e = cudaSuccess;
-  dispatch<true>(g, !imag && g.gauge == 1, !imag && op.plain, [&](auto stc, auto walk) {
+  dispatch(g, !imag && g.gauge == 1, op.plain, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
     constexpr int WALK = decltype(walk)::value;
     const auto in = make_in<WALK>(g, op, E, v_in);
-    if constexpr (WALK == kFixed)   // imaginary time: no absorber, no field
+    if constexpr (WALK == kFixed || WALK == kPlain)   // imaginary time: no absorber, no field
       if (imag) {
-        e = launch_pdl(taylor_stage_kernel<ST, true, kFixed, false>,
-                       op_launch<taylor_stage_kernel<ST, true, kFixed, false>, kFixed, 1>(g), st, in, s, psi,
+        e = launch_pdl(taylor_stage_kernel<ST, true, WALK, false>,
+                       op_launch<taylor_stage_kernel<ST, true, WALK, false>, WALK, 1>(g), st, in, s, psi,
                        v_out, op.mask, mstart);
         return;
       }
@@ -647,7 +653,7 @@ cudaError_t launch_rk_stage(const Geometry &g, const OperatorView &op, double E,
   const double ca = dt * a_next[stage - 1], cb = dt * b[stage - 1];
   const int mstart = imag ? g.N : op.mask_start;
   cudaError_t e = cudaSuccess;
-  dispatch<true>(g, !imag && g.gauge == 1, !imag && op.plain, [&](auto stc, auto walk) {
+  dispatch(g, !imag && g.gauge == 1, op.plain, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
     constexpr int WALK = decltype(walk)::value;
     const auto in = make_in<WALK>(g, op, E, gin);
@@ -664,7 +670,7 @@ cudaError_t launch_rk_stage(const Geometry &g, const OperatorView &op, double E,
       else if (stage < 4) go(IC<1>{}, im);
       else go(IC<2>{}, im);
     };
-    if constexpr (WALK == kFixed)
+    if constexpr (WALK == kFixed || WALK == kPlain)
       if (imag) return parts(BC<true>{});
     parts(BC<false>{});
   });
@@ -680,7 +686,7 @@ cudaError_t launch_rk_general_stage(const Geometry &g, const OperatorView &op, d
   cudaError_t e = cudaSuccess;
   if (!a.last && a.stage == kRkMaxStages - 1) return cudaErrorInvalidValue;   // no stage after the last
   if (a.fsal && (!a.last || a.stage == 0)) return cudaErrorInvalidValue;
-  dispatch<false>(g, g.gauge == 1, false, [&](auto stc, auto walk) {
+  dispatch(g, g.gauge == 1, op.plain, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
     constexpr int WALK = decltype(walk)::value;
     const auto in = make_in<WALK>(g, op, E, gin);
@@ -735,7 +741,7 @@ cudaError_t launch_lanczos_a(const Geometry &g, const OperatorView &op, double E
                              const double2 *u, const double2 *uprev, double2 *z,
                              Reduction *red, LanczosScalars *ls, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
-  dispatch<false>(g, g.gauge == 1, false, [&](auto stc, auto walk) {
+  dispatch(g, g.gauge == 1, op.plain, [&](auto stc, auto walk) {
     constexpr int ST = decltype(stc)::value;
     constexpr int WALK = decltype(walk)::value;
     const auto in = make_in<WALK>(g, op, E, u);

@@ -300,7 +300,7 @@ cudaError_t launch_lanczos_persistent(const Geometry &g, const OperatorView &op,
   PersistArgs a;
   FxIn &in = a.in;
   in.x = psi;
-  in.diagq = op.fx_ok ? op.diagq : reinterpret_cast<const long long *>(op.diag);
+  in.diagq = op.diagq;
   in.rj = op.rj;
   in.kappa = op.kappa;
   in.N = g.N;
@@ -310,7 +310,7 @@ cudaError_t launch_lanczos_persistent(const Geometry &g, const OperatorView &op,
   in.c1q = op.c1q;
   in.c2q = op.c2q;
   in.ec = op.fx_ec;
-  in.ok = op.fx_ok;
+  in.ok = 1;
   in.k = 0;
   in.E = 0.0;
   in.rinv = nullptr;

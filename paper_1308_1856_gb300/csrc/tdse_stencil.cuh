@@ -39,14 +39,14 @@ struct StencilIn {
 // First derivative of a row at column i (zero beyond the box): Sec. 2's
 // 4th-order formula [-f_{j+2} + 8 f_{j+1} - 8 f_{j-1} + f_{j-2}] / (12 dr), or
 // [f_{j+1} - f_{j-1}] / (2 dr) with the 3-point stencil.
-template <int ST>
+template <int ST, bool CG = false>
 __device__ __forceinline__ double2 d1_point(const StencilIn &in, const double2 *row, int i) {
   const double2 z = make_double2(0.0, 0.0);
-  const double2 m1 = (i >= 1) ? __ldcg(row + i - 1) : z;
-  const double2 p1 = (i + 1 < in.N) ? __ldcg(row + i + 1) : z;
+  const double2 m1 = (i >= 1) ? ldx<CG>(row + i - 1) : z;
+  const double2 p1 = (i + 1 < in.N) ? ldx<CG>(row + i + 1) : z;
   if (ST == 5) {
-    const double2 m2 = (i >= 2) ? __ldcg(row + i - 2) : z;
-    const double2 p2 = (i + 2 < in.N) ? __ldcg(row + i + 2) : z;
+    const double2 m2 = (i >= 2) ? ldx<CG>(row + i - 2) : z;
+    const double2 p2 = (i + 2 < in.N) ? ldx<CG>(row + i + 2) : z;
     return make_double2(
         __dmul_rn(in.d1c, __fma_rn(8.0, __dsub_rn(p1.x, m1.x), __dsub_rn(m2.x, p2.x))),
         __dmul_rn(in.d1c, __fma_rn(8.0, __dsub_rn(p1.y, m1.y), __dsub_rn(m2.y, p2.y))));
@@ -174,12 +174,36 @@ __device__ __forceinline__ void split2(double2 v, float2 &h, float2 &lo) {
   lo = make_float2(__double2float_rn(v.x - (double)h.x), __double2float_rn(v.y - (double)h.y));
 }
 
-// Walk rows [l0, l1) of column i (length gauge) and call f(i, idx, Hx, x_center).
-template <int ST, typename F>
+// The velocity gauge's coupling at (l, i): (A/c) p_z with p_z = -i [ (d/dr - l/r)
+// kappa_l f_{l-1} + (d/dr + (l+1)/r) kappa_{l+1} f_{l+1} ] (the partial-wave form
+// of -i d/dz; the paper prints the l/r terms with the opposite signs), added to t.
+template <int ST, bool CG = false>
+__device__ __forceinline__ void velocity_point(const StencilIn &in, int l, int i, double2 prev, double2 next,
+                                               double2 &t) {
+  const double ri = __ldg(in.rinv + i);
+  double wx = 0.0, wy = 0.0;
+  if (l > 0) {
+    const double2 dp = d1_point<ST, CG>(in, in.x + (size_t)(l - 1) * in.N, i);
+    const double k = in.kappa[l], lr = __dmul_rn((double)l, ri);
+    wx = __dmul_rn(k, __fma_rn(-lr, prev.x, dp.x));
+    wy = __dmul_rn(k, __fma_rn(-lr, prev.y, dp.y));
+  }
+  if (l < in.L) {
+    const double2 dn = d1_point<ST, CG>(in, in.x + (size_t)(l + 1) * in.N, i);
+    const double k = in.kappa[l + 1], lr = __dmul_rn((double)(l + 1), ri);
+    wx = __fma_rn(k, __fma_rn(lr, next.x, dn.x), wx);
+    wy = __fma_rn(k, __fma_rn(lr, next.y, dn.y), wy);
+  }
+  t.x = __fma_rn(in.E, wy, t.x);   // -i (A/c) w
+  t.y = __fma_rn(-in.E, wx, t.y);
+}
+
+// Walk rows [l0, l1) of column i and call f(i, idx, Hx, x_center).
+template <int ST, bool VG, typename F>
 __device__ __forceinline__ void walk_rows(const StencilIn &in, int i, int l0, int l1, F &&f) {
   const int N = in.N, L = in.L;
   const double2 z = make_double2(0.0, 0.0);
-  const double Er = __dmul_rn(in.E, in.rj[i]);
+  const double Er = VG ? 0.0 : __dmul_rn(in.E, in.rj[i]);
   double2 prev = (l0 > 0) ? ldx<false>(in.x + (size_t)(l0 - 1) * N + i) : z;
   double2 cur = ldx<false>(in.x + (size_t)l0 * N + i);
   double a_cur = __dmul_rn(in.kappa[l0], Er);
@@ -187,34 +211,14 @@ __device__ __forceinline__ void walk_rows(const StencilIn &in, int i, int l0, in
     const size_t idx = (size_t)l * N + i;
     const double2 next = (l < L) ? ldx<false>(in.x + idx + N) : z;
     const double a_next = __dmul_rn(in.kappa[l + 1], Er);
-    const double2 t = h_point<ST>(in, in.x + (size_t)l * N, i, __ldg(in.diag + idx), prev, cur, next, a_cur, a_next);
+    double2 t =
+        h_point<ST, !VG>(in, in.x + (size_t)l * N, i, __ldg(in.diag + idx), prev, cur, next, a_cur, a_next);
+    if (VG) velocity_point<ST>(in, l, i, prev, next, t);
     f(i, idx, t, cur);
     prev = cur;
     cur = next;
     a_cur = a_next;
   }
-}
-
-// The velocity gauge's coupling at (l, i): (A/c) p_z with p_z = -i [ (d/dr - l/r)
-// kappa_l f_{l-1} + (d/dr + (l+1)/r) kappa_{l+1} f_{l+1} ] (the partial-wave form
-// of -i d/dz; the paper prints the l/r terms with the opposite signs).
-template <int ST>
-__device__ __forceinline__ double2 velocity_point(const StencilIn &in, int l, int i, double2 prev, double2 next) {
-  const double ri = __ldg(in.rinv + i);
-  double wx = 0.0, wy = 0.0;
-  if (l > 0) {
-    const double2 dp = d1_point<ST>(in, in.x + (size_t)(l - 1) * in.N, i);
-    const double k = in.kappa[l], lr = __dmul_rn((double)l, ri);
-    wx = __dmul_rn(k, __fma_rn(-lr, prev.x, dp.x));
-    wy = __dmul_rn(k, __fma_rn(-lr, prev.y, dp.y));
-  }
-  if (l < in.L) {
-    const double2 dn = d1_point<ST>(in, in.x + (size_t)(l + 1) * in.N, i);
-    const double k = in.kappa[l + 1], lr = __dmul_rn((double)(l + 1), ri);
-    wx = __fma_rn(k, __fma_rn(lr, next.x, dn.x), wx);
-    wy = __fma_rn(k, __fma_rn(lr, next.y, dn.y), wy);
-  }
-  return make_double2(__dmul_rn(in.E, wy), __dmul_rn(-in.E, wx));   // -i (A/c) w
 }
 
 // First derivative of the mixed operand's row starting at element `row`, at

@@ -87,11 +87,7 @@ __device__ __noinline__ double2 h_point_fp64(const FxIn &in, int l, int i) {
   const double2 next = l < in.L ? __ldcg(in.x + idx + in.N) : z;
   double2 t = h_point<ST, !VG, true>(s, in.x + (size_t)l * in.N, i, fx_diag_double(in, in.diagq[idx]), prev,
                                __ldcg(in.x + idx), next, __dmul_rn(in.kappa[l], Er), __dmul_rn(in.kappa[l + 1], Er));
-  if (VG) {
-    const double2 v = velocity_point<ST>(s, l, i, prev, next);
-    t.x += v.x;
-    t.y += v.y;
-  }
+  if (VG) velocity_point<ST, true>(s, l, i, prev, next, t);
   return make_double2(ldexp(t.x, in.k), ldexp(t.y, in.k));
 }
 
