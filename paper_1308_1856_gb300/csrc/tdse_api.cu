@@ -33,7 +33,7 @@ struct tdse {
   double *rinv = nullptr;          // 1 / r_j (velocity gauge)
   long long *diagq = nullptr;      // diag for the fixed-point walker; null where it does not fit or memory is short
   long long c1q = 0, c2q = 0;      // c1, c2 likewise
-  int fx_ec = 0;
+  int fx_e1 = 0, fx_e2 = 0, fx_ec = 0;
   int mask_start = 0;
   Reduction *red = nullptr;
   LanczosScalars *ls = nullptr;
@@ -170,6 +170,8 @@ OperatorView view(const tdse *h, bool plain = false) {
   op.diagq = h->diagq;
   op.c1q = h->c1q;
   op.c2q = h->c2q;
+  op.fx_e1 = h->fx_e1;
+  op.fx_e2 = h->fx_e2;
   op.fx_ec = h->fx_ec;
   op.fx_ok = h->diagq ? 1 : 0;
   op.plain = plain || !h->diagq;
@@ -240,13 +242,11 @@ int build_fixed(tdse *h, double dmax) {
     h->diagq = nullptr;
     return TDSE_OK;
   }
-  auto coef = [&](double v) {
-    uint64_t u;
-    std::memcpy(&u, &v, 8);
-    return (long long)tdse_fx::fx_coef(u, h->fx_ec);
-  };
-  h->c1q = coef(h->g.c1);
-  h->c2q = coef(h->g.c2);
+  const tdse_fx::FxStencilCoef c1 = tdse_fx::fx_stencil_coef(h->g.c1), c2 = tdse_fx::fx_stencil_coef(h->g.c2);
+  h->c1q = c1.q;
+  h->c2q = c2.q;
+  h->fx_e1 = c1.e;
+  h->fx_e2 = c2.e;
   if (!h->diagq && DMALLOC(h, diagq, sizeof(long long) * npts(h)) != cudaSuccess) {
     cudaGetLastError();
     h->diagq = nullptr;

@@ -57,7 +57,8 @@ constexpr int kChunkSegs = TDSE_CHUNK_SEGS;  // 32-point row segments per chunk 
 // slots (one per 512 points).
 constexpr int kChunkPts = 512;
 constexpr int kFxThreads = 128;              // threads of a block of the fixed-point stencil kernel
-constexpr int kFxBlocksPerSM = 4;            // 128 registers a thread
+template <bool VG>
+constexpr int kFxBlocksPerSM = VG ? 3 : 4;   // 128 registers a thread, 168 in the velocity gauge
 constexpr int kFxMaxRows = 32;               // segments of a chunk at most (16: 5% slower on large batches)
 constexpr int kMixedCombinePts = 2;          // the same for the mixed combine, two vectors per round
 
@@ -327,6 +328,8 @@ __device__ __forceinline__ FxIn fixed_in(const BatchDev &B, const BatchInst &I, 
   in.E = field_of(B, inst);
   in.c1q = I.c1q;
   in.c2q = I.c2q;
+  in.e1 = I.fx_e1;
+  in.e2 = I.fx_e2;
   in.ec = I.fx_ec;
   in.ok = I.fx_ok;
   in.k = k;
@@ -353,13 +356,14 @@ __device__ __forceinline__ void for_strided_chunks(const ChunkList &cl, F &&f) {
 // Phase A (a launch for each gauge's instances): the fixed-point walker
 // (tdse_walk_fixed.cuh) with the recurrence and the dot product in FP64: six
 // FP64 instructions a point (two of them integer conversions) in place of 20.
-// What bounds it: the integer and FP64 pipes' issue together (integer 76%, FP64
-// 58% busy, 16 warps an SM at 128 registers; more warps spill and are slower).
+// What bounds it: the issue of the integer and the FP64 pipe together, 16 warps an
+// SM at 128 registers; more warps spill more (56 bytes here) and are slower.  The velocity
+// gauge's needs 12 warps at 168: a batch of 16 instances 11.4 ms for four steps, 12.1 at 128.
 // All phase A launches of one step of 128 instances (8.1e7 points): 36.9 ms in
 // FP64, 19.5 ms here; of 8 instances (1.3e6 points), 24 ms to 6 ms over 8 steps,
 // where the smaller chunks count as well.
 template <int ST, bool VG, int EX>
-__global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM) bt_lanczos_a_fixed(BatchDev B, ChunkList cl, int j) {
+__global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM<VG>) bt_lanczos_a_fixed(BatchDev B, ChunkList cl, int j) {
   extern __shared__ __align__(16) unsigned char fx_smem[];
   unsigned char *ring = fx_smem + (threadIdx.x >> 5) * fx_warp_bytes<EX, VG>();
   for_strided_chunks(cl, [&](int inst, int ci) {
@@ -1359,15 +1363,11 @@ int Engine::place(int slot, const tdse_instance_spec &s, void *mem) {
     // largest |diagonal|: the centrifugal and Coulomb terms at the first point
     const double dmax = c0 + 0.5 * (double)L * (double)(L + 1) / (rj[0] * rj[0]) + std::fabs(s.Z) / rj[0];
     I.fx_ok = tdse_fx::fx_scale(c0, I.fx_ec) && tdse_fx::fx_diag_fits(dmax, I.fx_ec) ? 1 : 0;
-    auto coef = [&](double v) {
-      uint64_t u;
-      std::memcpy(&u, &v, 8);
-      return tdse_fx::fx_coef(u, I.fx_ec);
-    };
-    if (I.fx_ok) {
-      I.c1q = coef(I.c1);
-      I.c2q = coef(I.c2);
-    }
+    const tdse_fx::FxStencilCoef k1 = tdse_fx::fx_stencil_coef(I.c1), k2 = tdse_fx::fx_stencil_coef(I.c2);
+    I.c1q = k1.q;
+    I.c2q = k2.q;
+    I.fx_e1 = k1.e;
+    I.fx_e2 = k2.e;
   }
   bt_diag_table<<<(unsigned)(sms * 4), 256, 0, st>>>(I, c0);
   EN_CUDA(cudaGetLastError(), "diagonal table");
@@ -1796,7 +1796,7 @@ int Engine::launch_a(const BatchDev &B, const ChunkList &cl, int j, const Schedu
     EN_CUDA(e, "batch lanczos a (mixed tiles)");
     return TDSE_OK;
   }
-  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM : kFxBlocksPerSM / 2));
+  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM<false> : 2));
   const cudaError_t e = stencil == 5 ? launch_fixed<5, false>(grid, stream, B, cl, j)
                                      : launch_fixed<3, false>(grid, stream, B, cl, j);
   EN_CUDA(e, "batch lanczos a");
@@ -1805,7 +1805,7 @@ int Engine::launch_a(const BatchDev &B, const ChunkList &cl, int j, const Schedu
 
 // Chunks the phase-A launch takes at once: one per warp (FP64) or block (mixed tiles).
 int Engine::stencil_wave() const {
-  return precision == TDSE_MIXED ? sms * sched.sblocks * (kBlockJ / 32) : sms * kFxBlocksPerSM * (kFxThreads / 32);
+  return precision == TDSE_MIXED ? sms * sched.sblocks * (kBlockJ / 32) : sms * kFxBlocksPerSM<false> * (kFxThreads / 32);
 }
 
 // Velocity-gauge instances: the same fixed-point walker with the (A/c) p_z coupling,
@@ -1818,7 +1818,7 @@ int Engine::launch_a_velocity(const BatchDev &B, const ChunkList &cl, int j, con
     EN_CUDA(cudaGetLastError(), "batch lanczos a (mixed, velocity gauge)");
     return TDSE_OK;
   }
-  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM : kFxBlocksPerSM / 2));
+  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM<true> : 2));
   const cudaError_t e = stencil == 5 ? launch_fixed<5, true>(grid, stream, B, cl, j)
                                      : launch_fixed<3, true>(grid, stream, B, cl, j);
   EN_CUDA(e, "batch lanczos a (velocity gauge)");

@@ -30,8 +30,9 @@ struct BatchInst {
   int nchunk_e;          // reduction chunks of the elementwise kernels (consecutive points)
   int nchunk_d;          // reduction chunks of the dipole kernel (kChunkSegs row segments, both precisions)
   int fx_seg, fx_rows;   // fixed-point stencil: row segments of kFxCols columns, segments per chunk
-  int fx_ok, fx_ec;      // whether the coefficients fit the fixed-point form; their exponent
-  long long c1q, c2q;    // c1, c2 against 2^fx_ec
+  int fx_ok, fx_ec;      // whether the coefficients fit the fixed-point form; the diagonal's exponent
+  int fx_e1, fx_e2;      // c1, c2 in fixed point (fx_stencil_coef)
+  long long c1q, c2q;
   int gauge;             // TDSE_GAUGE_LENGTH or TDSE_GAUGE_VELOCITY (FP64 only)
   double c1, c2;         // stencil coefficients (c0 is folded into diag)
   double d1c;            // first-derivative scale of the velocity gauge (1/(12 dr) or 1/(2 dr))

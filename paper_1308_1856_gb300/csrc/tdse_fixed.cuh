@@ -7,27 +7,35 @@
 // the same sums as integer limb products take about a third of that, and they
 // leave the FP64 pipe to the epilogue.
 //
-// Representation.  A block of doubles (a lane's share of one row) with largest
-// exponent field e holds each value as a 60-bit two's complement integer X,
+// Representation.  A block of doubles (in the stencil: the two parts of one value)
+// with largest exponent field e holds each as a 60-bit two's complement integer X,
 //   x = X 2^(e - 1082),  |X| < 2^60,
 // so the block's largest values keep 7 bits more than a double's 53 and any
 // value down to 2^-7 of the largest is exact.  A coefficient is held against an
 // exponent ec of its own, c = K 2^(ec - 61), |K| <= 2^61.  Products are formed
 // from 32-bit limbs, X = xh 2^32 + xl with xl signed:
 //   X K = xh kh 2^64 + (xh kl + xl kh) 2^32 + xl kl.
-// hh and mm below are the first two sums over all terms of a point; the last
-// (below 2^62) is dropped, and V = X K / 2^64 = hh + mm / 2^32 rounded, so that
-// its low half costs no shift.  One unit of V is 2^-57 of the largest operand
-// times 2^ec: about 2^-54 of c0 x, and the only two roundings of a point (V and
-// the result) are below that, where FP64 rounds seven partial sums.
+// hh and mm below are the first two sums over all terms of a point, each operand
+// shifted to the exponent T - ec of the sum first (T: the largest of the terms' e +
+// ec); the last (below 2^62) is dropped, and V = (hh 2^64 + mm 2^32) / 2^61 is
+// rounded.  One unit u of V is 2^(T - 1082).
+//
+// Error.  The dropped products of the five terms are below 2 u each, the cuts of
+// the operands (in the conversion and in the shift) and of the coefficients below 12 u
+// together: V is off by less than 24 u, typically by 2 u.  The largest of a point's
+// own terms is at least 2^(T - 1027) (fx_scale, fx_stencil_coef and the walker's
+// kDiagHigh see to that), 2^55 u, so that the worst case is 6 2^-53 of the terms'
+// sum in modulus.  FP64 rounds six partial sums and reaches the same.
 //
 // Sums fit: with five products (stencil sums up to 2^61 with coefficients up to
-// 2^59, the others up to 2^60 and 2^61) |mm| < 6.7 2^60 and |hh| < 2^60.
+// 2^59, the diagonal's to 2^61, the couplings' to 2^61 / 3^(1/2)) |mm| < 6.2 2^60 and
+// |hh| < 2^59; the velocity gauge's two more (operands of 58 bits) make it 7.6 2^60.
 //
 // The functions are plain C on integers, compiled for the host as well, where
 // they are tested against 128-bit arithmetic.
 #pragma once
 
+#include <math.h>
 #include <stdint.h>
 
 #ifdef __CUDACC__
@@ -42,7 +50,6 @@ constexpr uint32_t kExpMask = 0x7ff00000u;   // exponent field of a double's hig
 // Block exponents from here on convert by fx_from_words, where a zero beside
 // the block's largest value comes out as zero; smaller ones by fx_from_small.
 constexpr int kExpSmall = 64;
-constexpr int kExpNonFinite = 0x7ff;
 // Exponents (E of fx_to_bits) that give a normal double for any V != 0.
 constexpr int kOutLo = 64, kOutHi = 2000;
 constexpr int kNone = -(1 << 24);            // "no term": below every exponent, far enough to subtract from
@@ -114,8 +121,11 @@ FX_HD void fx_mac(const Limb &x, const Limb &k, int64_t &hh, int64_t &mm) {
 
 constexpr int64_t kHalf = (int64_t)1 << 31;   // mm's start value: V is rounded, not cut
 
-// V = (hh 2^64 + mm 2^32) / 2^64.
-FX_HD int64_t fx_value(int64_t hh, int64_t mm) { return hh + (mm >> 32); }
+// V = (hh 2^64 + mm 2^32) 2^(bits - 64), mm started at kHalf >> bits.
+FX_HD int64_t fx_value(int64_t hh, int64_t mm, int bits = 0) {
+  return (int64_t)((uint64_t)hh << bits) + (mm >> (32 - bits));
+}
+constexpr int kFineBits = 3;   // of the walker, whose sums stay below 7 2^56 without them
 
 // The product of two coefficients as a coefficient: K1 K2 / 2^60 (K1 against 2^0
 // is kappa 2^61, K2 an operand-format value below 2^60).
@@ -146,6 +156,13 @@ FX_HD uint64_t fx_to_bits(int64_t V, int E) {
   return A ? b : 0;
 }
 
+// The leading zeros of the larger of two values, less the six above 58 bits ...
+FX_HD int fx_lead(int64_t a, int64_t b) {
+  return fx_clz((uint64_t)(a < 0 ? -a : a) | (uint64_t)(b < 0 ? -b : b)) - 6;
+}
+// ... and a value brought to 58 bits by them.
+FX_HD int64_t fx_bring(int64_t v, int n) { return n < 0 ? v >> -n : (int64_t)((uint64_t)v << n); }
+
 // A warp's sum of 32 doubles: each is held as a 58-bit integer against the
 // largest exponent field e of the warp (kSumLo <= e <= kSumHi), rounded to
 // nearest, v = X 2^(e - kSumBias), |X| <= 2^57, so that the sum stays below 2^62;
@@ -163,7 +180,22 @@ FX_HD int64_t fx_total(uint32_t p0, uint32_t p1, int32_t p2) {
   return (int64_t)(((uint64_t)(int64_t)p2 << 40) + ((uint64_t)p1 << 20) + p0);
 }
 
-// The exponent of the Laplacian's and the diagonal's coefficients: room for
+// A neighbour's coefficient c = q 2^(e - 61), 2^58 <= |q| < 2^59: exact.
+struct FxStencilCoef {
+  int64_t q;
+  int e;
+};
+inline FxStencilCoef fx_stencil_coef(double c) {
+  FxStencilCoef r = {0, kNone};
+  if (c == 0.0) return r;
+  int e = 0;
+  const double m = frexp(c, &e);          // |m| in [1/2, 1)
+  r.q = (int64_t)(m * 576460752303423488.0);   // 2^59
+  r.e = e + 2;
+  return r;
+}
+
+// The exponent of the diagonal's coefficients: room for
 // diagonal entries of more than twice c0, the value the diagonal tends to;
 // larger ones (the centrifugal term next to the origin) carry a shift of their
 // own.  false: a grid spacing outside 2^+-30, left to the FP64 path.

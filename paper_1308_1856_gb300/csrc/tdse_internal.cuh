@@ -80,7 +80,7 @@ struct OperatorView {
   // the fixed-point walker's tables (tdse_walk_fixed.cuh); fx_ok 0: not held
   const long long *diagq = nullptr;
   long long c1q = 0, c2q = 0;
-  int fx_ec = 0, fx_ok = 0;
+  int fx_e1 = 0, fx_e2 = 0, fx_ec = 0, fx_ok = 0;
   bool plain = false;             // all in FP64 (where fx_ok is 0, and where the cluster path's bits are wanted)
 };
 

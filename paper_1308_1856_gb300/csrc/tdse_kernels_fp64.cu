@@ -527,6 +527,8 @@ OpIn<WALK> make_in(const Geometry &g, const OperatorView &op, double E, const do
     in.diagq = op.diagq;
     in.c1q = op.c1q;
     in.c2q = op.c2q;
+    in.e1 = op.fx_e1;
+    in.e2 = op.fx_e2;
     in.ec = op.fx_ec;
     in.ok = 1;
     in.k = 0;

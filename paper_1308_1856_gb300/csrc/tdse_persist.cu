@@ -309,6 +309,8 @@ cudaError_t launch_lanczos_persistent(const Geometry &g, const OperatorView &op,
   in.c2 = g.c2;
   in.c1q = op.c1q;
   in.c2q = op.c2q;
+  in.e1 = op.fx_e1;
+  in.e2 = op.fx_e2;
   in.ec = op.fx_ec;
   in.ok = 1;
   in.k = 0;

@@ -9,26 +9,29 @@
 // shuffles and the row's uniform work against one, and take 94% of the lanes'
 // work against 88% for the same halo.
 //
-// Exponents are local: a lane converts its two columns against their largest
-// exponent field, and forms the stencil's sums against the largest of its own and
-// its two neighbour lanes' (six columns).  One exponent for the whole strip costs
-// ~10% less, but loses what FP64 keeps next to the origin: there a high partial
-// wave is many orders below its value at the strip's other end, and rounding
-// errors relative to that value, put into the stiff centrifugal points, are
-// multiplied by the largest energies of the grid in every Krylov iteration
-// (measured: 3e-12 after one step where FP64 gives 6e-16).
+// Exponents are local to a point: a column is converted against its own exponent,
+// and a point's sum is formed against the largest of its own terms', each operand
+// shifted there by itself.  What FP64 keeps at a small value beside large ones,
+// next to the origin in a high partial wave, inside a wall or among scattered values, is
+// kept here too: over such states and ordinary ones the error at a point is at most
+// 4.6 2^-53 of its terms' sum in modulus, 0.1 to 0.9 2^-53 in the mean square, where the
+// FP64 walk has 5.8 and 0.3 to 1.1 2^-53, and the 2-norm's is below its in each.  One
+// exponent for the lane's two columns and their neighbours, six in all, was 1 to 8%
+// faster (velocity gauge 5 to 13%: H x of 512,000 points 17.4 us, 19.7 now) but
+// lost up to every digit there.
 //
 // The velocity gauge couples the rows l -+ 1 through their first derivatives and
 // l/r terms: four products a part in place of two, of the derivative's integer
 // difference D and of the values, and the parts cross (-i).  D of a row is formed
 // once, when the row is converted, and kept in the lane's shared memory until
-// the row after next.  The length gauge's bound on the sums becomes
-// |mm| < (3.8 + 2 1.08 + 2 0.72) 2^60 < 2^63: D is held to 2^58.2.
+// the row after next, in 58 bits of its own: the difference cancels on a smooth
+// state, and FP64 forms it exactly.
 //
 // Blocks near the limits of FP64 (subnormal values, results that under- or
-// overflow) take separate conversions.  A row with an Inf or NaN in reach is
-// computed by h_point_fp64, one point at a time in FP64, so such values spread
-// exactly as they do there.  These choices are uniform over the warp.
+// overflow) take separate conversions.  A row with an Inf or NaN in reach, or a
+// diagonal entry too small for the sum's last bit beside a large value, is
+// computed by h_point_fp64, one point at a time in FP64.  These choices are
+// uniform over the warp.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -44,6 +47,13 @@ namespace stencil {
 using namespace tdse_fx;
 
 constexpr int kFxCols = 60;    // output columns of a strip
+// A zero's exponent field is 0, and the sum's exponent T the largest of all terms',
+// zeros' too: from kInLo on it is none of theirs (coefficients are below kCoupHi, an
+// exponent field; the diagonal's by fx_diag_fits).
+constexpr int kInLo = 256, kCoupHi = 1022 + 128;
+// Diagonal entries from 2^(ec - 4) on are held exactly, and far enough above the
+// sum's last bit: |D| >= 2^(ec - 4) where the encoded entry's high word reaches this.
+constexpr int kDiagHigh = 1 << 25;
 
 struct FxIn {
   const double2 *__restrict__ x;
@@ -52,8 +62,9 @@ struct FxIn {
   const double *__restrict__ kappa;
   int N, L;
   double c1, c2, E;                      // E: the field (length gauge) or A/c (velocity gauge)
-  long long c1q, c2q;                    // c1, c2 against 2^ec
-  int ec;
+  long long c1q, c2q;                    // c1, c2 against 2^e1, 2^e2 (fx_stencil_coef)
+  int e1, e2;
+  int ec;                                // the diagonal's exponent
   int ok;                                // 0: the grid's coefficients do not fit, every row runs in FP64
   int k;                                 // the result is 2^k H x
   const double *__restrict__ rinv;       // velocity gauge: 1 / r_j
@@ -121,14 +132,16 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int PENDING>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory"); }
 
-// A row of the strip in fixed point: the lane's two columns.
+// A row of the strip in fixed point: the lane's two columns, each against its own
+// largest part's exponent field (0: zero).
 struct FxRow {
   int64_t X[2][2];   // [column][re, im]
-  int e;             // their exponent field (0: zero)
+  unsigned e;        // the exponent fields, column 0's in the low half
+  unsigned eD;       // velocity gauge: the exponent fields of D likewise
   bool ok;           // every value of the strip finite (uniform)
-  int eD;            // velocity gauge: the exponent field of D (0: zero)
 };
-constexpr int kDShift = 6;   // D = (8 (x_{j+1} - x_{j-1}) - (x_{j+2} - x_{j-2})) / 2^6
+// The half of a pair of exponent fields.
+__device__ __forceinline__ int fx_half(unsigned e, int c) { return c == 0 ? (int)(e & 0xffffu) : (int)(e >> 16); }
 
 __device__ __forceinline__ uint32_t fx_field(double v) { return (uint32_t)__double2hiint(v) & kExpMask; }
 __device__ __forceinline__ int64_t fx_word(double v, uint32_t m) {
@@ -139,24 +152,24 @@ __device__ __forceinline__ int64_t fx_small(double v, int e) {
 }
 
 __device__ __forceinline__ void fx_convert(const double2 &v0, const double2 &v1, FxRow &r) {
-  const uint32_t m = max(max(fx_field(v0.x), fx_field(v0.y)), max(fx_field(v1.x), fx_field(v1.y)));
-  r.e = (int)(m >> 20);
-  r.ok = true;
-  r.eD = 0;
   constexpr uint32_t kLo = (uint32_t)kExpSmall << 20;
-  if (__all_sync(0xffffffffu, m - kLo < kExpMask - kLo)) {   // kLo <= m < kExpMask
-    r.X[0][0] = fx_word(v0.x, m);
-    r.X[0][1] = fx_word(v0.y, m);
-    r.X[1][0] = fx_word(v1.x, m);
-    r.X[1][1] = fx_word(v1.y, m);
+  const uint32_t m0 = max(fx_field(v0.x), fx_field(v0.y)), m1 = max(fx_field(v1.x), fx_field(v1.y));
+  r.ok = true;
+  r.e = (m0 >> 20) | (m1 >> 4);
+  r.eD = 0;
+  if (__all_sync(0xffffffffu, min(m0, m1) >= kLo && max(m0, m1) < kExpMask)) {
+    r.X[0][0] = fx_word(v0.x, m0);
+    r.X[0][1] = fx_word(v0.y, m0);
+    r.X[1][0] = fx_word(v1.x, m1);
+    r.X[1][1] = fx_word(v1.y, m1);
   } else {
-    r.ok = __all_sync(0xffffffffu, m != kExpMask) != 0;
-    const int e = max(r.e, 1);
-    r.X[0][0] = fx_small(v0.x, e);
-    r.X[0][1] = fx_small(v0.y, e);
-    r.X[1][0] = fx_small(v1.x, e);
-    r.X[1][1] = fx_small(v1.y, e);
-    r.e = (r.X[0][0] | r.X[0][1] | r.X[1][0] | r.X[1][1]) ? e : 0;
+    r.ok = __all_sync(0xffffffffu, max(m0, m1) != kExpMask) != 0;
+    const int e0 = max((int)(m0 >> 20), 1), e1 = max((int)(m1 >> 20), 1);
+    r.X[0][0] = fx_small(v0.x, e0);
+    r.X[0][1] = fx_small(v0.y, e0);
+    r.X[1][0] = fx_small(v1.x, e1);
+    r.X[1][1] = fx_small(v1.y, e1);
+    r.e = ((r.X[0][0] | r.X[0][1]) ? e0 : 0u) | ((r.X[1][0] | r.X[1][1]) ? (unsigned)e1 << 16 : 0u);
   }
 }
 
@@ -165,6 +178,13 @@ __device__ __forceinline__ double fx_result(int64_t V, int E) {
   const double t = __ll2double_rn(V);
   const int h = __double2hiint(t);
   return __hiloint2double(h ? h + ((E - 1079) << 20) : 0, __double2loint(t));
+}
+
+// x >> n for any n >= 0
+__device__ __forceinline__ int64_t fx_shr(int64_t x, int n) {
+  int64_t r;
+  asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(n));   // clamps the count
+  return r;
 }
 
 __device__ __forceinline__ int64_t fx_shfl_up(int64_t v) { return __shfl_up_sync(0xffffffffu, v, 1); }
@@ -231,16 +251,15 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
   // the coupling w_j = E r_j (velocity gauge: E / r_j) of the lane's columns
   const double w0 = __dmul_rn(in.E, rj0), w1 = __dmul_rn(in.E, rj1);
   const double wd = VG ? __dmul_rn(in.E, in.d1c) : 0.0;    // velocity gauge: the derivative's coefficient
-  const uint32_t wm = max(fx_field(w0), fx_field(w1));
-  const bool all_ok = in.ok && __all_sync(0xffffffffu, max(wm, fx_field(wd)) != kExpMask) != 0;
-  const int we = max((int)(wm >> 20), 1), ew = we - 1022;  // w = W 2^(ew - 60)
-  const Limb W[2] = {fx_limbs(fx_small(w0, we)), fx_limbs(fx_small(w1, we))};
-  const bool has_w = (W[0].h | W[0].l | W[1].h | W[1].l) != 0;
+  const bool all_ok =
+      in.ok && __all_sync(0xffffffffu, max(max(fx_field(w0), fx_field(w1)), fx_field(wd)) < (uint32_t)kCoupHi << 20) != 0;
+  const int we0 = max((int)(fx_field(w0) >> 20), 1), we1 = max((int)(fx_field(w1) >> 20), 1);
+  const int ew[2] = {we0 - 1022, we1 - 1022};              // w = W 2^(ew - 60)
+  const Limb W[2] = {fx_limbs(fx_small(w0, we0)), fx_limbs(fx_small(w1, we1))};
   // length gauge: a = kappa_l w = A 2^(ew - 61); velocity gauge: a = kappa_l l w =
   // A 2^(ew + el - 61) with 2^el > l, and d = kappa_l E d1c = D 2^(ed - 61)
   const int wde = max((int)(fx_field(wd) >> 20), 1), ed = wde - 1022;
   const Limb WD = fx_limbs(VG ? fx_small(wd, wde) : 0);
-  const bool has_d = (WD.h | WD.l) != 0;
   auto coupling = [&](int l, double kappa, Limb (&a)[2], Limb &d, int &el) {
     const int64_t K = fx_coef((uint64_t)__double_as_longlong(kappa), 0);
     Limb kp = fx_limbs(K);
@@ -253,28 +272,39 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
 #pragma unroll
     for (int c = 0; c < 2; ++c) a[c] = fx_limbs(fx_coef_product(kp, W[c]) | (VG ? 1 : 0));
   };
-  // velocity gauge: the differences D of a row, against the largest exponent of
-  // the lane's and its neighbours' columns, into the slot
+  // velocity gauge: the differences D of a row into the slot, each column's against
+  // the largest exponent of its terms and then brought to 58 bits, so that what
+  // cancels costs no bits: D = 8 Q (5-point) or Q (3-point)
   auto differences = [&](FxRow &r, int slot) {
-    const int eU = __shfl_up_sync(0xffffffffu, r.e, 1), eD = __shfl_down_sync(0xffffffffu, r.e, 1);
-    r.eD = max(r.e, max(eU, eD));
-    const int sC = min(r.eD - r.e, 63), sU = min(r.eD - eU, 63), sD = min(r.eD - eD, 63);
+    const unsigned u = __shfl_up_sync(0xffffffffu, r.e, 1), d = __shfl_down_sync(0xffffffffu, r.e, 1);
+    const int eA = fx_half(r.e, 0), eB = fx_half(r.e, 1), eU = fx_half(u, 1), eV = fx_half(d, 0);
+    const int eUA = fx_half(u, 0), eVB = fx_half(d, 1);
+    int b0 = max(eU, eB), b1 = max(eA, eV);
+    if (ST == 5) {
+      b0 = max(b0, max(eUA, eV));
+      b1 = max(b1, max(eU, eVB));
+    }
+    int64_t Q[2][2];
 #pragma unroll
     for (int p = 0; p < 2; ++p) {
-      const int64_t lB = fx_shfl_up(r.X[1][p]) >> sU, rA = fx_shfl_down(r.X[0][p]) >> sD;
-      const int64_t A = r.X[0][p] >> sC, B = r.X[1][p] >> sC;
-      longlong2 D;
-      constexpr int64_t half = (int64_t)1 << (kDShift - 1);
+      const int64_t A = r.X[0][p], B = r.X[1][p], lB = fx_shfl_up(B), rA = fx_shfl_down(A);
+      Q[0][p] = fx_shr(B, b0 - eB) - fx_shr(lB, b0 - eU);
+      Q[1][p] = fx_shr(rA, b1 - eV) - fx_shr(A, b1 - eA);
       if (ST == 5) {
-        const int64_t lA = fx_shfl_up(r.X[0][p]) >> sU, rB = fx_shfl_down(r.X[1][p]) >> sD;
-        D.x = (B - lB - ((rA - lA) >> 3) + half / 8) >> (kDShift - 3);
-        D.y = (rA - A - ((rB - lB) >> 3) + half / 8) >> (kDShift - 3);
-      } else {
-        D.x = (B - lB + half) >> kDShift;
-        D.y = (rA - A + half) >> kDShift;
+        const int64_t lA = fx_shfl_up(A), rB = fx_shfl_down(B);
+        Q[0][p] -= (fx_shr(rA, b0 - eV) - fx_shr(lA, b0 - eUA)) >> 3;
+        Q[1][p] -= (fx_shr(rB, b1 - eVB) - fx_shr(lB, b1 - eU)) >> 3;
       }
+    }
+    constexpr int k8 = ST == 5 ? 3 : 0;
+    const int n0 = min(fx_lead(Q[0][0], Q[0][1]), b0 + k8 - 1), n1 = min(fx_lead(Q[1][0], Q[1][1]), b1 + k8 - 1);
+#pragma unroll
+    for (int p = 0; p < 2; ++p) {
+      const longlong2 D = make_longlong2(fx_bring(Q[0][p], n0), fx_bring(Q[1][p], n1));
       *reinterpret_cast<longlong2 *>(mine + slot * kSlot + kSlot - 1024 + 512 * p) = D;
     }
+    r.eD = ((Q[0][0] | Q[0][1]) ? (unsigned)(b0 - n0 + k8) : 0u) |
+           ((Q[1][0] | Q[1][1]) ? (unsigned)(b1 - n1 + k8) << 16 : 0u);
   };
   const Limb k1 = fx_limbs(in.c1q), k2 = fx_limbs(in.c2q);
   Limb acur[2], anext[2], dcur = {0, 0}, dnext = {0, 0};
@@ -292,6 +322,8 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
     differences(cur, 1);
   }
   stage(l0 + 2, 0);
+  // T between these: nothing near FP64's limits
+  const int tlo = max(kInLo, kOutLo - in.k), thi = kOutHi - in.k;
   int s0 = 1, s1 = 2;                                      // slots of rows l and l + 1
 #pragma unroll 1
   for (int l = l0; l < l1; ++l) {
@@ -300,90 +332,87 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
     if (VG) differences(next, s1);
     coupling(l + 1, kap, anext, dnext, lnext);
     if (l + 1 < l1) kap = __ldg(in.kappa + l + 2);
-    const int eU = __shfl_up_sync(0xffffffffu, cur.e, 1), eD = __shfl_down_sync(0xffffffffu, cur.e, 1);
-    // exponent of the point's sum: the largest of its terms', coefficients included
-    const int eb = max(cur.e, max(eU, eD));
-    const int EP = (prev.e && has_w) ? prev.e + ew + lcur : kNone;
-    const int EN = (next.e && has_w) ? next.e + ew + lnext : kNone;
-    int Em = max(eb ? eb + in.ec : kNone, max(EP, EN));
-    const int EPD = (VG && prev.eD && has_d) ? prev.eD + ed + kDShift : kNone;
-    const int END = (VG && next.eD && has_d) ? next.eD + ed + kDShift : kNone;
-    if (VG) Em = max(Em, max(EPD, END));
-    if (all_ok && prev.ok && cur.ok && next.ok) {
-      const unsigned char *body = mine + s0 * kSlot;
-      const longlong2 dq = *reinterpret_cast<const longlong2 *>(body + 1024 + 1024 * EX);
-      // every operand is moved to that exponent before its product
-      const int eL = Em == kNone ? 0 : Em - in.ec;
-      const int sC = min(eL - cur.e, 63), sU = min(eL - eU, 63), sD = min(eL - eD, 63);
-      const int sP = min(Em - EP, 63), sN = min(Em - EN, 63);
-      const int sPD = min(Em - EPD, 63), sND = min(Em - END, 63);
-      const unsigned char *pd = mine + (kFxSlots - s0 - s1) * kSlot + kSlot - 1024, *nd = mine + s1 * kSlot + kSlot - 1024;
-      const int E = Em + in.k;
-      int64_t V[2][2];
-      // the sums without (D = false) or with the diagonal's term
-      auto sums = [&](auto with_d) {
+    const unsigned char *body = mine + s0 * kSlot;
+    const longlong2 dq = *reinterpret_cast<const longlong2 *>(body + 1024 + 1024 * EX);
+    const unsigned u = __shfl_up_sync(0xffffffffu, cur.e, 1), d = __shfl_down_sync(0xffffffffu, cur.e, 1);
+    // columns: UA UB | A B | VA VB
+    const int eUA = fx_half(u, 0), eUB = fx_half(u, 1), eA = fx_half(cur.e, 0), eB = fx_half(cur.e, 1);
+    const int eVA = fx_half(d, 0), eVB = fx_half(d, 1);
+    const int near[2] = {max(eUB, eB), max(eA, eVA)};
+    const int far[2] = {ST == 5 ? max(eUA, eVA) : 0, ST == 5 ? max(eUB, eVB) : 0};
+    // T: exponent of a point's sum, the largest of its own terms'
+    int T[2], td[2];
 #pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          const int64_t lB = fx_shfl_up(cur.X[1][p]) >> sU, rA = fx_shfl_down(cur.X[0][p]) >> sD;
-          int64_t lA = 0, rB = 0;
-          if (ST == 5) {
-            lA = fx_shfl_up(cur.X[0][p]) >> sU;
-            rB = fx_shfl_down(cur.X[1][p]) >> sD;
-          }
-          const int64_t A = cur.X[0][p] >> sC, B = cur.X[1][p] >> sC;
+    for (int c = 0; c < 2; ++c) {
+      td[c] = in.ec + fx_diag_shift(c == 0 ? dq.x : dq.y);
+      T[c] = max(near[c] + in.e1, (c == 0 ? eA : eB) + td[c]);
+      if (ST == 5) T[c] = max(T[c], far[c] + in.e2);
+      T[c] = max(T[c], max(fx_half(prev.e, c) + lcur, fx_half(next.e, c) + lnext) + ew[c]);
+      if (VG) T[c] = max(T[c], max(fx_half(prev.eD, c), fx_half(next.eD, c)) + ed);
+    }
+    bool fixed = all_ok && prev.ok && cur.ok && next.ok, limits = false;   // uniform
+    const int h0 = (int)(dq.x >> 32), h1 = (int)(dq.y >> 32);
+    if (fixed && !__all_sync(0xffffffffu, !inner || (min(T[0], T[1]) >= tlo && max(T[0], T[1]) <= thi &&
+                                                     min(abs(h0), abs(h1)) >= kDiagHigh))) {
+      // near FP64's limits, zeros, small diagonal entries: T again, of the terms that are not zero
+      auto term = [](int e, int c) { return e ? e + c : kNone; };
+      bool good = true, range = true;
 #pragma unroll
-          for (int c = 0; c < 2; ++c) {
-            int64_t hh = 0, mm = kHalf;
-            fx_mac(fx_limbs(c == 0 ? lB + B : A + rA), k1, hh, mm);
-            if (ST == 5) fx_mac(fx_limbs(c == 0 ? lA + rA : lB + rB), k2, hh, mm);
-            if (!VG) {
-              fx_mac(fx_limbs(prev.X[c][p] >> sP), acur[c], hh, mm);
-              fx_mac(fx_limbs(next.X[c][p] >> sN), anext[c], hh, mm);
-            } else {   // -i (A/c) w: the real part takes +w's imaginary part, the imaginary part -w's real part
-              int64_t ch = 0, cm = 0;
-              const int64_t *dp = reinterpret_cast<const int64_t *>(pd + 512 * (1 - p)) + c;
-              const int64_t *dn = reinterpret_cast<const int64_t *>(nd + 512 * (1 - p)) + c;
-              fx_mac(fx_limbs(prev.X[c][1 - p] >> sP), acur[c], ch, cm);
-              fx_mac(fx_limbs(next.X[c][1 - p] >> sN), anext[c], ch, cm);
-              fx_mac(fx_limbs(*dp >> sPD), dcur, ch, cm);
-              fx_mac(fx_limbs(*dn >> sND), dnext, ch, cm);
-              hh = p == 0 ? hh + ch : hh - ch;
-              mm = p == 0 ? mm + cm : mm - cm;
-            }
-            if (decltype(with_d)::value) fx_mac(fx_limbs(c == 0 ? A : B), fx_limbs(c == 0 ? dq.x : dq.y), hh, mm);
-            V[c][p] = fx_value(hh, mm);
-          }
-        }
-      };
-      int Ev[2] = {E, E};
-      if (!__any_sync(0xffffffffu, ((dq.x | dq.y) & kDiagMask) != 0)) {
-        sums(std::true_type{});
-      } else {   // entries above 2^ec: the other terms move down to their scale
-        sums(std::false_type{});
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int64_t d = c == 0 ? dq.x : dq.y;
-          const int s = fx_diag_shift(d);
-#pragma unroll
-          for (int p = 0; p < 2; ++p) {
-            int64_t hd = 0, md = kHalf;
-            fx_mac(fx_limbs(cur.X[c][p] >> sC), fx_limbs(fx_diag_value(d)), hd, md);
-            V[c][p] = (V[c][p] >> s) + fx_value(hd, md);
-          }
-          Ev[c] += s;
+      for (int c = 0; c < 2; ++c) {
+        const int e = c == 0 ? eA : eB;
+        T[c] = max(term(near[c], in.e1), term(e, td[c]));
+        if (ST == 5) T[c] = max(T[c], term(far[c], in.e2));
+        T[c] = max(T[c], max(term(fx_half(prev.e, c), lcur + ew[c]), term(fx_half(next.e, c), lnext + ew[c])));
+        if (VG) T[c] = max(T[c], max(term(fx_half(prev.eD, c), ed), term(fx_half(next.eD, c), ed)));
+        if (c == 0 ? out0 : out1) {
+          good = good && (abs(c == 0 ? h0 : h1) >= kDiagHigh || e <= near[c]);
+          range = range && (T[c] == kNone || (T[c] >= kOutLo - in.k && T[c] <= thi));
         }
       }
+      fixed = __all_sync(0xffffffffu, good) != 0;
+      limits = !__all_sync(0xffffffffu, range);
+    }
+    if (fixed) {
+      const unsigned char *pd = mine + (kFxSlots - s0 - s1) * kSlot + kSlot - 1024, *nd = mine + s1 * kSlot + kSlot - 1024;
+      const Limb kd[2] = {fx_limbs(fx_diag_value(dq.x)), fx_limbs(fx_diag_value(dq.y))};
       double t[2][2];
 #pragma unroll
-      for (int c = 0; c < 2; ++c)
+      for (int p = 0; p < 2; ++p) {
+        const int64_t A = cur.X[0][p], B = cur.X[1][p], UB = fx_shfl_up(B), VA = fx_shfl_down(A);
+        int64_t UA = 0, VB = 0;
+        if (ST == 5) {
+          UA = fx_shfl_up(A);
+          VB = fx_shfl_down(B);
+        }
 #pragma unroll
-        for (int p = 0; p < 2; ++p) t[c][p] = fx_result(V[c][p], Ev[c]);
-      if (!__all_sync(0xffffffffu, Em == kNone || (E >= kOutLo && E <= kOutHi))) {   // near FP64's limits
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-          for (int p = 0; p < 2; ++p)
-            t[c][p] = ldexp(fx_double(fx_to_bits(V[c][p], 1000)), V[c][p] ? Ev[c] - 1000 : 0);
+        for (int c = 0; c < 2; ++c) {   // every operand is moved to T before its product
+          int64_t hh = 0, mm = kHalf >> kFineBits;
+          const int t1 = T[c] - in.e1, t2 = T[c] - in.e2;
+          fx_mac(fx_limbs(c == 0 ? fx_shr(UB, t1 - eUB) + fx_shr(B, t1 - eB) : fx_shr(A, t1 - eA) + fx_shr(VA, t1 - eVA)),
+                 k1, hh, mm);
+          if (ST == 5)
+            fx_mac(fx_limbs(c == 0 ? fx_shr(UA, t2 - eUA) + fx_shr(VA, t2 - eVA)
+                                   : fx_shr(UB, t2 - eUB) + fx_shr(VB, t2 - eVB)), k2, hh, mm);
+          fx_mac(fx_limbs(fx_shr(c == 0 ? A : B, T[c] - td[c] - (c == 0 ? eA : eB))), kd[c], hh, mm);
+          const int sp = T[c] - ew[c] - lcur - fx_half(prev.e, c), sn = T[c] - ew[c] - lnext - fx_half(next.e, c);
+          if (!VG) {
+            fx_mac(fx_limbs(fx_shr(prev.X[c][p], sp)), acur[c], hh, mm);
+            fx_mac(fx_limbs(fx_shr(next.X[c][p], sn)), anext[c], hh, mm);
+          } else {   // -i (A/c) w: the real part takes +w's imaginary part, the imaginary part -w's real part
+            int64_t ch = 0, cm = 0;
+            const int64_t *dp = reinterpret_cast<const int64_t *>(pd + 512 * (1 - p)) + c;
+            const int64_t *dn = reinterpret_cast<const int64_t *>(nd + 512 * (1 - p)) + c;
+            fx_mac(fx_limbs(fx_shr(prev.X[c][1 - p], sp)), acur[c], ch, cm);
+            fx_mac(fx_limbs(fx_shr(next.X[c][1 - p], sn)), anext[c], ch, cm);
+            fx_mac(fx_limbs(fx_shr(*dp, T[c] - ed - fx_half(prev.eD, c))), dcur, ch, cm);
+            fx_mac(fx_limbs(fx_shr(*dn, T[c] - ed - fx_half(next.eD, c))), dnext, ch, cm);
+            hh = p == 0 ? hh + ch : hh - ch;
+            mm = p == 0 ? mm + cm : mm - cm;
+          }
+          const int64_t V = fx_value(hh, mm, kFineBits);
+          const int E = T[c] + in.k - kFineBits;
+          t[c][p] = limits ? ldexp(fx_double(fx_to_bits(V, 1000)), V ? E - 1000 : 0) : fx_result(V, E);
+        }
       }
 #pragma unroll
       for (int c = 0; c < 2; ++c)
