@@ -50,8 +50,7 @@ __device__ __forceinline__ void cb_setup(CbTable &t, const LanczosScalars *ls) {
   const double2 c = __ldcg(&ls->coef[j]);
   const int e = max((int)(max(fx_field(c.x), fx_field(c.y)) >> 20), 1);
   CbCoef q;
-  // the imaginary part odd: its low limb is not -2^31 and can be negated
-  const Limb x = fx_limbs(fx_small(c.x, e) >> 3), y = fx_limbs((fx_small(c.y, e) >> 3) | 1);
+  const Limb x = fx_limbs(fx_small(c.x, e) >> 3), y = fx_limbs(fx_small(c.y, e) >> 3);
   q.k = make_int4(x.h, x.l, y.h, y.l);
   q.ec = e - 1022;
   q.ok = (c.x == 0.0 && c.y == 0.0) || (e >= 512 && e <= 1534);
@@ -88,6 +87,7 @@ __device__ __forceinline__ double2 cb_sum(const CbTable &t, Load &&load) {
     }
     if (t.ok && __all_sync(0xffffffffu, E == kNone || (lo >= kCbLo && hi <= kCbHi && E > kOutLo && E <= kOutHi))) {
       int64_t xh = 0, xm = kHalf >> 6, yh = 0, ym = kHalf >> 6;   // rounded, not cut
+      int64_t nh = 0, nm = 0;                                     // the real part's second products: subtracted
 #pragma unroll
       for (int q = 0; q < kCbGroup; ++q) {
         if (j0 + q >= k) break;
@@ -96,12 +96,14 @@ __device__ __forceinline__ double2 cb_sum(const CbTable &t, Load &&load) {
         // value here, and at least 64, from where a zero converts to zero
         const uint32_t ee = (uint32_t)min(max(E - f.ec + 1, 64), 4095) << 20;
         const Limb X = fx_limbs(fx_word(u[q].x, ee)), Y = fx_limbs(fx_word(u[q].y, ee));
-        const Limb a = {f.k.x, f.k.y}, b = {f.k.z, f.k.w}, nb = {-f.k.z, -f.k.w};
+        const Limb a = {f.k.x, f.k.y}, b = {f.k.z, f.k.w};
         fx_mac(X, a, xh, xm);
-        fx_mac(Y, nb, xh, xm);
+        fx_mac(Y, b, nh, nm);
         fx_mac(Y, a, yh, ym);
         fx_mac(X, b, yh, ym);
       }
+      xh -= nh;
+      xm -= nm;
       o.x = __dadd_rn(o.x, fx_result((xh << 6) + (xm >> 26), E - 1));
       o.y = __dadd_rn(o.y, fx_result((yh << 6) + (ym >> 26), E - 1));
     } else {
