@@ -83,6 +83,10 @@ __device__ __forceinline__ double2 cb_sum(const CbTable &t, Load &&load) {
         lo = min(lo, e);
         hi = max(hi, e);
         E = max(E, e + t.f[j0 + q].ec);
+      } else if ((((unsigned)__double2hiint(u[q].x) | (unsigned)__double2hiint(u[q].y)) & 0xfffffu) |
+                 (unsigned)__double2loint(u[q].x) | (unsigned)__double2loint(u[q].y)) {
+        E = max(E, 0);   // subnormal (seen in integers: an FP64 comparison takes its pipe even where it is not due)
+        lo = 0;
       }
     }
     if (t.ok && __all_sync(0xffffffffu, E == kNone || (lo >= kCbLo && hi <= kCbHi && E > kOutLo && E <= kOutHi))) {
