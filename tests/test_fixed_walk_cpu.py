@@ -1,7 +1,8 @@
 """The arithmetic of the fixed-point walker's sums (csrc/tdse_fixed.cuh, compiled
 here with g++) at the ends of its ranges: the extreme sums of both gauges stay
 inside 64 bits, a neighbour's coefficient is exact, and the differences of the
-velocity gauge are brought to 58 bits without losing any that are there."""
+velocity gauge are brought to 58 bits without losing any that are there.  Also the
+norm and its inverse from an approximate reciprocal square root."""
 import os
 import shutil
 import struct
@@ -35,6 +36,9 @@ int main() {
       printf("%lld\n", (long long)fx_value(hh - ch, mm - cm, kFineBits));
     } else if (c == "coef") { std::string s; std::cin >> s; uint64_t u = std::stoull(s, nullptr, 16); double d;
       memcpy(&d, &u, 8); FxStencilCoef q = fx_stencil_coef(d); printf("%lld %d\n", (long long)q.q, q.e);
+    } else if (c == "norm") { std::string s, t; std::cin >> s >> t; uint64_t u = std::stoull(s, nullptr, 16),
+      v = std::stoull(t, nullptr, 16); double d, y, n, i; memcpy(&d, &u, 8); memcpy(&y, &v, 8); fx_norm(d, y, n, i);
+      memcpy(&u, &n, 8); memcpy(&v, &i, 8); printf("%llx %llx\n", (unsigned long long)u, (unsigned long long)v);
     } else if (c == "bring") { long long a, b; std::cin >> a >> b; int n = fx_lead(a, b);
       printf("%d %lld %lld\n", n, (long long)fx_bring(a, n), (long long)fx_bring(b, n)); }
   }
@@ -107,3 +111,26 @@ def test_differences_keep_their_bits(fx):
             assert n < 0 or w == v << n
         if a or b:
             assert max(abs(p), abs(q)) >= 2 ** 57 - 1
+
+
+def test_norm_and_inverse(fx):
+    """From a reciprocal square root up to two units off: the norm within 0.51 of a unit in
+    the last place, the inverse within 0.51 of the norm's inverse as it is rounded."""
+    rng = np.random.default_rng(5)
+    hx = lambda v: f"{struct.unpack('<Q', struct.pack('<d', v))[0]:x}"
+    db = lambda h: struct.unpack("<d", struct.pack("<Q", int(h, 16)))[0]
+    lines, vals = [], []
+    for _ in range(2000):
+        s2 = float(rng.uniform(1, 4) * 2.0 ** int(rng.integers(-920, 1022)))
+        y = float(1.0 / np.sqrt(s2))
+        for _ in range(abs(k := int(rng.integers(-2, 3)))):
+            y = float(np.nextafter(y, np.inf if k > 0 else 0.0))
+        lines.append(f"norm {hx(s2)} {hx(y)}")
+        vals.append(s2)
+    for s2, o in zip(vals, fx(lines)):
+        n, i = map(db, o.split())
+        # |n - sqrt| <= 0.51 ulp  <=>  (n -+ 0.51 ulp)^2 brackets s2
+        u = Fraction(51, 100) * Fraction(float(np.spacing(n)))
+        assert (Fraction(n) - u) ** 2 <= Fraction(s2) <= (Fraction(n) + u) ** 2
+        v = Fraction(51, 100) * Fraction(float(np.spacing(i)))
+        assert abs(Fraction(i) - 1 / Fraction(n)) <= v
