@@ -666,8 +666,8 @@ int tdse_batch_profile_read(tdse_batch_t *b, int kind, double *total_ms, long lo
 
 /*
  * Launch schedule of the batched kernels.
- *   prefetch_rows: the rows the FP64 stencil kernel prefetches ahead into L2
- *     (0, 3, 6 or 10);
+ *   prefetch_rows: 0, 3, 6 or 10; accepted and returned, without effect (the
+ *     stencil kernels stage their rows in shared memory);
  *   ring_rows: the mixed-precision stencil kernel walks tiles of 256 radial
  *     columns x 32 partial waves, its rows brought into a ring of shared-memory
  *     slots by bulk asynchronous copies; 0, 3 or 5 selects a ring of 4, 8 or

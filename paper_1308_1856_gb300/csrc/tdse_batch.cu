@@ -1656,7 +1656,6 @@ std::vector<long long> Engine::segment_key(const Segment &sg) const {
   k.reserve(32 + 9 * sg.off.size() + hlists.size());
   k.push_back(precision);
   k.push_back(stencil);
-  k.push_back(sched.pf);
   k.push_back(sched.ring);
   k.push_back(sched.sblocks);
   k.push_back(sched.eblocks);
@@ -2309,32 +2308,26 @@ int Engine::autotune(const std::vector<int> &slots) {
   const int nring = precision == TDSE_MIXED ? (int)(sizeof(kRingChoices) / sizeof(int)) : 1;
   // three blocks per SM only for the mixed tile kernel (the FP64 kernels' blocks fill an SM at two)
   const int sbmax = precision == TDSE_MIXED ? kTileBlocksPerSM : kStencilBlocksPerSM;
-  // the prefetch distance is the FP64 velocity-gauge kernel's: the others stage their rows in shared memory
-  const bool tune_pf = precision == TDSE_FP64 && sg.vtotal[0] > 0;
+  // FP64: the velocity-gauge instances' launch takes its blocks per SM from the same choice
+  const bool tune_vg = precision == TDSE_FP64 && sg.vtotal[0] > 0;
   const ChunkList v0 = list_at(lists, sg.voff[0], sg.vnact[0], sg.vtotal[0]);
-  for (int sb = 1; sb <= sbmax && !rc && (sg.total[0] > 0 || tune_pf); ++sb)
-    for (int ri = 0; ri < nring && !rc; ++ri)
-      for (int pf : kPfChoices) {
-        const int ring = kRingChoices[ri];
-        if (!tune_pf && pf != kPfChoices[0]) continue;
-        Schedule c = sched;
-        c.pf = pf;
-        c.ring = ring;
-        c.sblocks = sb;
-        float t = 0.f;
-        rc = time_it([&]() {
-          int r = sg.total[0] > 0 ? launch_a(B, a0, 0, c) : (int)TDSE_OK;
-          if (!r && tune_pf) r = launch_a_velocity(B, v0, 0, c);
-          return r;
-        }, t);
-        if (rc) break;
-        if (t < bestA) {
-          bestA = t;
-          bestS.pf = pf;
-          bestS.ring = ring;
-          bestS.sblocks = sb;
-        }
+  for (int sb = 1; sb <= sbmax && !rc && (sg.total[0] > 0 || tune_vg); ++sb)
+    for (int ri = 0; ri < nring && !rc; ++ri) {
+      Schedule c = sched;
+      c.ring = kRingChoices[ri];
+      c.sblocks = sb;
+      float t = 0.f;
+      rc = time_it([&]() {
+        int r = sg.total[0] > 0 ? launch_a(B, a0, 0, c) : (int)TDSE_OK;
+        if (!r && tune_vg) r = launch_a_velocity(B, v0, 0, c);
+        return r;
+      }, t);
+      if (!rc && t < bestA) {
+        bestA = t;
+        bestS.ring = c.ring;
+        bestS.sblocks = sb;
       }
+    }
   if (!rc && sg.vtotal[0] > 0) {
     // the velocity-gauge instances' phase-0 z, which lanczos_b below reads
     rc = launch_a_velocity(B, v0, 0, sched);

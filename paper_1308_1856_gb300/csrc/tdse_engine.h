@@ -102,7 +102,7 @@ struct FluxDev {
 // (chunks and their reduction order are fixed per instance); the autotuner
 // picks the fastest for the resident instances.
 struct Schedule {
-  int pf = 6;                        // rows the stencil kernels prefetch ahead (kPfChoices)
+  int pf = 6;                        // no kernel takes it: kept for the callers that set it (kPfChoices)
   int ring = 0;                      // mixed stencil kernel: rows staged ahead in shared memory (0: off)
   int sblocks = kStencilBlocksPerSM; // blocks per SM of the stencil kernels (1 or 2; 3 for the mixed tiles)
   int eblocks = kElemBlocksPerSM;    // blocks per SM of the elementwise kernels (1 or 2)
