@@ -1787,6 +1787,11 @@ int Engine::norm_pass(const BatchDev &B, const std::vector<int> &ids, int off, i
   return TDSE_OK;
 }
 
+// Blocks per SM of the FP64 stencil launch: the schedule's one or two of kBlockJ
+// threads stand for half its blocks or all of them.
+template <bool VG>
+static int fx_blocks(const Schedule &s) { return s.sblocks > 1 ? kFxBlocksPerSM<VG> : 2; }
+
 int Engine::launch_a(const BatchDev &B, const ChunkList &cl, int j, const Schedule &s) {
   if (precision == TDSE_MIXED) {
     const unsigned grid = (unsigned)(sms * s.sblocks);
@@ -1795,16 +1800,17 @@ int Engine::launch_a(const BatchDev &B, const ChunkList &cl, int j, const Schedu
     EN_CUDA(e, "batch lanczos a (mixed tiles)");
     return TDSE_OK;
   }
-  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM<false> : 2));
+  const unsigned grid = (unsigned)(sms * fx_blocks<false>(s));
   const cudaError_t e = stencil == 5 ? launch_fixed<5, false>(grid, stream, B, cl, j)
                                      : launch_fixed<3, false>(grid, stream, B, cl, j);
   EN_CUDA(e, "batch lanczos a");
   return TDSE_OK;
 }
 
-// Chunks the phase-A launch takes at once: one per warp (FP64) or block (mixed tiles).
+// Chunks the phase-A launch of the current schedule takes at once: one per warp (FP64,
+// length gauge; of the mixed tiles a block takes 16 one after the other).
 int Engine::stencil_wave() const {
-  return precision == TDSE_MIXED ? sms * sched.sblocks * (kBlockJ / 32) : sms * kFxBlocksPerSM<false> * (kFxThreads / 32);
+  return precision == TDSE_MIXED ? sms * sched.sblocks * (kBlockJ / 32) : sms * fx_blocks<false>(sched) * (kFxThreads / 32);
 }
 
 // Velocity-gauge instances: the same fixed-point walker with the (A/c) p_z coupling,
@@ -1817,7 +1823,7 @@ int Engine::launch_a_velocity(const BatchDev &B, const ChunkList &cl, int j, con
     EN_CUDA(cudaGetLastError(), "batch lanczos a (mixed, velocity gauge)");
     return TDSE_OK;
   }
-  const unsigned grid = (unsigned)(sms * (s.sblocks > 1 ? kFxBlocksPerSM<true> : 2));
+  const unsigned grid = (unsigned)(sms * fx_blocks<true>(s));
   const cudaError_t e = stencil == 5 ? launch_fixed<5, true>(grid, stream, B, cl, j)
                                      : launch_fixed<3, true>(grid, stream, B, cl, j);
   EN_CUDA(e, "batch lanczos a (velocity gauge)");
