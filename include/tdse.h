@@ -411,8 +411,8 @@ int tdse_small_grid_path_used(const tdse_t *h);
  * tdse_set_small_grid_path: FORCE takes this path at any size where the
  * device allows the cooperative launch (the small-grid path, if it applies,
  * still comes first); AUTO (default) and OFF keep the multi-launch path,
- * which is faster on the grids measured (its kernels read the Krylov vectors
- * through L1; here every read of data another block wrote goes to L2).
+ * which is faster on the grids measured (its launches cost about what the grid
+ * barriers do, and its elementwise kernels run two blocks per SM).
  * tdse_persistent_path_used returns 1 if the last tdse_propagate ran on it.
  * Errors: TDSE_ERR_ARG (unknown mode).
  */

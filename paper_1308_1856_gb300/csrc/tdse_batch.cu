@@ -2,10 +2,10 @@
 // Lanczos phase for the whole batch.
 //
 // Each instance has its own grid (N, lmax, dr, potential), pulse, absorber,
-// Krylov dimension m and step dt.  Its (lmax+1) x N points are cut into
-// 32-point row segments (radial-group-major, as in the single-instance
-// kernels) and the segments into chunks of kChunkSegs.  A launch of phase j
-// walks the chunks of every instance still active in that phase (m_i > j),
+// Krylov dimension m and step dt.  Its (lmax+1) x N points are cut into chunks:
+// for the FP64 stencil fx_rows row segments of the walker's strips (chunk_strips),
+// for the mixed one tiles (velocity gauge: kChunkSegs segments of 32 columns), for
+// the elementwise kernels kChunkPts consecutive points.  A launch of phase j walks the chunks of every instance still active in that phase (m_i > j),
 // statically split over the warps of a persistent grid.  Each chunk's partial
 // sum goes to its own slot; the warp that finishes an instance's last chunk
 // (per-instance arrival counter) adds that instance's chunk partials in chunk
@@ -120,22 +120,6 @@ __device__ __forceinline__ void chunk_columns(const BatchInst &I, int ci, F &&f)
   }
 }
 
-// The same segments as chunk_columns, for warp-collective walkers: every lane
-// gets f(jg, l0, l1) (its column jg*32 + lane may be >= N).
-template <typename F>
-__device__ __forceinline__ void chunk_groups(const BatchInst &I, int ci, F &&f) {
-  const int Lp1 = I.L + 1;
-  int s = ci * kChunkSegs;
-  const int s_end = min(s + kChunkSegs, I.nseg);
-  while (s < s_end) {
-    const int jg = s / Lp1;
-    const int l0 = s - jg * Lp1;
-    const int l1 = min(Lp1, l0 + (s_end - s));
-    f(jg, l0, l1);
-    s += l1 - l0;
-  }
-}
-
 // Visit chunk ci of an instance in the fixed-point stencil layout: strips of
 // kFxCols columns, I.fx_rows row segments of a strip-major order per chunk.
 // f(j0, l0, l1) is called by every lane of the warp.
@@ -155,26 +139,10 @@ __device__ __forceinline__ void chunk_strips(const BatchInst &I, int ci, F &&f) 
 
 // Visit chunk ci of an instance in the elementwise layout: the kChunkPts
 // consecutive points [ci*C, min((ci+1)*C, G)) of the l-major array, lane-strided
-// so that every load is coalesced; f(idx, i) with i = idx mod N, the radial index.
-template <typename F>
-__device__ __forceinline__ void chunk_points(const BatchInst &I, int ci, F &&f) {
-  const unsigned N = (unsigned)I.N;
-  const unsigned G = N * (unsigned)(I.L + 1);
-  const unsigned base = (unsigned)ci * kChunkPts + (threadIdx.x & 31);
-  const unsigned end = min(G, (unsigned)(ci + 1) * kChunkPts);
-  unsigned i = base % N;
-#pragma unroll 4
-  for (unsigned idx = base; idx < end; idx += 32) {
-    f((size_t)idx, (int)i);
-    i += 32;
-    while (i >= N) i -= N;
-  }
-}
-
-// As chunk_points, NQ lane-strided points at a time: the loads of all NQ
-// (load(idx) -> V) are issued before the first op(idx, i, V), whose stores
-// the compiler could not otherwise move loads across (the arrays may alias as
-// far as it knows).  The points reach op in the same order as in chunk_points.
+// so that every load is coalesced, with i = idx mod N the radial index.  NQ points
+// at a time: their loads (load(idx) -> V) are issued before the first op(idx, i, V),
+// whose stores the compiler could not otherwise move loads across (the arrays may
+// alias as far as it knows).
 template <int NQ, typename Ld, typename Op>
 __device__ __forceinline__ void chunk_points_xn(const BatchInst &I, int ci, Ld &&load, Op &&op) {
   const unsigned N = (unsigned)I.N;
@@ -203,7 +171,7 @@ __device__ __forceinline__ void chunk_points_x4(const BatchInst &I, int ci, Ld &
   chunk_points_xn<4>(I, ci, load, op);
 }
 
-// The points of chunk_points in groups of Q consecutive lane-strided points:
+// The points of such a chunk in groups of Q consecutive lane-strided points:
 // f(idx[Q], i[Q], nq) with the first nq entries valid.
 template <int Q, typename F>
 __device__ __forceinline__ void chunk_groups_of(const BatchInst &I, int ci, F &&f) {
@@ -807,8 +775,8 @@ __global__ void __launch_bounds__(kElemThreads, kElemBlocksPerSM)
 }
 
 // The diagonal of a new instance, c0 + l(l+1)/(2 r^2) - Z/r in the roundings of
-// plain FP64 (no fused step): as doubles (velocity gauge, or coefficients
-// outside the fixed-point range), encoded for the fixed-point walker, or in
+// plain FP64 (no fused step): as doubles (coefficients outside the
+// fixed-point range), encoded for the fixed-point walker, or in
 // FP32 without c0 (mixed).  On the device because a served instance is built
 // while others run: two divisions a point on one host core took longer than
 // an instance's Lanczos step.

@@ -17,18 +17,18 @@
 //   - a cluster barrier separates the stages: each stage reads the halo of
 //     the vector the previous stage wrote;
 //   - a grid-wide sum (the Lanczos dot products and norms) is every warp's
-//     shuffle-tree sum, a cluster barrier, and the C x 8 warp sums added in
+//     sum (warp_sum_fx), a cluster barrier, and the C x 8 warp sums added in
 //     one fixed order by warp 0 of every CTA, so that every CTA holds the
 //     same bits (cluster_sum);
 //   - every CTA forms the small exponential of the Lanczos step itself from
 //     those identical scalars, so no broadcast is needed.
 // The per-point arithmetic of Taylor and RK4 is that of the multi-launch
-// kernels (tdse_kernels_fp64.cu), so either path gives bitwise the same state;
+// kernels' FP64 walk (tdse_kernels_fp64.cu), so either path gives bitwise the same state;
 // the field couplings kappa_l E r_j of a Taylor or Lanczos step are formed
 // once per step into a table, with the walker's roundings.  Lanczos applies
-// the unscaled operator and then sigma_j (the multi-launch kernels fold
-// sigma_j into the coefficients), and associates its grid sums differently:
-// it agrees with that path to rounding.
+// the unscaled FP64 operator and then sigma_j (the multi-launch kernels scale by
+// a power of two, their operator in fixed point), and associates its grid sums
+// differently: it agrees with that path to rounding.
 // The only waits are cluster barriers (hardware), reached the same number of
 // times by every CTA: the control flow is uniform over the cluster.
 #include <cooperative_groups.h>
