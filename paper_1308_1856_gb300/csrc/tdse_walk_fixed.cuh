@@ -350,7 +350,7 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
       T[c] = max(T[c], max(fx_half(prev.e, c) + lcur, fx_half(next.e, c) + lnext) + ew[c]);
       if (VG) T[c] = max(T[c], max(fx_half(prev.eD, c), fx_half(next.eD, c)) + ed);
     }
-    bool fixed = all_ok && prev.ok && cur.ok && next.ok, limits = false;   // uniform
+    bool fixed = all_ok && prev.ok && cur.ok && next.ok, limits = false, zero = false;   // uniform
     const int h0 = (int)(dq.x >> 32), h1 = (int)(dq.y >> 32);
     if (fixed && !__all_sync(0xffffffffu, !inner || (min(T[0], T[1]) >= tlo && max(T[0], T[1]) <= thi &&
                                                      min(abs(h0), abs(h1)) >= kDiagHigh))) {
@@ -371,13 +371,15 @@ __device__ __forceinline__ void walk_rows_fixed(const FxIn &in, const FxExtra<EX
       }
       fixed = __all_sync(0xffffffffu, good) != 0;
       limits = !__all_sync(0xffffffffu, range);
+      zero = __all_sync(0xffffffffu, (prev.e | cur.e | next.e) == 0) != 0;   // a tail that has underflowed, an empty wave
     }
     if (fixed) {
       const unsigned char *pd = mine + (kFxSlots - s0 - s1) * kSlot + kSlot - 1024, *nd = mine + s1 * kSlot + kSlot - 1024;
       const Limb kd[2] = {fx_limbs(fx_diag_value(dq.x)), fx_limbs(fx_diag_value(dq.y))};
-      double t[2][2];
+      double t[2][2] = {};
 #pragma unroll
       for (int p = 0; p < 2; ++p) {
+        if (zero) break;
         const int64_t A = cur.X[0][p], B = cur.X[1][p], UB = fx_shfl_up(B), VA = fx_shfl_down(A);
         int64_t UA = 0, VB = 0;
         if (ST == 5) {
