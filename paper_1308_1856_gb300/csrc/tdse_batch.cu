@@ -327,9 +327,9 @@ __device__ __forceinline__ void for_strided_chunks(const ChunkList &cl, F &&f) {
 // What bounds it: the issue of the integer and the FP64 pipe together, 16 warps an
 // SM at 128 registers; more warps spill more (56 bytes here) and are slower.  The velocity
 // gauge's needs 12 warps at 168: a batch of 16 instances 11.4 ms for four steps, 12.1 at 128.
-// All phase A launches of one step of 128 instances (8.1e7 points): 36.9 ms in
-// FP64, 19.5 ms here; of 8 instances (1.3e6 points), 24 ms to 6 ms over 8 steps,
-// where the smaller chunks count as well.
+// One launch over 16 instances (1.08e7 points, caches cold): 534 us in FP64, 240 us
+// here; of 8 instances (1.3e6 points), all launches of 8 steps, 24 ms to 6 ms, where the
+// smaller chunks count as well.
 template <int ST, bool VG, int EX>
 __global__ void __launch_bounds__(kFxThreads, kFxBlocksPerSM<VG>) bt_lanczos_a_fixed(BatchDev B, ChunkList cl, int j) {
   extern __shared__ __align__(16) unsigned char fx_smem[];

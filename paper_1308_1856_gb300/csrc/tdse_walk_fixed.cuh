@@ -15,7 +15,7 @@
 // next to the origin in a high partial wave, inside a wall or among scattered values, is
 // kept here too: over such states and ordinary ones the error at a point is at most
 // 4.6 2^-53 of its terms' sum in modulus, 0.1 to 0.9 2^-53 in the mean square, where the
-// FP64 walk has 5.8 and 0.3 to 1.1 2^-53, and the 2-norm's is below its in each.  One
+// FP64 walk has 5.8 and 0.3 to 1.1 2^-53, in each of them more in the mean square.  One
 // exponent for the lane's two columns and their neighbours, six in all, was 1 to 8%
 // faster (velocity gauge 5 to 13%: H x of 512,000 points 17.4 us, 19.7 now) but
 // lost up to every digit there.
